@@ -59,59 +59,272 @@ struct DBuf {
 // ---------------------------------------------------------------------------
 // k-means per part, fp64 (Sec. 4.1)
 // ---------------------------------------------------------------------------
-// One thread per training row.  The row's part is staged in shared memory as
-// float (exact for bytes and float32); the distance to each center is summed
-// in dimension order with separate multiply and add (no FMA), the same
-// arithmetic as a plain sequential fp64 loop.
-template <int DT>
-__global__ void km_assign_kernel(const void *X, int64_t N, int d, int dp, int p, int n, const double *C,
-                                 int32_t *assign) {
-    extern __shared__ float srow[];  // dp * blockDim.x
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int tid = threadIdx.x, B = blockDim.x;
-    if (i < N) {
-        for (int e = 0; e < dp; e++) {
-            int64_t at = i * d + (int64_t)p * dp + e;
-            srow[e * B + tid] = DT == ANN_U8 ? (float)((const uint8_t *)X)[at] : ((const float *)X)[at];
-        }
-    }
-    if (i >= N) return;
-    double best = 0.0;
-    int arg = -1;
-    for (int j = 0; j < n; j++) {
-        const double *cj = C + (int64_t)j * dp;
-        double s = 0.0;
-        for (int e = 0; e < dp; e++) {
-            double t = __dsub_rn((double)srow[e * B + tid], cj[e]);
-            s = __dadd_rn(s, __dmul_rn(t, t));
-        }
-        if (arg < 0 || s < best) {
-            best = s;
-            arg = j;
-        }
-    }
-    assign[i] = arg;
+// The assignment is the one of a plain sequential fp64 loop (separate multiply
+// and add in dimension order, ties to the lower center), but fp64 decides only
+// the rows where float32 cannot: the fp64 rate of this part is about 1/64 of
+// its float32 rate, and ann_train_centers took 538 ms for 200,000 x 128 bytes,
+// P = 4, n = 256, 10 iterations, 531 of them in fp64 distances.
+// km_assign_kernel takes every distance in float32 and keeps a row's two
+// smallest; when their error bounds do not overlap the smaller one is the fp64
+// answer too, else km_exact_kernel scans the row: 8.0 ms for the same call.
+//
+// Bound.  c' = float32(c), t = float32(x - c') (|t - (x - c)| <= u (|c| + |t|)),
+// a = the float32 sum of the fused t * t.  With s the real distance,
+// |a - s| <= 2 sqrt(a) |dt| + |dt|^2 + (dp + 4) u a, |dt| <= u (|c| + sqrt(a))
+// (Cauchy-Schwarz); twice that, plus the underflow floor.
+__device__ __forceinline__ float km_eps(float a, float cmax, int dp) {
+    const float u = 5.9604645e-8f;
+    const float r = sqrtf(a), dt = u * (cmax + r);
+    return 2.0f * (2.0f * r * dt + dt * dt + (float)(dp + 4) * u * a) + (float)dp * 1e-37f;
 }
 
 template <int DT>
-__global__ void km_accumulate_kernel(const void *X, int64_t N, int d, int dp, int p, const int32_t *assign,
+__device__ __forceinline__ float km_elem(const void *X, int64_t at) {
+    return DT == ANN_U8 ? (float)((const uint8_t *)X)[at] : __ldg((const float *)X + at);
+}
+
+// float32 negated centers of every part and the largest center norm of the part
+__global__ void km_prep_kernel(const double *C, int n, int dp, float *cneg, float *cmax) {
+    __shared__ float red[256];
+    const double *Cp = C + (int64_t)blockIdx.x * n * dp;
+    float *out = cneg + (int64_t)blockIdx.x * n * dp;
+    float m = 0.f;
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        float s = 0.f;
+        for (int e = 0; e < dp; e++) {
+            const float c = __double2float_rn(Cp[(int64_t)j * dp + e]);
+            out[(int64_t)j * dp + e] = -c;
+            s = __fmaf_ru(c, c, s);
+        }
+        s = __fsqrt_ru(s) * 1.00001f;
+        m = s > m || s != s ? s : m;  // a NaN center sends every row to the exact scan
+    }
+    red[threadIdx.x] = m;
+    __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+        if (threadIdx.x < w) {
+            const float a = red[threadIdx.x], b = red[threadIdx.x + w];
+            red[threadIdx.x] = a != a || b != b ? __int_as_float(0x7fc00000) : fmaxf(a, b);
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) cmax[blockIdx.x] = red[0];
+}
+
+// two float32 operations per instruction, each rounded as the single ones are
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// Bound by float32 issue.  A CTA takes 8 x (256 / TX) rows against tiles of
+// 8 x TX centers; a thread holds 8 x 8 distances (two centers to a register
+// pair), so every dimension costs it 4 16-byte shared loads for 64 add + 64
+// fma, done as 32 + 32 two-wide instructions.  TX = 16 when n > 64, else 8
+// (a tile of 128 centers would be mostly padding).
+constexpr int KM_KC = 32;  // dimensions per shared-memory pass
+template <int DT, int TX>
+__global__ void __launch_bounds__(256) km_assign_kernel(const void *X, int64_t N, int d, int dp, int n,
+                                                        const float *cneg, const float *cmax, int32_t *assign,
+                                                        int32_t *amb, int32_t *namb) {
+    constexpr int TY = 256 / TX, BM = 8 * TY, BN = 8 * TX;
+    constexpr int LDX = BM + 4, LDC = BN + 4;
+    __shared__ __align__(16) float xs[KM_KC * LDX];
+    __shared__ __align__(16) float cs[KM_KC * LDC];
+    const int p = blockIdx.y, tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+    const int64_t r0 = (int64_t)blockIdx.x * BM;
+    const float *cp = cneg + (int64_t)p * n * dp;
+    const float inf = __int_as_float(0x7f800000);
+    float m1[8], m2[8];
+    int arg[8];
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        m1[i] = m2[i] = inf;
+        arg[i] = 0;
+    }
+    for (int c0 = 0; c0 < n; c0 += BN) {
+        uint64_t acc[8][4];
+#pragma unroll
+        for (int i = 0; i < 8; i++)
+#pragma unroll
+            for (int j = 0; j < 4; j++) acc[i][j] = 0ull;
+        for (int k0 = 0; k0 < dp; k0 += KM_KC) {
+            const int kc = dp - k0 < KM_KC ? dp - k0 : KM_KC;
+            __syncthreads();
+            if (c0 == 0 || dp > KM_KC)  // the rows stay when one pass holds a whole part
+                for (int e = tid; e < BM * KM_KC; e += 256) {
+                    const int r = e / KM_KC, k = e % KM_KC;
+                    xs[k * LDX + r] =
+                        k < kc && r0 + r < N ? km_elem<DT>(X, (r0 + r) * d + (int64_t)p * dp + k0 + k) : 0.f;
+                }
+            for (int e = tid; e < BN * KM_KC; e += 256) {
+                const int j = e / KM_KC, k = e % KM_KC;
+                cs[k * LDC + j] = k < kc && c0 + j < n ? cp[(int64_t)(c0 + j) * dp + k0 + k] : 0.f;
+            }
+            __syncthreads();
+#pragma unroll 2
+            for (int k = 0; k < kc; k++) {
+                const float4 xa = *(const float4 *)&xs[k * LDX + 4 * ty];
+                const float4 xb = *(const float4 *)&xs[k * LDX + BM / 2 + 4 * ty];
+                const ulonglong2 ca = *(const ulonglong2 *)&cs[k * LDC + 4 * tx];
+                const ulonglong2 cb = *(const ulonglong2 *)&cs[k * LDC + BN / 2 + 4 * tx];
+                const float x[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
+                const uint64_t c[4] = {ca.x, ca.y, cb.x, cb.y};
+#pragma unroll
+                for (int i = 0; i < 8; i++) {
+                    const uint64_t xx = pack2(x[i], x[i]);
+#pragma unroll
+                    for (int j = 0; j < 4; j++) {
+                        const uint64_t t = add2(xx, c[j]);
+                        acc[i][j] = fma2(t, t, acc[i][j]);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; i++)
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                float v[2];
+                unpack2(acc[i][j], v[0], v[1]);
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    const int c = c0 + (j >> 1) * (BN / 2) + 4 * tx + 2 * (j & 1) + h;
+                    if (c >= n) continue;
+                    if (v[h] < m1[i]) {
+                        m2[i] = m1[i];
+                        m1[i] = v[h];
+                        arg[i] = c;
+                    } else if (v[h] < m2[i]) {
+                        m2[i] = v[h];
+                    }
+                }
+            }
+    }
+    const float cm = cmax[p];
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        for (int off = TX / 2; off > 0; off >>= 1) {  // the TX threads of a row are neighbours in a warp
+            const float o1 = __shfl_xor_sync(0xffffffffu, m1[i], off), o2 = __shfl_xor_sync(0xffffffffu, m2[i], off);
+            const int oa = __shfl_xor_sync(0xffffffffu, arg[i], off);
+            m2[i] = fminf(fmaxf(m1[i], o1), fminf(m2[i], o2));
+            if (o1 < m1[i]) {
+                m1[i] = o1;
+                arg[i] = oa;
+            }
+        }
+        const int64_t r = r0 + (i >> 2) * (BM / 2) + 4 * ty + (i & 3);
+        if (tx == 0 && r < N) {
+            assign[(int64_t)p * N + r] = arg[i];
+            // not so for NaN: infinities and NaN take the exact scan
+            const bool sure = m2[i] - km_eps(m2[i], cm, dp) > m1[i] + km_eps(m1[i], cm, dp);
+            if (!sure) amb[(int64_t)p * N + atomicAdd(&namb[p], 1)] = (int32_t)r;
+        }
+    }
+}
+
+// the fp64 scan of the rows float32 left open: one warp per row
+template <int DT>
+__global__ void km_exact_kernel(const void *X, int64_t N, int d, int dp, int n, const double *C, const int32_t *amb,
+                                const int32_t *namb, int32_t *assign) {
+    const int p = blockIdx.y, lane = lane_id();
+    const double *Cp = C + (int64_t)p * n * dp;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < namb[p]; w += warps) {
+        const int64_t r = amb[(int64_t)p * N + w];
+        double best = 0.0;
+        int arg = n;
+        bool nan0 = false;
+        for (int j = lane; j < n; j += 32) {
+            double s = 0.0;
+            for (int e = 0; e < dp; e++) {
+                const double t =
+                    __dsub_rn((double)km_elem<DT>(X, r * d + (int64_t)p * dp + e), __ldg(Cp + (int64_t)j * dp + e));
+                s = __dadd_rn(s, __dmul_rn(t, t));
+            }
+            if (j == 0 && s != s) nan0 = true;
+            if (s == s && (arg == n || s < best)) {
+                best = s;
+                arg = j;
+            }
+        }
+        for (int off = 16; off > 0; off >>= 1) {
+            const double ob = __shfl_xor_sync(0xffffffffu, best, off);
+            const int oa = __shfl_xor_sync(0xffffffffu, arg, off);
+            if (oa < n && (arg == n || ob < best || (ob == best && oa < arg))) {
+                best = ob;
+                arg = oa;
+            }
+        }
+        // a sequential scan starts from center 0 and nothing compares below a NaN
+        if (__any_sync(0xffffffffu, nan0) || arg == n) arg = 0;
+        if (lane == 0) assign[(int64_t)p * N + r] = arg;
+    }
+}
+
+// Cluster sums of the bytes of every part: integers, so any order gives the
+// same sums.  A CTA adds its share of the rows in shared memory (32 bits hold
+// 2^24 rows of 255; neighbouring lanes add to neighbouring dimensions, without
+// bank conflicts) and flushes what is not zero.  One global atomic per element
+// took 190 us per part of 200,000 x 32 bytes.
+__global__ void km_accumulate_u8_kernel(const uint8_t *X, int64_t N, int d, int dp, int n, const int32_t *assign,
+                                        unsigned long long *isums, unsigned long long *counts) {
+    extern __shared__ uint32_t sums[];  // n * dp, then n counts
+    uint32_t *cnt = sums + n * dp;
+    const int p = blockIdx.y;
+    for (int i = threadIdx.x; i < n * dp + n; i += blockDim.x) sums[i] = 0;
+    __syncthreads();
+    const int64_t share = (N + gridDim.x - 1) / gridDim.x;
+    const int64_t lo = blockIdx.x * share, hi = lo + share < N ? lo + share : N;
+    const int lane = lane_id(), nw = blockDim.x >> 5;
+    for (int64_t r = lo + (threadIdx.x >> 5); r < hi; r += nw) {
+        const int j = assign[(int64_t)p * N + r];
+        const uint8_t *x = X + r * d + (int64_t)p * dp;
+        for (int e = lane; e < dp; e += 32) atomicAdd(&sums[j * dp + e], (uint32_t)x[e]);
+        if (lane == 0) atomicAdd(&cnt[j], 1u);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < n * dp; i += blockDim.x)
+        if (sums[i]) atomicAdd(&isums[(int64_t)p * n * dp + i], (unsigned long long)sums[i]);
+    for (int i = threadIdx.x; i < n; i += blockDim.x)
+        if (cnt[i]) atomicAdd(&counts[(int64_t)p * n + i], (unsigned long long)cnt[i]);
+}
+
+// fp64 sums: one warp per row, so that the lanes' atomics fall in one line
+template <int DT>
+__global__ void km_accumulate_kernel(const void *X, int64_t N, int d, int dp, int n, const int32_t *assign,
                                      unsigned long long *isums, double *fsums, unsigned long long *counts) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    int j = assign[i];
-    atomicAdd(&counts[j], 1ull);
-    for (int e = 0; e < dp; e++) {
-        int64_t at = i * d + (int64_t)p * dp + e;
-        if (DT == ANN_U8) atomicAdd(&isums[(int64_t)j * dp + e], (unsigned long long)((const uint8_t *)X)[at]);
-        else atomicAdd(&fsums[(int64_t)j * dp + e], (double)((const float *)X)[at]);
+    const int p = blockIdx.y, lane = lane_id();
+    const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (r >= N) return;
+    const int64_t j = (int64_t)p * n + assign[(int64_t)p * N + r];
+    if (lane == 0) atomicAdd(&counts[j], 1ull);
+    for (int e = lane; e < dp; e += 32) {
+        const int64_t at = r * d + (int64_t)p * dp + e;
+        if (DT == ANN_U8) atomicAdd(&isums[j * dp + e], (unsigned long long)((const uint8_t *)X)[at]);
+        else atomicAdd(&fsums[j * dp + e], (double)((const float *)X)[at]);
     }
 }
 
 template <int DT>
-__global__ void km_update_kernel(int n, int dp, const unsigned long long *isums, const double *fsums,
+__global__ void km_update_kernel(int total, int dp, const unsigned long long *isums, const double *fsums,
                                  const unsigned long long *counts, double *C) {
-    int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n * dp) return;
+    int idx = blockIdx.x * blockDim.x + threadIdx.x;  // over P*n*dp
+    if (idx >= total) return;
     int j = idx / dp;
     unsigned long long c = counts[j];
     if (c == 0) return;  // empty cluster keeps its center
@@ -650,46 +863,76 @@ extern "C" int ann_train_centers(const void *train, int dtype, int64_t ntrain, i
     for (int j = 0; j < n; j++) ANN_ARG(init_rows[j] >= 0 && init_rows[j] < ntrain, "init row out of range");
     cudaStream_t s = (cudaStream_t)stream;
     const int dp = d / P;
+    int dev = 0, optin = 0, nsm = 0;
+    ANN_CUDA(cudaGetDevice(&dev));
+    ANN_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    ANN_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    if (dp > optin / 512) return fail(ANN_ERR_CUDA, "a part has too many dimensions");
+    const int total = P * n * dp;
     DBuf<double> C;
     DBuf<int64_t> rows;
-    DBuf<int32_t> assign;
+    DBuf<int32_t> assign, amb, namb;
     DBuf<unsigned long long> isums, counts;
     DBuf<double> fsums;
-    ANN_CUDA_ALLOC(C, (size_t)P * n * dp);
+    DBuf<float> cneg, cmax;
+    ANN_CUDA_ALLOC(C, total);
     ANN_CUDA_ALLOC(rows, n);
-    ANN_CUDA_ALLOC(assign, ntrain);
-    ANN_CUDA_ALLOC(isums, (size_t)n * dp);
-    ANN_CUDA_ALLOC(fsums, (size_t)n * dp);
-    ANN_CUDA_ALLOC(counts, n);
+    ANN_CUDA_ALLOC(assign, (size_t)P * ntrain);
+    ANN_CUDA_ALLOC(amb, (size_t)P * ntrain);
+    ANN_CUDA_ALLOC(namb, P);
+    ANN_CUDA_ALLOC(isums, total);
+    ANN_CUDA_ALLOC(fsums, total);
+    ANN_CUDA_ALLOC(counts, (size_t)P * n);
+    ANN_CUDA_ALLOC(cneg, total);
+    ANN_CUDA_ALLOC(cmax, P);
     ANN_CUDA(cudaMemcpyAsync(rows.p, init_rows, 8 * n, cudaMemcpyHostToDevice, s));
-    const int total = P * n * dp;
     if (dtype == ANN_U8) km_init_kernel<ANN_U8><<<nblk(total), 256, 0, s>>>(train, d, dp, P, n, rows.p, C.p);
     else km_init_kernel<ANN_F32><<<nblk(total), 256, 0, s>>>(train, d, dp, P, n, rows.p, C.p);
-    const int TB = 128;
-    size_t sm = sizeof(float) * dp * TB;
-    if (dtype == ANN_U8)
-        ANN_CUDA(cudaFuncSetAttribute(km_assign_kernel<ANN_U8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    else
-        ANN_CUDA(cudaFuncSetAttribute(km_assign_kernel<ANN_F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    for (int p = 0; p < P; p++) {
-        double *Cp = C.p + (size_t)p * n * dp;
-        for (int it = 0; it < iters; it++) {
-            ANN_CUDA(cudaMemsetAsync(isums.p, 0, 8 * (size_t)n * dp, s));
-            ANN_CUDA(cudaMemsetAsync(fsums.p, 0, 8 * (size_t)n * dp, s));
-            ANN_CUDA(cudaMemsetAsync(counts.p, 0, 8 * (size_t)n, s));
-            if (dtype == ANN_U8) {
-                km_assign_kernel<ANN_U8><<<nblk(ntrain, TB), TB, sm, s>>>(train, ntrain, d, dp, p, n, Cp, assign.p);
-                km_accumulate_kernel<ANN_U8><<<nblk(ntrain), 256, 0, s>>>(train, ntrain, d, dp, p, assign.p, isums.p,
-                                                                          fsums.p, counts.p);
-                km_update_kernel<ANN_U8><<<nblk(n * dp), 256, 0, s>>>(n, dp, isums.p, fsums.p, counts.p, Cp);
-            } else {
-                km_assign_kernel<ANN_F32><<<nblk(ntrain, TB), TB, sm, s>>>(train, ntrain, d, dp, p, n, Cp, assign.p);
-                km_accumulate_kernel<ANN_F32><<<nblk(ntrain), 256, 0, s>>>(train, ntrain, d, dp, p, assign.p, isums.p,
-                                                                           fsums.p, counts.p);
-                km_update_kernel<ANN_F32><<<nblk(n * dp), 256, 0, s>>>(n, dp, isums.p, fsums.p, counts.p, Cp);
-            }
-            ANN_CUDA(cudaGetLastError());
+    // all parts of an iteration in one launch (blockIdx.y); byte sums in shared
+    // memory where a CTA's copy of a part's sums fits and cannot overflow
+    const int BM = n > 64 ? 128 : 256;
+    const dim3 grid_a((unsigned)((ntrain + BM - 1) / BM), (unsigned)P);
+    const size_t sum_bytes = 4 * ((size_t)n * dp + n);
+    const unsigned gx = (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)2 * nsm / P, (ntrain + 63) / 64));
+    const bool shared_sums = dtype == ANN_U8 && sum_bytes <= (size_t)optin && (ntrain + gx - 1) / gx < (1 << 24);
+    if (shared_sums)
+        ANN_CUDA(cudaFuncSetAttribute(km_accumulate_u8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)sum_bytes));
+    for (int it = 0; it < iters; it++) {
+        ANN_CUDA(cudaMemsetAsync(isums.p, 0, 8 * (size_t)total, s));
+        ANN_CUDA(cudaMemsetAsync(fsums.p, 0, 8 * (size_t)total, s));
+        ANN_CUDA(cudaMemsetAsync(counts.p, 0, 8 * (size_t)P * n, s));
+        ANN_CUDA(cudaMemsetAsync(namb.p, 0, 4 * (size_t)P, s));
+        km_prep_kernel<<<P, 256, 0, s>>>(C.p, n, dp, cneg.p, cmax.p);
+        const dim3 grid_e((unsigned)(4 * nsm), (unsigned)P), grid_w(nblk(32 * ntrain), (unsigned)P);
+        if (dtype == ANN_U8) {
+            if (n > 64)
+                km_assign_kernel<ANN_U8, 16><<<grid_a, 256, 0, s>>>(train, ntrain, d, dp, n, cneg.p, cmax.p, assign.p,
+                                                                    amb.p, namb.p);
+            else
+                km_assign_kernel<ANN_U8, 8><<<grid_a, 256, 0, s>>>(train, ntrain, d, dp, n, cneg.p, cmax.p, assign.p,
+                                                                   amb.p, namb.p);
+            km_exact_kernel<ANN_U8><<<grid_e, 256, 0, s>>>(train, ntrain, d, dp, n, C.p, amb.p, namb.p, assign.p);
+            if (shared_sums)
+                km_accumulate_u8_kernel<<<dim3(gx, P), 512, sum_bytes, s>>>((const uint8_t *)train, ntrain, d, dp, n,
+                                                                            assign.p, isums.p, counts.p);
+            else
+                km_accumulate_kernel<ANN_U8><<<grid_w, 256, 0, s>>>(train, ntrain, d, dp, n, assign.p, isums.p,
+                                                                    fsums.p, counts.p);
+            km_update_kernel<ANN_U8><<<nblk(total), 256, 0, s>>>(total, dp, isums.p, fsums.p, counts.p, C.p);
+        } else {
+            if (n > 64)
+                km_assign_kernel<ANN_F32, 16><<<grid_a, 256, 0, s>>>(train, ntrain, d, dp, n, cneg.p, cmax.p, assign.p,
+                                                                     amb.p, namb.p);
+            else
+                km_assign_kernel<ANN_F32, 8><<<grid_a, 256, 0, s>>>(train, ntrain, d, dp, n, cneg.p, cmax.p, assign.p,
+                                                                    amb.p, namb.p);
+            km_exact_kernel<ANN_F32><<<grid_e, 256, 0, s>>>(train, ntrain, d, dp, n, C.p, amb.p, namb.p, assign.p);
+            km_accumulate_kernel<ANN_F32><<<grid_w, 256, 0, s>>>(train, ntrain, d, dp, n, assign.p, isums.p, fsums.p,
+                                                                 counts.p);
+            km_update_kernel<ANN_F32><<<nblk(total), 256, 0, s>>>(total, dp, isums.p, fsums.p, counts.p, C.p);
         }
+        ANN_CUDA(cudaGetLastError());
     }
     km_store_kernel<<<nblk(total), 256, 0, s>>>(total, dtype, C.p, out_centers);
     if (out_centers_f64)

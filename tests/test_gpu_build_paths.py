@@ -1,0 +1,55 @@
+"""Index-build kernels at the edges of their tiles and of their dispatch rules,
+against the CPU oracle (whole numbers exactly; fp64 centers within the rounding
+of a differently ordered sum)."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+import oracle  # noqa: E402
+from paper_1312_3062_gb300 import datagen  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def ann():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_1312_3062_gb300 import _build
+    _build.build()
+    from paper_1312_3062_gb300 import ann as mod
+    return mod
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+@pytest.mark.parametrize("kind,N,d,P,n", [("u8", 300, 16, 1, 1), ("u8", 129, 16, 4, 64), ("u8", 1000, 100, 4, 65),
+                                          ("u8", 2049, 96, 2, 256), ("ties", 600, 64, 4, 70),
+                                          ("f32", 257, 100, 2, 64), ("f32", 900, 264, 2, 130),
+                                          ("far", 513, 96, 3, 33), ("huge", 300, 32, 2, 8)])
+def test_kmeans_tile_edges_and_rows_left_to_fp64(ann, kind, N, d, P, n):
+    rng = np.random.default_rng(N)
+    if kind == "ties":  # many equidistant centers: every row needs the fp64 scan and its tie rule
+        X = rng.integers(0, 3, size=(N, d)).astype(np.uint8) * 2
+    elif kind == "u8":
+        X = datagen.mixture(N, N, d, 9, np.uint8)
+    elif kind == "far":  # float32 cannot separate the centers
+        X = (4096.0 + rng.standard_normal((N, d)) * 0.01).astype(np.float32)
+    elif kind == "huge":  # squares overflow float32, not fp64
+        X = (rng.standard_normal((N, d)) * 1e25).astype(np.float32)
+    else:
+        X = datagen.mixture(N, N, d, 9, np.float32)
+    init = rng.permutation(N)[:n]
+    want = oracle.kmeans(X, P, n, 2, init)
+    got, got64 = ann.ann_train_centers(dev(X), P, n, 2, init, want_f64=True)
+    if X.dtype == np.uint8:
+        np.testing.assert_array_equal(got64.cpu().numpy(), want)
+        np.testing.assert_array_equal(got.cpu().numpy(), oracle.round_centers(want, np.uint8))
+    else:
+        # sums of up to N equal-sized terms in another order: N * 2^-53 relative to the largest term
+        np.testing.assert_allclose(got64.cpu().numpy(), want, rtol=0, atol=N * 2.0 ** -52 * np.abs(X).max())
