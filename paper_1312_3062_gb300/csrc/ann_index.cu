@@ -11,6 +11,7 @@
 #include <cub/cub.cuh>
 #include <functional>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "ann_device.cuh"
@@ -358,69 +359,202 @@ __global__ void km_store_kernel(int total, int dtype, const double *C, void *out
 // then the b nearest references of every bridge vector.
 // ---------------------------------------------------------------------------
 // A tuple of ranks r can be among the t smallest only if prod_p (r_p + 1) <= t
-// (every tuple below it in every coordinate precedes it).  Each warp scores
-// all such candidate tuples for its reference and sorts them by
-// (key, ranks): exactly the first t tuples of the multi-sequence order.
+// (every tuple below it in every coordinate precedes it): the candidates.  The
+// other way round a tuple with prod_p (r_p + 1) >= t has t tuples at or below
+// its key, so the smallest key over such tuples (`bound`: the minimal ones) is
+// an upper limit of the t-th smallest.  One warp per reference: the candidates
+// up to that limit go to a buffer (300 to 1200 of the 3575 candidates of
+// P = 4, t = 100 on SIFT-shaped keys), and a bisection over their distinct
+// (key, ranks) composites finds the t-th.  A buffer that overflows lowers the
+// limit by the same bisection over all candidates.  The t pairs are written in
+// no particular order: the sort by bridge that follows does not need one.
+// Issue-bound (the part tables and sorts, then one pass over the candidates).
+// Sorting all candidates by one warp in shared memory took 210 ms for
+// 200,000 x 128 bytes, P = 4, n = 256, t = 100; this takes 5.3 ms.
+constexpr int BG_WARPS = 4;
+
+// One part of a row against one center, 16 bytes per load (dp * element size a
+// multiple of 16); the operations and their order are part_key_lane's.
 template <int DT>
-__global__ void bg_topt_kernel(const void *X, int64_t N, int d, int P, int n, const void *C,
-                               const uint32_t *cands, int ncand, int Lc, int t_eff, uint32_t slice,
-                               uint64_t *out_keys, uint32_t *out_vals) {
+__device__ __forceinline__ uint32_t part_key_wide(const uint8_t *qbytes, const void *C, int p, int c, int n, int dp) {
+    if (DT == ANN_U8) {
+        const uint4 *cent = (const uint4 *)((const uint8_t *)C + ((int64_t)p * n + c) * dp);
+        const uint4 *qp = (const uint4 *)(qbytes + p * dp);
+        uint32_t acc = 0;
+        for (int w = 0; w < dp / 16; w++) {
+            const uint4 a = qp[w], b = __ldg(cent + w);
+            uint32_t df = __vabsdiffu4(a.x, b.x);
+            acc = __dp4a(df, df, acc);
+            df = __vabsdiffu4(a.y, b.y);
+            acc = __dp4a(df, df, acc);
+            df = __vabsdiffu4(a.z, b.z);
+            acc = __dp4a(df, df, acc);
+            df = __vabsdiffu4(a.w, b.w);
+            acc = __dp4a(df, df, acc);
+        }
+        return acc;
+    }
+    const float4 *cent = (const float4 *)((const float *)C + ((int64_t)p * n + c) * dp);
+    const float4 *qp = (const float4 *)((const float *)qbytes + p * dp);
+    float hi = 0.f, lo = 0.f;
+    for (int w = 0; w < dp / 4; w++) {
+        const float4 a = qp[w], b = __ldg(cent + w);
+        df_acc_sqdiff(a.x, b.x, hi, lo);
+        df_acc_sqdiff(a.y, b.y, hi, lo);
+        df_acc_sqdiff(a.z, b.z, hi, lo);
+        df_acc_sqdiff(a.w, b.w, hi, lo);
+    }
+    return __float_as_uint(__fadd_rn(hi, lo));
+}
+
+// sort part p's keys by (key, center id) in registers: the keys in rank order
+// over the unsorted ones, the center id at each rank
+template <int EPL, bool PACK>
+__device__ __forceinline__ void bg_sort_part(uint32_t *key, uint8_t *cid, int n) {
+    const int lane = lane_id();
+    using K = typename std::conditional<PACK, uint32_t, uint64_t>::type;
+    constexpr int SH = PACK ? 8 : 32;
+    K v[EPL];
+#pragma unroll
+    for (int s = 0; s < EPL; s++) {
+        const int c = lane * EPL + s;
+        v[s] = c < n ? (((K)key[c]) << SH) | (K)c : ~(K)0;
+    }
+    reg_bitonic_sort_t<EPL, K>(v);
+    __syncwarp();
+#pragma unroll
+    for (int s = 0; s < EPL; s++) {
+        const int r = lane * EPL + s;
+        if (r < n) {
+            key[r] = (uint32_t)(v[s] >> SH);
+            cid[r] = (uint8_t)(v[s] & (PACK ? 0xffu : 0xffffffffu));
+        }
+    }
+}
+
+template <bool PACK>
+__device__ __forceinline__ void bg_sort_any(uint32_t *key, uint8_t *cid, int n) {
+    if (n <= 32) bg_sort_part<1, PACK>(key, cid, n);
+    else if (n <= 64) bg_sort_part<2, PACK>(key, cid, n);
+    else if (n <= 128) bg_sort_part<4, PACK>(key, cid, n);
+    else bg_sort_part<8, PACK>(key, cid, n);
+}
+
+// (key, ranks) of a packed rank tuple; ~0 when its key is above limk
+// (float32: a bound taken downwards first, the exact sum only below it)
+template <int DT>
+__device__ __forceinline__ uint64_t bg_composite(const uint32_t *skey, int P, int n, uint32_t rr, uint32_t limk) {
+    uint32_t s[kMaxP];
+#pragma unroll
+    for (int p = 0; p < kMaxP; p++) s[p] = p < P ? skey[p * n + ((rr >> (8 * (P - 1 - p))) & 255u)] : 0u;
+    if (DT == ANN_F32) {
+        const uint32_t low = KeyOps<DT>::add_lo(KeyOps<DT>::add_lo(s[0], s[1]), KeyOps<DT>::add_lo(s[2], s[3]));
+        if (__uint_as_float(low) > __uint_as_float(limk)) return ~0ull;  // a NaN goes on to the exact sum
+    }
+    const uint32_t key = KeyOps<DT>::sum4(s[0], s[1], s[2], s[3]);
+    return key > limk ? ~0ull : ((uint64_t)key << 32) | rr;
+}
+
+// how many candidates lie at or below lim; the first cap of them to buf
+template <int DT>
+__device__ __forceinline__ uint32_t bg_collect(const uint32_t *skey, int P, int n, const uint32_t *cands, int ncand,
+                                               uint64_t lim, uint64_t *buf, uint32_t cap) {
+    const int lane = lane_id();
+    uint32_t c = 0;
+    for (int i0 = 0; i0 < ncand; i0 += 32) {
+        const int i = i0 + lane;
+        const uint64_t v =
+            i < ncand ? bg_composite<DT>(skey, P, n, __ldg(cands + i), (uint32_t)(lim >> 32)) : ~0ull;
+        const bool in = v <= lim && i < ncand && v != ~0ull;
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        const uint32_t pos = c + __popc(m & ((1u << lane) - 1));
+        if (in && pos < cap) buf[pos] = v;
+        c += __popc(m);
+    }
+    __syncwarp();
+    return c;
+}
+
+template <int DT>
+__global__ void __launch_bounds__(32 * BG_WARPS) bg_topt_kernel(const void *X, int64_t N, int d, int P, int n,
+                                                                const void *C, const uint32_t *cands, int ncand,
+                                                                const uint32_t *bound, int nbound, uint32_t cap,
+                                                                int t_eff, uint32_t slice, uint64_t *out_keys,
+                                                                uint32_t *out_vals) {
     extern __shared__ __align__(16) uint8_t smem_all[];
     const int warp = threadIdx.x >> 5, lane = lane_id();
     uint8_t *sm = smem_all + (size_t)warp * slice;
     const int vb = d * (DT == ANN_U8 ? 1 : 4);
     uint8_t *qb = sm;
-    uint32_t *D = (uint32_t *)(sm + align_up16(vb));
-    uint32_t *skey = D + P * n;
+    uint32_t *skey = (uint32_t *)(sm + align_up16(vb));
     uint8_t *scid = (uint8_t *)(skey + P * n);
-    uint64_t *tmp = (uint64_t *)(sm + align_up16(align_up16(vb) + 8 * P * n + P * n));
+    uint64_t *buf = (uint64_t *)(sm + align_up16(align_up16(vb) + 5 * P * n));
     const int dp = d / P;
-    int Lp = 1;
-    while (Lp < n) Lp <<= 1;
+    const bool wide = dp % (DT == ANN_U8 ? 16 : 4) == 0;
+    const bool pack = DT == ANN_U8 && (uint64_t)dp * 65025u < (1u << 24);
     const int64_t gw = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
     const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t i = gw; i < N; i += nw) {
         const uint4 *src = (const uint4 *)((const uint8_t *)X + i * (int64_t)vb);
         for (int c = lane; c < (vb >> 4); c += 32) ((uint4 *)qb)[c] = __ldg(src + c);
         __syncwarp();
-        for (int idx = lane; idx < P * n; idx += 32) D[idx] = part_key_lane<DT>(qb, C, idx / n, idx % n, n, dp);
+        for (int idx = lane; idx < P * n; idx += 32) {
+            const int p = idx / n, c = idx - p * n;
+            skey[idx] = wide ? part_key_wide<DT>(qb, C, p, c, n, dp) : part_key_lane<DT>(qb, C, p, c, n, dp);
+        }
         __syncwarp();
         for (int p = 0; p < P; p++) {
-            for (int r = lane; r < Lp; r += 32)
-                tmp[r] = r < n ? (((uint64_t)D[p * n + r]) << 32) | (uint32_t)r : ~0ull;
-            __syncwarp();
-            warp_sort_pairs(tmp, nullptr, Lp);
-            for (int r = lane; r < n; r += 32) {
-                skey[p * n + r] = (uint32_t)(tmp[r] >> 32);
-                scid[p * n + r] = (uint8_t)(uint32_t)tmp[r];
-            }
-            __syncwarp();
-        }
-        for (int c = lane; c < Lc; c += 32) {
-            uint64_t v = ~0ull;
-            if (c < ncand) {
-                uint32_t rr = cands[c];
-                uint32_t r[kMaxP];
-                for (int p = 0; p < P; p++) r[p] = (rr >> (8 * (P - 1 - p))) & 255u;
-                // Sec. 4.2: the sum of the part keys (float32: nearest to the exact sum)
-                const uint32_t key = KeyOps<DT>::sum4(skey[r[0]], skey[n + r[1]], P > 2 ? skey[2 * n + r[2]] : 0u,
-                                                      P > 3 ? skey[3 * n + r[3]] : 0u);
-                v = ((uint64_t)key << 32) | rr;
-            }
-            tmp[c] = v;
+            if (pack) bg_sort_any<true>(skey + p * n, scid + p * n, n);
+            else bg_sort_any<false>(skey + p * n, scid + p * n, n);
         }
         __syncwarp();
-        warp_sort_pairs(tmp, nullptr, Lc);
-        for (int j = lane; j < t_eff; j += 32) {
-            uint64_t v = tmp[j];
-            uint32_t rr = (uint32_t)v;
-            uint64_t bid = 0;
-            for (int p = 0; p < P; p++) {
-                uint32_t r = (rr >> (8 * (P - 1 - p))) & 255u;
-                bid = bid * (uint64_t)n + scid[p * n + r];
+        uint32_t limk = 0xffffffffu;
+        for (int c = lane; c < nbound; c += 32)
+            limk = min(limk, (uint32_t)(bg_composite<DT>(skey, P, n, __ldg(bound + c), limk) >> 32));
+        limk = __reduce_min_sync(0xffffffffu, limk);
+        // at or below hi there are at least t candidates, at or below lo fewer
+        uint64_t lo = bg_composite<DT>(skey, P, n, 0u, 0xffffffffu), hi = ((uint64_t)limk << 32) | 0xffffffffull;
+        if (t_eff == 1) hi = lo;
+        uint32_t c = bg_collect<DT>(skey, P, n, cands, ncand, hi, buf, cap);
+        while (c > cap) {
+            const uint64_t mid = lo + (hi - lo) / 2;
+            const uint32_t cm = bg_collect<DT>(skey, P, n, cands, ncand, mid, buf, cap);
+            if (cm < (uint32_t)t_eff) {
+                lo = mid;
+            } else {
+                hi = mid;
+                c = cm;
             }
-            out_keys[i * t_eff + j] = (bid << 32) | (v >> 32);
-            out_vals[i * t_eff + j] = (uint32_t)i;
+        }
+        // the t-th smallest composite of the buffer
+        if (c > (uint32_t)t_eff)
+            while (hi - lo > 1) {
+                const uint64_t mid = lo + (hi - lo) / 2;
+                uint32_t cm = 0;
+                for (uint32_t j = lane; j < c; j += 32) cm += buf[j] <= mid;
+                cm = __reduce_add_sync(0xffffffffu, cm);
+                if (cm < (uint32_t)t_eff) {
+                    lo = mid;
+                } else {
+                    hi = mid;
+                    if (cm == (uint32_t)t_eff) break;
+                }
+            }
+        uint32_t at = 0;
+        for (uint32_t j0 = 0; j0 < c; j0 += 32) {
+            const uint32_t j = j0 + lane;
+            const uint64_t v = j < c ? buf[j] : ~0ull;
+            const bool keep = j < c && v <= hi;
+            const unsigned m = __ballot_sync(0xffffffffu, keep);
+            if (keep) {
+                const uint32_t rr = (uint32_t)v;
+                uint64_t bid = 0;
+                for (int p = 0; p < P; p++) bid = bid * (uint64_t)n + scid[p * n + ((rr >> (8 * (P - 1 - p))) & 255u)];
+                const int64_t o = i * t_eff + at + __popc(m & ((1u << lane) - 1));
+                out_keys[o] = (bid << 32) | (v >> 32);
+                out_vals[o] = (uint32_t)i;
+            }
+            at += __popc(m);
         }
         __syncwarp();
     }
@@ -703,19 +837,51 @@ static int build_bridges_gpu(ann_index *ix, cudaStream_t s) {
     while (Lc < ncand) Lc <<= 1;
     int Lp = 1;
     while (Lp < n) Lp <<= 1;
-    DBuf<uint32_t> dcand;
+    // minimal tuples with prod(r_p + 1) >= t_eff: one step up from a candidate
+    // and no longer so one step down; evenly thinned to a few hundred
+    std::vector<uint32_t> bound;
+    for (uint32_t v : cands) {
+        int64_t prod = 1;
+        int r[kMaxP];
+        for (int p = 0; p < P; p++) {
+            r[p] = (int)((v >> (8 * (P - 1 - p))) & 255u);
+            prod *= r[p] + 1;
+        }
+        if (prod >= t_eff) bound.push_back(v);  // t_eff = prod: its own bound
+        for (int p = 0; p < P; p++) {
+            if (r[p] + 1 >= n) continue;
+            const int64_t up = prod / (r[p] + 1) * (r[p] + 2);
+            bool minimal = up >= t_eff;
+            r[p]++;
+            for (int q = 0; q < P; q++)
+                if (r[q] > 0 && up / (r[q] + 1) * r[q] >= t_eff) minimal = false;
+            r[p]--;
+            if (minimal) bound.push_back(v + (1u << (8 * (P - 1 - p))));
+        }
+    }
+    std::sort(bound.begin(), bound.end());
+    bound.erase(std::unique(bound.begin(), bound.end()), bound.end());
+    const size_t thin = (bound.size() + 511) / 512;
+    for (size_t i = 0; thin > 1 && i * thin < bound.size(); i++) bound[i] = bound[i * thin];
+    if (thin > 1) bound.resize((bound.size() + thin - 1) / thin);
+    const int nbound = (int)bound.size();
+    DBuf<uint32_t> dcand, dbound;
     ANN_CUDA_ALLOC(dcand, ncand);
+    ANN_CUDA_ALLOC(dbound, nbound);
     ANN_CUDA(cudaMemcpyAsync(dcand.p, cands.data(), 4 * ncand, cudaMemcpyHostToDevice, s));
+    ANN_CUDA(cudaMemcpyAsync(dbound.p, bound.data(), 4 * nbound, cudaMemcpyHostToDevice, s));
     const int vb = dv.d * (DT == ANN_U8 ? 1 : 4);
-    uint32_t slice = align_up16(align_up16(vb) + 8 * P * n + P * n) + 8 * std::max(Lc, Lp);
-    slice = align_up16(slice);
     int dev;
     ANN_CUDA(cudaGetDevice(&dev));
     int optin = 0, nsm = 0;
     ANN_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     ANN_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    int warps = (int)std::min<int64_t>(8, optin / slice);
-    if (warps < 1) return fail(ANN_ERR_CAPACITY, "bridge builder: per-reference state exceeds shared memory");
+    // room for every candidate in shared memory is still what limits t
+    if (align_up16(align_up16(align_up16(vb) + 9 * P * n) + 8 * std::max(Lc, Lp)) > (uint32_t)optin)
+        return fail(ANN_ERR_CAPACITY, "bridge builder: per-reference state exceeds shared memory");
+    const uint32_t cap = Lc <= 1024 ? (uint32_t)Lc : (uint32_t)std::max(1024, t_eff);
+    const uint32_t slice = align_up16(align_up16(align_up16(vb) + 5 * P * n) + 8 * cap);
+    const int warps = std::max(1, std::min(BG_WARPS, (int)(optin / slice)));
     size_t smem = (size_t)warps * slice;
     ANN_CUDA(cudaFuncSetAttribute(bg_topt_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int64_t m = N * t_eff;
@@ -728,7 +894,8 @@ static int build_bridges_gpu(ann_index *ix, cudaStream_t s) {
     int64_t blocks = std::min<int64_t>((N + warps - 1) / warps, (int64_t)nsm * 16);
     if (N > 0)
         bg_topt_kernel<DT><<<(unsigned)blocks, warps * 32, smem, s>>>(dv.X, N, dv.d, P, n, dv.C, dcand.p, ncand,
-                                                                       Lc, t_eff, slice, k0.p, v0.p);
+                                                                       dbound.p, nbound, cap, t_eff, slice, k0.p,
+                                                                       v0.p);
     ANN_CUDA(cudaGetLastError());
     // sort by (bridge id, key); stable, so references stay in id order within ties
     size_t tb = 0;

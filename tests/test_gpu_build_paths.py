@@ -53,3 +53,29 @@ def test_kmeans_tile_edges_and_rows_left_to_fp64(ann, kind, N, d, P, n):
     else:
         # sums of up to N equal-sized terms in another order: N * 2^-53 relative to the largest term
         np.testing.assert_allclose(got64.cpu().numpy(), want, rtol=0, atol=N * 2.0 ** -52 * np.abs(X).max())
+
+
+@pytest.mark.parametrize("kind,N,d,P,n,t,b", [("u8", 70, 64, 4, 256, 100, 5),    # a buffer smaller than the candidates
+                                              ("u8", 33, 48, 2, 256, 700, 2),    # t beyond the buffer's first size
+                                              ("u8", 40, 96, 3, 33, 1, 5),
+                                              ("u8", 40, 64, 4, 3, 500, 8),      # every bridge is among the t nearest
+                                              ("equal", 35, 64, 4, 64, 100, 3),  # all keys equal: ranks decide
+                                              ("f32", 45, 60, 4, 128, 100, 5), ("f32", 40, 36, 2, 100, 100, 1),
+                                              ("f32equal", 33, 16, 4, 48, 100, 5)])
+def test_bridge_lists_where_candidates_are_cut(ann, kind, N, d, P, n, t, b):
+    dt = np.float32 if kind.startswith("f32") else np.uint8
+    rng = np.random.default_rng(N)
+    if kind.endswith("equal"):
+        X = np.ones((N, d), dt)
+        C = np.full((P, n, d // P), 3, dt)
+    else:
+        X = datagen.mixture(N, N, d, 4, dt)
+        C = rng.integers(0, 256, (P, n, d // P)).astype(dt) if dt == np.uint8 else \
+            rng.random((P, n, d // P)).astype(dt) * 0.2
+    want = oracle.bridge_graph(X, C, t, b)
+    ix = ann.Index.create(dev(X), dev(np.zeros((N, 4), np.int32)), dev(C), t=t, b=b)
+    ids, refs = ix.bridges()
+    np.testing.assert_array_equal(ids, want["bridges"])
+    lens = np.diff(want["offsets"])
+    np.testing.assert_array_equal((refs >= 0).sum(1), lens)
+    np.testing.assert_array_equal(refs[refs >= 0], want["refs"])
