@@ -79,3 +79,40 @@ def test_bridge_lists_where_candidates_are_cut(ann, kind, N, d, P, n, t, b):
     lens = np.diff(want["offsets"])
     np.testing.assert_array_equal((refs >= 0).sum(1), lens)
     np.testing.assert_array_equal(refs[refs >= 0], want["refs"])
+
+
+@pytest.mark.parametrize("N,nq,d,k,shift", [(8192, 256, 60, 1, 0), (8193, 257, 100, 32, 0), (9001, 300, 4, 20, 0),
+                                            (8257, 259, 384, 10, 1), (10_003, 256, 36, 7, 3)])
+def test_f32_knn_odd_sizes_and_alignments(ann, N, nq, d, k, shift):
+    X, Q = datagen.mixture(N, N, d, 9, np.float32), datagen.mixture(N, nq, d, 9, np.float32)
+
+    def at(a):  # rows that start `shift` floats off a 16-byte boundary
+        flat = torch.empty(a.size + shift, dtype=torch.float32, device="cuda")
+        flat[shift:] = dev(a.reshape(-1))
+        return flat[shift:].view(a.shape)
+
+    ids, keys = ann.ann_exact_knn(at(X), at(Q), k)
+    want_ids, want_keys = oracle.exact_knn(X, Q, k)
+    np.testing.assert_array_equal(ids.cpu().numpy(), want_ids)
+    np.testing.assert_allclose(keys.cpu().numpy(), want_keys, rtol=1e-5)
+
+
+@pytest.mark.parametrize("kind", ["descending", "late_cluster", "ties"])
+def test_f32_knn_when_the_first_columns_mislead(ann, kind):
+    # the candidate limit starts from the first 4096 columns: here those are
+    # the farthest rows, the near ones come all at once, or most are equal
+    N, nq, d, k = 20_011, 256, 32, 20
+    X, Q = datagen.mixture(5, N, d, 6, np.float32), datagen.mixture(6, nq, d, 6, np.float32)
+    Q[1:] = Q[0] + 0.001 * Q[1:]
+    dist = ((X - Q[0]) ** 2).sum(1)
+    if kind == "descending":
+        X = X[np.argsort(-dist)]
+    elif kind == "late_cluster":
+        X[4096:12_000] = Q[0] + 0.1 * X[4096:12_000]
+    else:
+        X[3000:9000] = X[3000]
+    X = np.ascontiguousarray(X)
+    ids, keys = ann.ann_exact_knn(dev(X), dev(Q), k)
+    want_ids, want_keys = oracle.exact_knn(X, Q, k)
+    np.testing.assert_array_equal(ids.cpu().numpy(), want_ids)
+    np.testing.assert_allclose(keys.cpu().numpy(), want_keys, rtol=1e-5)
