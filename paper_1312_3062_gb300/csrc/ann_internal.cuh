@@ -141,7 +141,6 @@ int search_num_buckets();
 // implemented in ann_knn_tc.cu: exact k-NN of uint8 rows on the tensor cores, d in {64, 128}, k <= 32
 int knn_u8_tensor(const uint8_t *refs, int64_t N, const uint8_t *queries, int64_t nq, int d, int k,
                   int exclude_self, int32_t *out_ids, uint32_t *out_keys, cudaStream_t s);
-bool knn_u8_tensor_fits(int d, int k);
 // implemented in ann_index.cu
 int build_bridge_index_from_host(ann_index *ix, int64_t M, const uint64_t *ids,
                                  const int64_t *offsets, const int32_t *refs);

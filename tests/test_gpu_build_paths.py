@@ -116,3 +116,33 @@ def test_f32_knn_when_the_first_columns_mislead(ann, kind):
     want_ids, want_keys = oracle.exact_knn(X, Q, k)
     np.testing.assert_array_equal(ids.cpu().numpy(), want_ids)
     np.testing.assert_allclose(keys.cpu().numpy(), want_keys, rtol=1e-5)
+
+
+@pytest.mark.parametrize("kind,N,nq,d,k", [
+    ("mix", 5, 1, 64, 8), ("mix", 255, 127, 128, 1), ("mix", 256, 128, 64, 9), ("mix", 257, 129, 128, 16),
+    ("mix", 3001, 33, 128, 17), ("mix", 20_011, 700, 64, 25), ("mix", 70_003, 3, 128, 32), ("mix", 40_000, 2500, 128, 10),
+    ("black_white", 3000, 300, 128, 20), ("white", 700, 130, 128, 32), ("equal", 2000, 140, 64, 24),
+    ("descending", 9000, 200, 128, 10), ("graph", 2500, 0, 128, 24), ("graph", 1100, 0, 64, 31)])
+def test_u8_tensor_knn_tile_edges_and_extreme_rows(ann, kind, N, nq, d, k):
+    rng = np.random.default_rng(N + k)
+    X, Q = datagen.mixture(N, N, d, 7, np.uint8), datagen.mixture(N, max(nq, 1), d, 7, np.uint8)
+    if kind == "black_white":    # the largest norms and products
+        X, Q = (rng.integers(0, 2, X.shape) * 255).astype(np.uint8), (rng.integers(0, 2, Q.shape) * 255).astype(np.uint8)
+    elif kind == "white":
+        X[:] = 255
+        Q[::2] = 255
+        Q[1::2] = 0
+    elif kind == "equal":        # every key equal: ids decide, also across the lists of a row
+        X[:] = X[0]
+    elif kind == "descending":   # every tile beats the ones before it
+        X = X[np.argsort(-((X.astype(np.int64) - Q[0]) ** 2).sum(1), kind="stable")]
+        Q[:] = Q[0]
+    if kind == "graph":
+        ids, keys = ann.ann_build_knn_graph(dev(X), k)
+        want_ids, want_keys = oracle.exact_knn(X, X, k, exclude_self=True)
+    else:
+        ids, keys = ann.ann_exact_knn(dev(X), dev(Q), k)
+        want_ids, want_keys = oracle.exact_knn(X, Q, k)
+    np.testing.assert_array_equal(ids.cpu().numpy(), want_ids)
+    np.testing.assert_array_equal(ann.keys_as_uint32(keys).astype(np.float64),
+                                  np.where(np.isinf(want_keys), 4294967295.0, want_keys))
