@@ -152,6 +152,40 @@ __device__ __forceinline__ uint32_t part_key_lane<ANN_F32>(const uint8_t *qbytes
     return __float_as_uint(__fadd_rn(hi, lo));
 }
 
+// One part of a row against one center, 16 bytes per load (dp * element size a
+// multiple of 16); the operations and their order are part_key_lane's.
+template <int DT>
+__device__ __forceinline__ uint32_t part_key_wide(const uint8_t *qbytes, const void *C, int p, int c, int n, int dp) {
+    if (DT == ANN_U8) {
+        const uint4 *cent = (const uint4 *)((const uint8_t *)C + ((int64_t)p * n + c) * dp);
+        const uint4 *qp = (const uint4 *)(qbytes + p * dp);
+        uint32_t acc = 0;
+        for (int w = 0; w < dp / 16; w++) {
+            const uint4 a = qp[w], b = __ldg(cent + w);
+            uint32_t df = __vabsdiffu4(a.x, b.x);
+            acc = __dp4a(df, df, acc);
+            df = __vabsdiffu4(a.y, b.y);
+            acc = __dp4a(df, df, acc);
+            df = __vabsdiffu4(a.z, b.z);
+            acc = __dp4a(df, df, acc);
+            df = __vabsdiffu4(a.w, b.w);
+            acc = __dp4a(df, df, acc);
+        }
+        return acc;
+    }
+    const float4 *cent = (const float4 *)((const float *)C + ((int64_t)p * n + c) * dp);
+    const float4 *qp = (const float4 *)((const float *)qbytes + p * dp);
+    float hi = 0.f, lo = 0.f;
+    for (int w = 0; w < dp / 4; w++) {
+        const float4 a = qp[w], b = __ldg(cent + w);
+        df_acc_sqdiff(a.x, b.x, hi, lo);
+        df_acc_sqdiff(a.y, b.y, hi, lo);
+        df_acc_sqdiff(a.z, b.z, hi, lo);
+        df_acc_sqdiff(a.w, b.w, hi, lo);
+    }
+    return __float_as_uint(__fadd_rn(hi, lo));
+}
+
 // ---------------------------------------------------------------------------
 // bridge-key arithmetic (Sec. 4.2: the bridge key is the sum over parts of the
 // part keys).  uint8: exact integer sums.  float32: the key is the float32

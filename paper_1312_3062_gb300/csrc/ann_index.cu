@@ -373,40 +373,6 @@ __global__ void km_store_kernel(int total, int dtype, const double *C, void *out
 // 200,000 x 128 bytes, P = 4, n = 256, t = 100; this takes 5.3 ms.
 constexpr int BG_WARPS = 4;
 
-// One part of a row against one center, 16 bytes per load (dp * element size a
-// multiple of 16); the operations and their order are part_key_lane's.
-template <int DT>
-__device__ __forceinline__ uint32_t part_key_wide(const uint8_t *qbytes, const void *C, int p, int c, int n, int dp) {
-    if (DT == ANN_U8) {
-        const uint4 *cent = (const uint4 *)((const uint8_t *)C + ((int64_t)p * n + c) * dp);
-        const uint4 *qp = (const uint4 *)(qbytes + p * dp);
-        uint32_t acc = 0;
-        for (int w = 0; w < dp / 16; w++) {
-            const uint4 a = qp[w], b = __ldg(cent + w);
-            uint32_t df = __vabsdiffu4(a.x, b.x);
-            acc = __dp4a(df, df, acc);
-            df = __vabsdiffu4(a.y, b.y);
-            acc = __dp4a(df, df, acc);
-            df = __vabsdiffu4(a.z, b.z);
-            acc = __dp4a(df, df, acc);
-            df = __vabsdiffu4(a.w, b.w);
-            acc = __dp4a(df, df, acc);
-        }
-        return acc;
-    }
-    const float4 *cent = (const float4 *)((const float *)C + ((int64_t)p * n + c) * dp);
-    const float4 *qp = (const float4 *)((const float *)qbytes + p * dp);
-    float hi = 0.f, lo = 0.f;
-    for (int w = 0; w < dp / 4; w++) {
-        const float4 a = qp[w], b = __ldg(cent + w);
-        df_acc_sqdiff(a.x, b.x, hi, lo);
-        df_acc_sqdiff(a.y, b.y, hi, lo);
-        df_acc_sqdiff(a.z, b.z, hi, lo);
-        df_acc_sqdiff(a.w, b.w, hi, lo);
-    }
-    return __float_as_uint(__fadd_rn(hi, lo));
-}
-
 // sort part p's keys by (key, center id) in registers: the keys in rank order
 // over the unsorted ones, the center id at each rank
 template <int EPL, bool PACK>

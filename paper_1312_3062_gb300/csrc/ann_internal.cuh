@@ -126,10 +126,6 @@ struct ann_index {
 namespace ann {
 // implemented in ann_search.cu
 void free_plans(ann_index *ix);
-// plain launch of Algorithm 1 sized for a budget capT known on the host (no sync)
-int search_launch_plain(const ann_index *ix, const void *queries, int64_t nq, const int32_t *k, const int32_t *T,
-                        int32_t kmax, int capT, int32_t *out_ids, void *out_keys, int32_t *out_status,
-                        cudaStream_t stream);
 // plain launch over the queries listed in list[0 .. count) (device), sized for capT
 int search_launch_list(const ann_index *ix, const void *queries, int64_t nq, const int32_t *k, const int32_t *T,
                        int32_t kmax, int capT, const int32_t *list, int64_t count, int32_t *out_ids, void *out_keys,

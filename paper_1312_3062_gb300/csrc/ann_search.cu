@@ -43,164 +43,245 @@ static int device_props() {
 // slice of a query no longer grows with its budget.
 static const int kWindowedFromT = 1024;
 
-// Launch configuration for a budget bucket: warps per CTA and batch capacity.
+// Launch shape of the main loop for a budget bucket.
 struct Tune {
-    int warps;
-    int bcap;
-    bool stage;         // stage the next pop's neighbour vectors (cp.async)
-    bool tickets = true;  // persistent form: pull queries from a ticket (else a fixed grid-stride share)
+    int warps;                         // per CTA
+    bool stage;                        // stage the next pop's neighbour vectors (cp.async)
     int spill_heap = (int)kSpillHeap;  // large budgets: queue entries kept in shared memory
 };
-
-// Warps per CTA: the count that keeps the most warps resident per SM given
-// the per-warp shared-memory slice (ties go to more warps per CTA).
-static Tune choose_tune_heap(const DevIndex &ix, int capT, int kmax, int spill_heap) {
-    Tune t;
-    t.spill_heap = spill_heap;
-    // bridge batch: budgets below the windowed kernels pop few bridges
-    t.bcap = capT >= kWindowedFromT ? 128 : 64;
-    t.stage = true;
-    WarpLayout L = make_layout(ix.dtype, ix.d, ix.P, ix.n, ix.PA, capT, kmax, t.bcap, ix.b, ix.R, true,
-                               ix.ngroups > 0, capT >= kWindowedFromT, (uint32_t)t.spill_heap);
-    const size_t per_sm = 228 * 1024, per_cta_reserved = 1024;
-    size_t budget = g_smem_optin ? g_smem_optin : 227 * 1024;
-    // register-file limit of the kernel (both instantiations use the same budget)
-    static int regs = 0;
-    if (!regs) {
-        cudaFuncAttributes fa;
-        regs = cudaFuncGetAttributes(&fa, search_kernel<ANN_U8, false, false>) == cudaSuccess ? fa.numRegs : 168;
-        if (regs < 32) regs = 32;
-    }
-    const int warps_by_regs = 65536 / (regs * 32);
-    int best_w = 1, best_res = 0;
-    for (int w = 1; w <= 6; w++) {
-        size_t cta = (size_t)w * L.total;
-        if (cta > budget) break;
-        int ctas = (int)(per_sm / (cta + per_cta_reserved));
-        if (ctas > 32 / w) ctas = 32 / w;
-        if (ctas > warps_by_regs / w) ctas = warps_by_regs / w;
-        int res = ctas * w;
-        if (res >= best_res) {
-            best_res = res;
-            best_w = w;
-        }
-    }
-    t.warps = best_w;
-    return t;
-}
-
-static Tune choose_tune(const DevIndex &ix, int capT, int kmax) {
-    return choose_tune_heap(ix, capT, kmax, (int)kSpillHeap);
-}
-
 
 // The dynamic shared-memory limit of a kernel is a property of the function,
 // read again whenever a launch (or a graph node) is checked, so it is raised
 // once to the device's opt-in maximum rather than set per launch: a captured
 // graph may hold nodes of one kernel with different sizes.
-template <int DT, bool WIN>
-static cudaError_t config_kernel(size_t smem, int threads, int *blocks_per_sm) {
-    static bool raised = false;
+template <class F>
+static cudaError_t occupancy_of(F kernel, bool &raised, size_t smem, int threads, int *blocks_per_sm) {
     if (!raised) {
-        cudaError_t e = cudaFuncSetAttribute(search_kernel<DT, WIN, false>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g_smem_optin);
+        cudaError_t e =
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g_smem_optin);
         if (e != cudaSuccess) return e;
         raised = true;
     }
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, search_kernel<DT, WIN, false>, threads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kernel, threads, smem);
 }
 
-// Launch configuration of one search launch: layout, grid and the size of the
-// per-warp global scratch (windowed kernels only).
-struct LaunchCfg {
-    SearchArgs A;
+// main_kernel of a type, a layout and a register budget, as fn(kernel, index)
+template <class Fn>
+static auto with_main(int dtype, bool sp, bool wide, Fn fn) {
+    if (dtype == ANN_U8) {
+        if (sp && wide) return fn(main_kernel<ANN_U8, true, kMainCtasWide>, 0);
+        return sp ? fn(main_kernel<ANN_U8, true, kMainCtas>, 1) : fn(main_kernel<ANN_U8, false, kMainCtas>, 2);
+    }
+    return sp ? fn(main_kernel<ANN_F32, true, kMainCtas>, 3) : fn(main_kernel<ANN_F32, false, kMainCtas>, 4);
+}
+
+static cudaError_t main_occupancy(int dtype, bool sp, bool wide, size_t smem, int threads, int *blocks) {
+    static bool raised[5] = {};
+    return with_main(dtype, sp, wide,
+                     [&](auto kernel, int i) { return occupancy_of(kernel, raised[i], smem, threads, blocks); });
+}
+
+static cudaError_t resume_occupancy(const DevIndex &ix, bool sp, size_t smem, int threads, int *blocks) {
+    static bool raised[4] = {};
+    if (ix.ngroups > 0) return config_grouped(ix.dtype, sp, smem, threads, blocks);
+    if (ix.dtype == ANN_U8)
+        return sp ? occupancy_of(resume_kernel<ANN_U8, true, false>, raised[0], smem, threads, blocks)
+                  : occupancy_of(resume_kernel<ANN_U8, false, false>, raised[1], smem, threads, blocks);
+    return sp ? occupancy_of(resume_kernel<ANN_F32, true, false>, raised[2], smem, threads, blocks)
+              : occupancy_of(resume_kernel<ANN_F32, false, false>, raised[3], smem, threads, blocks);
+}
+
+static cudaError_t prologue_occupancy(const DevIndex &ix, size_t smem, int threads, int *blocks) {
+    static bool raised[2] = {};
+    if (ix.ngroups > 0) return config_grouped_prologue(ix.dtype, smem, threads, blocks);
+    return ix.dtype == ANN_U8 ? occupancy_of(prologue_kernel<ANN_U8, false>, raised[0], smem, threads, blocks)
+                              : occupancy_of(prologue_kernel<ANN_F32, false>, raised[1], smem, threads, blocks);
+}
+
+// one kernel of a search: its layout and launch shape
+struct Shape {
+    WarpLayout L;
     dim3 grid, block;
-    size_t smem;
-    bool win;
-    size_t scratch_bytes;
+    size_t smem = 0;
+    int warps = 0;  // resident warps at most
 };
 
-static int plan_launch(const SearchArgs &base, int capT, bool persistent, const int32_t *list,
-                       const int32_t *list_count, int64_t list_len, int32_t *ticket, LaunchCfg &cfg,
-                       const Tune *tune = nullptr) {
-    SearchArgs A = base;
-    A.capT = capT;
-    const Tune tn = tune ? *tune : choose_tune(A.ix, capT, A.kmax);
-    A.bcap = tn.bcap;
-    A.L = make_layout(A.ix.dtype, A.ix.d, A.ix.P, A.ix.n, A.ix.PA, capT, A.kmax, tn.bcap, A.ix.b, A.ix.R,
-                      tn.stage, A.ix.ngroups > 0, capT >= kWindowedFromT, (uint32_t)tn.spill_heap);
-    A.list = list;
-    A.list_count = list_count;
-    A.list_len = list_len;
-    A.ticket = (persistent && tn.tickets) ? ticket : nullptr;
-    const bool win = capT >= kWindowedFromT;
-    uint32_t gcap = (uint32_t)(2 * capT);
-    if (gcap > 8192) gcap = 8192;
-    A.gcap = win ? gcap : 0;
-    // per-warp scratch: windows, then the queue's overflow, then the visited set
-    auto al = [](uint64_t x) { return (x + 255) & ~(uint64_t)255; };
-    A.spill_off = win ? al((uint64_t)gcap * 24) : 0;
-    A.hash_off = win ? A.spill_off + al(8ull * (uint64_t)capT) : 0;
-    A.wstride = win ? A.hash_off + al(4ull << A.L.hash_log) : 0;
-    size_t smem = (size_t)A.L.total * tn.warps;
-    if (smem > g_smem_optin) return fail(ANN_ERR_CAPACITY, "per-query state exceeds shared memory");
-    int blocks_per_sm = 0;
-    const int threads = tn.warps * 32;
-    cudaError_t e;
-    if (A.ix.ngroups > 0)
-        e = config_grouped(A.ix.dtype, win, smem, threads, &blocks_per_sm);
-    else if (A.ix.dtype == ANN_U8)
-        e = win ? config_kernel<ANN_U8, true>(smem, threads, &blocks_per_sm)
-                : config_kernel<ANN_U8, false>(smem, threads, &blocks_per_sm);
-    else
-        e = win ? config_kernel<ANN_F32, true>(smem, threads, &blocks_per_sm)
-                : config_kernel<ANN_F32, false>(smem, threads, &blocks_per_sm);
-    if (e != cudaSuccess) return cuda_fail(e, "search kernel configuration");
-    if (blocks_per_sm < 1) blocks_per_sm = 1;
-    const int64_t cap = (int64_t)g_num_sms * blocks_per_sm;
-    // ticket queue: one wave; fixed shares: up to four waves, sized by the
-    // query count when it is known on the host
-    const bool by_ticket = persistent && ticket && tn.tickets;
-    int64_t want = by_ticket ? cap : (list_count ? cap * 4 : (list_len + tn.warps - 1) / tn.warps);
-    // plain launches grid-stride beyond four waves; windowed ones beyond one wave (bounded scratch)
-    const int64_t lim = win ? cap : cap * 4;
-    if (want > lim) want = lim;
-    if (want < 1) want = 1;
-    cfg.A = A;
-    cfg.grid = dim3((unsigned)want);
-    cfg.block = dim3(threads);
-    cfg.smem = smem;
-    cfg.win = win;
-    cfg.scratch_bytes = win ? (size_t)want * tn.warps * A.wstride : 0;
+// The shape that keeps the most warps resident for slices of L.total bytes
+// (ties go to more warps per CTA), for `count` queries at most: few queries
+// spread over the SMs one warp to a CTA.  waves > 1: more CTAs than fit.
+template <class Occ>
+static int fit_shape(Shape &sh, int max_warps, int64_t count, int waves, Occ occ) {
+    if (sh.L.total > g_smem_optin) return fail(ANN_ERR_CAPACITY, "per-query state exceeds shared memory");
+    const int64_t spread = (count + g_num_sms - 1) / g_num_sms;
+    if (max_warps > spread) max_warps = (int)std::max<int64_t>(1, spread);
+    int best = 0, best_w = 1, best_blocks = 1;
+    for (int w = 1; w <= max_warps; w++) {
+        const size_t smem = (size_t)w * sh.L.total;
+        if (smem > g_smem_optin) break;
+        int blocks = 0;
+        const cudaError_t e = occ(smem, 32 * w, &blocks);
+        if (e != cudaSuccess) return cuda_fail(e, "search kernel configuration");
+        if (blocks * w >= best) {
+            best = blocks * w;
+            best_w = w;
+            best_blocks = std::max(1, blocks);
+        }
+    }
+    int64_t grid = std::min<int64_t>((count + best_w - 1) / best_w, (int64_t)g_num_sms * best_blocks * waves);
+    if (grid < 1) grid = 1;
+    sh.grid = dim3((unsigned)grid);
+    sh.block = dim3(32 * best_w);
+    sh.smem = (size_t)best_w * sh.L.total;
+    sh.warps = (int)std::min<int64_t>(grid, (int64_t)g_num_sms * best_blocks) * best_w;
     return ANN_OK;
 }
 
-static int do_launch(LaunchCfg &cfg, uint8_t *scratch, cudaStream_t stream) {
-    cfg.A.gscratch = scratch;
-    if (cfg.A.ix.ngroups > 0) {
-        launch_grouped(cfg.A.ix.dtype, cfg.win, cfg.grid, cfg.block, cfg.smem, stream, cfg.A);
-    } else if (cfg.A.ix.dtype == ANN_U8) {
-        if (cfg.win) search_kernel<ANN_U8, true, false><<<cfg.grid, cfg.block, cfg.smem, stream>>>(cfg.A);
-        else search_kernel<ANN_U8, false, false><<<cfg.grid, cfg.block, cfg.smem, stream>>>(cfg.A);
-    } else {
-        if (cfg.win) search_kernel<ANN_F32, true, false><<<cfg.grid, cfg.block, cfg.smem, stream>>>(cfg.A);
-        else search_kernel<ANN_F32, false, false><<<cfg.grid, cfg.block, cfg.smem, stream>>>(cfg.A);
+// Launch configuration of one search: its three kernels and their workspace.
+struct LaunchCfg {
+    SearchArgs A;
+    Shape pro, main, res;
+    uint64_t main_stride, res_stride;  // global scratch per warp (large budgets)
+    uint64_t main_spill, main_hash, res_spill, res_hash;
+    bool win, wide;
+    int64_t total, chunk;              // queries, and queries per pass over the three kernels
+    // offsets into the workspace
+    size_t o_rec, o_bk, o_bi, o_susp, o_save, o_scratch, bytes;
+};
+
+// A pass holds the records and first bridge batches of at most kChunk queries
+// (0.9 to 1.7 KB each), and states of suspended ones up to kSaveBytes; queries
+// that find no room there start again when they are resumed.
+static const int64_t kChunk = 65536;
+static const size_t kSaveBytes = (size_t)256 << 20;
+
+static int plan_launch(const SearchArgs &base, int capT, const int32_t *list, const int32_t *list_count,
+                       int64_t list_len, LaunchCfg &cfg, const Tune *tune = nullptr) {
+    SearchArgs A = base;
+    const DevIndex &ix = A.ix;
+    const bool win = capT >= kWindowedFromT, grouped = ix.ngroups > 0;
+    const Tune tn = tune ? *tune : Tune{kMainWarps, true, (int)kSpillHeap};
+    A.capT = capT;
+    // bridge batch: budgets below the windowed kernels pop few bridges
+    A.bcap = win ? 128 : 64;
+    A.bstore = A.bcap + (int)kFirstBridges;
+    A.list = list;
+    A.list_count = list_count;
+    A.list_len = list_len;
+    cfg.win = win;
+    cfg.wide = list_len > (int64_t)g_num_sms * kMainWarps * kMainCtas;
+    cfg.total = list_len;
+    cfg.chunk = std::min(list_len, kChunk);
+    cfg.pro.L = prologue_layout(ix.dtype, ix.d, ix.P, ix.n, ix.PA, A.bcap, grouped, win);
+    cfg.main.L = main_layout(ix.dtype, ix.d, capT, A.kmax, ix.b, ix.R, tn.stage, win, (uint32_t)tn.spill_heap);
+    cfg.res.L = make_layout(ix.dtype, ix.d, ix.P, ix.n, ix.PA, capT, A.kmax, A.bcap, ix.b, ix.R, true, grouped, win,
+                            (uint32_t)tn.spill_heap, true);
+    int r = fit_shape(cfg.pro, 4, cfg.chunk, 8, [&](size_t smem, int threads, int *blocks) {
+        return prologue_occupancy(ix, smem, threads, blocks);
+    });
+    if (r == ANN_OK)
+        r = fit_shape(cfg.main, tn.warps, cfg.chunk, 1, [&](size_t smem, int threads, int *blocks) {
+            return main_occupancy(ix.dtype, win, cfg.wide, smem, threads, blocks);
+        });
+    if (r == ANN_OK)
+        r = fit_shape(cfg.res, 6, cfg.chunk, 1, [&](size_t smem, int threads, int *blocks) {
+            return resume_occupancy(ix, win, smem, threads, blocks);
+        });
+    if (r != ANN_OK) return r;
+    auto al = [](uint64_t x) { return (x + 255) & ~(uint64_t)255; };
+    // a sorted window serves many batches of bridges
+    const uint32_t gcap = (uint32_t)std::min(8192, std::max(1024, 2 * capT));
+    A.gcap = gcap;
+    // per-warp scratch: the queue's overflow, then the visited set; the
+    // resuming kernel's starts with its sorted bridge windows
+    const uint64_t spill = al(8ull * (uint64_t)capT), hash = al(4ull << cfg.main.L.hash_log);
+    cfg.main_spill = 0;
+    cfg.main_hash = spill;
+    cfg.main_stride = win ? spill + hash : 0;
+    cfg.res_spill = al((uint64_t)gcap * 24);
+    cfg.res_hash = cfg.res_spill + spill;
+    cfg.res_stride = win ? cfg.res_hash + hash : cfg.res_spill;
+    // a suspended query's state
+    A.save_rbuf = kSaveHeader;
+    A.save_heap = A.save_rbuf + (A.kmax > 32 ? 8u * (uint32_t)A.kmax : 0u);
+    A.save_hash = align_up(A.save_heap + 8u * cfg.main.L.heap_cap, 16);
+    A.save_spill = A.save_hash + (4u << cfg.main.L.hash_log);
+    A.save_stride = al(A.save_spill + (win ? 8ull * (uint64_t)capT : 0ull));
+    A.nslots = (uint32_t)std::min<int64_t>(cfg.chunk, (int64_t)(kSaveBytes / A.save_stride));
+    size_t o = 256;  // counters
+    cfg.o_rec = o;   o = al(o + sizeof(QRec) * (size_t)cfg.chunk);
+    cfg.o_bk = o;    o = al(o + 8 * (size_t)A.bstore * cfg.chunk);
+    cfg.o_bi = o;    o = al(o + 4 * (size_t)A.bstore * cfg.chunk);
+    cfg.o_susp = o;  o = al(o + 4 * (size_t)cfg.chunk);
+    cfg.o_save = o;  o = al(o + (size_t)A.nslots * A.save_stride);
+    cfg.o_scratch = o;
+    o = al(o + std::max(cfg.main.warps * cfg.main_stride, cfg.res.warps * cfg.res_stride));
+    cfg.bytes = o;
+    cfg.A = A;
+    return ANN_OK;
+}
+
+// the three kernels of passes over the queries; stages: how many of them to launch (3 = all)
+static int do_launch(LaunchCfg &cfg, uint8_t *ws, cudaStream_t stream, int first = 0, int last = 2) {
+    SearchArgs &A = cfg.A;
+    const bool u8 = A.ix.dtype == ANN_U8, grouped = A.ix.ngroups > 0;
+    A.counters = (int32_t *)ws;
+    A.rec = (QRec *)(ws + cfg.o_rec);
+    A.bkeys = (uint64_t *)(ws + cfg.o_bk);
+    A.bidxs = (uint32_t *)(ws + cfg.o_bi);
+    A.susp = (int32_t *)(ws + cfg.o_susp);
+    A.save = ws + cfg.o_save;
+    A.gscratch = ws + cfg.o_scratch;
+    A.chunk = cfg.chunk;
+    for (A.base = 0; A.base < cfg.total; A.base += cfg.chunk) {
+        if (first <= 0) {
+            const Shape &s = cfg.pro;
+            A.L = s.L;
+            if (grouped) launch_grouped_prologue(A.ix.dtype, s.grid, s.block, s.smem, stream, A);
+            else if (u8) prologue_kernel<ANN_U8, false><<<s.grid, s.block, s.smem, stream>>>(A);
+            else prologue_kernel<ANN_F32, false><<<s.grid, s.block, s.smem, stream>>>(A);
+        }
+        if (first <= 1 && last >= 1) {
+            const Shape &s = cfg.main;
+            A.L = s.L;
+            A.spill_off = cfg.main_spill;
+            A.hash_off = cfg.main_hash;
+            A.wstride = cfg.main_stride;
+            with_main(A.ix.dtype, cfg.win, cfg.wide, [&](auto kernel, int) {
+                kernel<<<s.grid, s.block, s.smem, stream>>>(A);
+                return 0;
+            });
+        }
+        if (last >= 2) {
+            const Shape &s = cfg.res;
+            A.L = s.L;
+            A.spill_off = cfg.res_spill;
+            A.hash_off = cfg.res_hash;
+            A.wstride = cfg.res_stride;
+            if (grouped) {
+                launch_grouped(A.ix.dtype, cfg.win, s.grid, s.block, s.smem, stream, A);
+            } else if (u8) {
+                if (cfg.win) resume_kernel<ANN_U8, true, false><<<s.grid, s.block, s.smem, stream>>>(A);
+                else resume_kernel<ANN_U8, false, false><<<s.grid, s.block, s.smem, stream>>>(A);
+            } else {
+                if (cfg.win) resume_kernel<ANN_F32, true, false><<<s.grid, s.block, s.smem, stream>>>(A);
+                else resume_kernel<ANN_F32, false, false><<<s.grid, s.block, s.smem, stream>>>(A);
+            }
+        }
     }
     ANN_CUDA(cudaGetLastError());
     return ANN_OK;
 }
 
-// plan + stream-ordered scratch (windowed kernels) + launch
-static int launch_search(const SearchArgs &base, int capT, cudaStream_t stream, bool persistent,
-                         const int32_t *list, const int32_t *list_count, int64_t list_len,
-                         int32_t *ticket) {
+// plan + stream-ordered workspace + launch
+static int launch_search(const SearchArgs &base, int capT, cudaStream_t stream, const int32_t *list,
+                         int64_t list_len) {
     LaunchCfg cfg;
-    int r = plan_launch(base, capT, persistent, list, list_count, list_len, ticket, cfg);
+    int r = plan_launch(base, capT, list, nullptr, list_len, cfg);
     if (r != ANN_OK) return r;
-    uint8_t *scratch = nullptr;
-    if (cfg.scratch_bytes) ANN_CUDA(cudaMallocAsync((void **)&scratch, cfg.scratch_bytes, stream));
-    r = do_launch(cfg, scratch, stream);
-    if (scratch) cudaFreeAsync(scratch, stream);
+    uint8_t *ws = nullptr;
+    ANN_CUDA(cudaMallocAsync((void **)&ws, cfg.bytes, stream));
+    r = do_launch(cfg, ws, stream);
+    cudaFreeAsync(ws, stream);
     return r;
 }
 
@@ -212,8 +293,7 @@ __global__ void max_kernel(const int32_t *v, int64_t n, int32_t *out) {
 // ---- persistent mode: bucket queries by budget on the device ----
 static const int kBuckets = 7;  // capT = 128 << i  (128 .. 8192)
 
-__global__ void bucket_kernel(int64_t nq, const int32_t *T, int32_t T_all, int32_t *counts,
-                              int32_t *lists, int32_t *tickets) {
+__global__ void bucket_kernel(int64_t nq, const int32_t *T, int32_t T_all, int32_t *counts, int32_t *lists) {
     // counts[kBuckets], lists[kBuckets * nq]
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nq) return;
@@ -226,8 +306,8 @@ __global__ void bucket_kernel(int64_t nq, const int32_t *T, int32_t T_all, int32
 
 struct Plan {
     cudaGraphExec_t exec = nullptr;
-    int32_t *scratch = nullptr;   // counts[kBuckets] + tickets[kBuckets] + lists[kBuckets*nq]
-    uint8_t *wscratch = nullptr;  // per-warp sorted bridge windows (largest windowed bucket's need)
+    int32_t *scratch = nullptr;   // counts[kBuckets], then lists[kBuckets*nq]
+    uint8_t *wscratch = nullptr;  // the buckets' workspaces, one after another
     uint64_t last_use = 0;        // for evicting the least recently used plan
 };
 
@@ -288,11 +368,10 @@ static const Tune *tuned_for(const PlanCache *pc, int capT, int kmax) {
 static int bucket_cap(int bkt) { return (128 << bkt) > kMaxT ? kMaxT : (128 << bkt); }
 
 // One replay of the persistent form.  A uniform budget is one bucket and the
-// queries are taken in order; otherwise a device pass sorts them into
-// buckets first.  Every bucket's kernel pulls its queries from a ticket.
-// Buckets without global scratch run concurrently on forked streams (largest
-// budget first), so the smaller ones fill the SMs the larger leave idle at
-// their tail; windowed buckets share one scratch and run one after another.
+// queries are taken in order; otherwise a device pass sorts them into buckets
+// first.  The buckets run concurrently on forked streams (largest budget
+// first), each with a workspace of its own: a bucket's last queries leave most
+// SMs idle, above all those that pop many bridges.
 // streams and events of the fork/join; they must outlive the capture
 struct ForkSet {
     cudaStream_t side[kBuckets] = {};
@@ -309,10 +388,10 @@ struct ForkSet {
 
 static int record_persistent(const PlanCache *pc, const SearchArgs &A, int64_t nq, const int32_t *T, int32_t T_all,
                              int32_t *scratch, uint8_t *wscratch, cudaStream_t s, ForkSet &fs) {
-    int32_t *counts = scratch, *tickets = scratch + kBuckets, *lists = scratch + 2 * kBuckets;
-    ANN_CUDA(cudaMemsetAsync(scratch, 0, sizeof(int32_t) * 2 * kBuckets, s));
+    int32_t *counts = scratch, *lists = scratch + kBuckets;
     if (T) {
-        bucket_kernel<<<(unsigned)((nq + 255) / 256), 256, 0, s>>>(nq, T, T_all, counts, lists, tickets);
+        ANN_CUDA(cudaMemsetAsync(counts, 0, sizeof(int32_t) * kBuckets, s));
+        bucket_kernel<<<(unsigned)((nq + 255) / 256), 256, 0, s>>>(nq, T, T_all, counts, lists);
         ANN_CUDA(cudaGetLastError());
     }
     int b0, b1;
@@ -321,12 +400,13 @@ static int record_persistent(const PlanCache *pc, const SearchArgs &A, int64_t n
     for (int bkt = b1; bkt >= b0 && rc == ANN_OK; bkt--) {
         const int capT = bucket_cap(bkt);
         LaunchCfg cfg;
-        rc = T ? plan_launch(A, capT, true, lists + (int64_t)bkt * nq, counts + bkt, nq, tickets + bkt, cfg,
-                             tuned_for(pc, capT, A.kmax))
-               : plan_launch(A, capT, true, nullptr, nullptr, nq, tickets + bkt, cfg, tuned_for(pc, capT, A.kmax));
+        rc = T ? plan_launch(A, capT, lists + (int64_t)bkt * nq, counts + bkt, nq, cfg, tuned_for(pc, capT, A.kmax))
+               : plan_launch(A, capT, nullptr, nullptr, nq, cfg, tuned_for(pc, capT, A.kmax));
         if (rc != ANN_OK) break;
-        if (cfg.win || b0 == b1) {
-            rc = do_launch(cfg, wscratch, s);
+        uint8_t *ws = wscratch;
+        wscratch += cfg.bytes;
+        if (b0 == b1) {
+            rc = do_launch(cfg, ws, s);
             continue;
         }
         if (!fs.fork) {
@@ -347,7 +427,7 @@ static int record_persistent(const PlanCache *pc, const SearchArgs &A, int64_t n
             rc = cuda_fail(cudaGetLastError(), "fork");
             break;
         }
-        rc = do_launch(cfg, nullptr, fs.side[i]);
+        rc = do_launch(cfg, ws, fs.side[i]);
         if (rc != ANN_OK) break;
         if (cudaEventRecord(fs.join[i], fs.side[i]) != cudaSuccess || cudaStreamWaitEvent(s, fs.join[i], 0) != cudaSuccess) {
             rc = cuda_fail(cudaGetLastError(), "join");
@@ -357,28 +437,16 @@ static int record_persistent(const PlanCache *pc, const SearchArgs &A, int64_t n
     return rc;
 }
 
-// Launch shapes worth measuring for a bucket: the analytic choice, fewer warps
-// per CTA (finer CTA granularity, fewer registers per SM in use), the
-// analytic choice without cp.async staging, with fixed shares instead of the
-// ticket, and, for large budgets, other shared-memory heap capacities (a
+// Launch shapes of the main loop worth measuring for a bucket: as many warps
+// per CTA as the kernel takes, fewer (finer granularity), without cp.async
+// staging, and, for large budgets, other shared-memory heap capacities (a
 // smaller heap leaves room for more resident queries, a larger one moves
 // entries out less often).  All give identical results.
-static std::vector<Tune> tune_candidates(const DevIndex &ix, int capT, int kmax) {
-    const Tune d = choose_tune(ix, capT, kmax);
-    std::vector<Tune> c{d};
-    for (int w : {1, 2, 3, 4})
-        if (w < d.warps) c.push_back(Tune{w, d.bcap, true, true});
-    c.push_back(Tune{d.warps, d.bcap, false, true});
-    c.push_back(Tune{d.warps, d.bcap, true, false});  // the plain form's fixed grid-stride shares
+static std::vector<Tune> tune_candidates(int capT) {
+    std::vector<Tune> c{Tune{kMainWarps, true}, Tune{kMainWarps / 2, true}, Tune{kMainWarps, false}};
     if (capT >= kWindowedFromT)
-        for (int hc : {256, 1024, 2048})
-            if (hc < capT) {
-                Tune t = d;
-                t.spill_heap = hc;
-                Tune a = choose_tune_heap(ix, capT, kmax, hc);
-                t.warps = a.warps;
-                c.push_back(t);
-            }
+        for (int hc : {256, 1024})
+            if (hc < capT) c.push_back(Tune{kMainWarps, true, hc});
     return c;
 }
 
@@ -391,12 +459,11 @@ static int autotune(PlanCache *pc, const SearchArgs &A, int64_t nq, const int32_
     bool todo = false;
     for (int bkt = b0; bkt <= b1; bkt++) todo |= tuned_for(pc, bucket_cap(bkt), A.kmax) == nullptr;
     if (!todo) return ANN_OK;
-    int32_t *counts = scratch, *tickets = scratch + kBuckets, *lists = scratch + 2 * kBuckets;
-    int32_t *tcount = scratch + kBuckets * (2 + nq);  // one extra word: queries per tuning run
-    ANN_CUDA(cudaMemsetAsync(scratch, 0, sizeof(int32_t) * 2 * kBuckets, s));
+    int32_t *counts = scratch, *lists = scratch + kBuckets;
     int32_t hc[kBuckets] = {0};
     if (T) {
-        bucket_kernel<<<(unsigned)((nq + 255) / 256), 256, 0, s>>>(nq, T, T_all, counts, lists, tickets);
+        ANN_CUDA(cudaMemsetAsync(counts, 0, sizeof(int32_t) * kBuckets, s));
+        bucket_kernel<<<(unsigned)((nq + 255) / 256), 256, 0, s>>>(nq, T, T_all, counts, lists);
         ANN_CUDA(cudaGetLastError());
         ANN_CUDA(cudaMemcpyAsync(hc, counts, sizeof(hc), cudaMemcpyDeviceToHost, s));
         ANN_CUDA(cudaStreamSynchronize(s));
@@ -410,29 +477,26 @@ static int autotune(PlanCache *pc, const SearchArgs &A, int64_t nq, const int32_
     for (int bkt = b0; bkt <= b1 && rc == ANN_OK; bkt++) {
         const int capT = bucket_cap(bkt);
         if (tuned_for(pc, capT, A.kmax) || hc[bkt] == 0) continue;
-        const std::vector<Tune> cands = tune_candidates(A.ix, capT, A.kmax);
+        const std::vector<Tune> cands = tune_candidates(capT);
+        const int32_t *list = T ? lists + (int64_t)bkt * nq : nullptr;
         // tune on up to four rounds of the default shape's resident warps
         LaunchCfg c0;
-        rc = plan_launch(A, capT, true, nullptr, nullptr, nq, tickets + bkt, c0, &cands[0]);
+        rc = plan_launch(A, capT, list, nullptr, hc[bkt], c0, &cands[0]);
         if (rc != ANN_OK) break;
-        const int64_t resident = (int64_t)c0.grid.x * (c0.block.x / 32);
-        const int32_t ntune = (int32_t)std::min<int64_t>(hc[bkt], 4 * resident);
-        ANN_CUDA(cudaMemcpyAsync(tcount, &ntune, sizeof(int32_t), cudaMemcpyHostToDevice, s));
-        const int32_t *list = T ? lists + (int64_t)bkt * nq : nullptr;
+        const int64_t ntune = std::min<int64_t>(std::min<int64_t>(hc[bkt], kChunk), 4 * (int64_t)c0.main.warps);
         float best_ms = 0.f;
         int best = -1;
         for (size_t ci = 0; ci < cands.size() && rc == ANN_OK; ci++) {
+            LaunchCfg cfg;
+            if (plan_launch(A, capT, list, nullptr, ntune, cfg, &cands[ci]) != ANN_OK) continue;
+            uint8_t *ws = nullptr;
+            if (cudaMallocAsync((void **)&ws, cfg.bytes, s) != cudaSuccess) continue;
             float ms_min = 0.f;
-            for (int rep = 0; rep < 2; rep++) {
-                LaunchCfg cfg;
-                if (plan_launch(A, capT, true, list, tcount, nq, tickets + bkt, cfg, &cands[ci]) != ANN_OK) break;
-                uint8_t *ws = nullptr;
-                if (cfg.scratch_bytes && cudaMallocAsync((void **)&ws, cfg.scratch_bytes, s) != cudaSuccess) break;
-                cudaMemsetAsync(tickets + bkt, 0, sizeof(int32_t), s);
+            for (int rep = 0; rep < 2 && rc == ANN_OK; rep++) {
+                rc = do_launch(cfg, ws, s, 0, 0);
                 cudaEventRecord(e0, s);
-                rc = do_launch(cfg, ws, s);
+                if (rc == ANN_OK) rc = do_launch(cfg, ws, s, 1, 1);
                 cudaEventRecord(e1, s);
-                if (ws) cudaFreeAsync(ws, s);
                 if (rc != ANN_OK) break;
                 cudaError_t ce = cudaEventSynchronize(e1);
                 if (ce != cudaSuccess) {
@@ -444,6 +508,7 @@ static int autotune(PlanCache *pc, const SearchArgs &A, int64_t nq, const int32_
                 if (rep == 0 || ms < ms_min) ms_min = ms;
                 if (ms > 50.f) break;  // long runs: one measurement is enough
             }
+            cudaFreeAsync(ws, s);
             if (rc == ANN_OK && ms_min > 0.f && (best < 0 || ms_min < best_ms)) {
                 best_ms = ms_min;
                 best = (int)ci;
@@ -455,27 +520,6 @@ static int autotune(PlanCache *pc, const SearchArgs &A, int64_t nq, const int32_
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     return rc;
-}
-
-int search_launch_plain(const ann_index *ix, const void *queries, int64_t nq, const int32_t *k, const int32_t *T,
-                        int32_t kmax, int capT, int32_t *out_ids, void *out_keys, int32_t *out_status,
-                        cudaStream_t stream) {
-    int r = device_props();
-    if (r != ANN_OK) return r;
-    if (nq == 0) return ANN_OK;
-    SearchArgs A{};
-    A.ix = ix->dev;
-    A.queries = queries;
-    A.nq = nq;
-    A.k = k;
-    A.T = T;
-    A.kmax = kmax;
-    A.out_ids = out_ids;
-    A.out_keys = out_keys;
-    A.out_status = out_status;
-    if (capT > kMaxT) capT = kMaxT;
-    if (capT < 32) capT = 32;
-    return launch_search(A, capT, stream, false, nullptr, nullptr, nq, nullptr);
 }
 
 int search_launch_list(const ann_index *ix, const void *queries, int64_t nq, const int32_t *k, const int32_t *T,
@@ -496,7 +540,7 @@ int search_launch_list(const ann_index *ix, const void *queries, int64_t nq, con
     A.out_status = out_status;
     if (capT > kMaxT) capT = kMaxT;
     if (capT < 32) capT = 32;
-    return launch_search(A, capT, stream, false, list, nullptr, count, nullptr);
+    return launch_search(A, capT, stream, list, count);
 }
 
 int search_bucket_of(int32_t T) {
@@ -557,7 +601,7 @@ extern "C" int ann_search_batch(const ann_index *index, const void *queries, int
         }
         if (capT > kMaxT) capT = kMaxT;
         if (capT < 32) capT = 32;
-        return launch_search(A, capT, s, false, nullptr, nullptr, nq, nullptr);
+        return launch_search(A, capT, s, nullptr, nq);
     }
     // persistent: bucket by budget, one persistent kernel per bucket, replayed as a CUDA graph
     ann_index *ixm = const_cast<ann_index *>(index);
@@ -579,7 +623,7 @@ extern "C" int ann_search_batch(const ann_index *index, const void *queries, int
     }
     if (it == pc->plans.end()) {
         Plan p;
-        ANN_CUDA(cudaMalloc(&p.scratch, sizeof(int32_t) * (2 * kBuckets + (size_t)kBuckets * nq + 1)));
+        ANN_CUDA(cudaMalloc(&p.scratch, sizeof(int32_t) * (kBuckets + (size_t)kBuckets * nq)));
         {
             int r = autotune(pc, A, nq, T, T_all, p.scratch, s);
             if (r != ANN_OK) {
@@ -591,13 +635,12 @@ extern "C" int ann_search_batch(const ann_index *index, const void *queries, int
             bucket_range(T, T_all, b0, b1);
             for (int bkt = b0; bkt <= b1; bkt++) {
                 LaunchCfg cfg;
-                r = plan_launch(A, bucket_cap(bkt), true, nullptr, p.scratch, nq, p.scratch, cfg,
-                                tuned_for(pc, bucket_cap(bkt), kmax));
+                r = plan_launch(A, bucket_cap(bkt), nullptr, p.scratch, nq, cfg, tuned_for(pc, bucket_cap(bkt), kmax));
                 if (r != ANN_OK) {
                     cudaFree(p.scratch);
                     return r;
                 }
-                need = cfg.scratch_bytes > need ? cfg.scratch_bytes : need;
+                need += cfg.bytes;
             }
             if (need) {
                 cudaError_t ae = cudaMalloc(&p.wscratch, need);

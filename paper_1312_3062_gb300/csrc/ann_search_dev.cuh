@@ -1,12 +1,29 @@
 // ann_search_dev.cuh -- device code of Algorithm 1 (Sec. 4.2) of arXiv:1312.3062
 // on sm_103a, shared by the translation units that instantiate its kernels.
 //
-// One warp runs one query from start to finish:
-//   1. part tables  D_p[c] = ||q^p - c_p||^2           (Sec. 4.2, first step)
-//   2. per-part sort by (key, center id) -> ranks        (Sec. 4.2)
-//   3. the main loop of Algorithm 1: a shared min-queue of reference vectors
-//      and the current bridge vector, the visited set (Color), the result set
-//      R and the exact budget T.
+// One warp runs one query, in up to three kernels:
+//   prologue_kernel  1. part tables  D_p[c] = ||q^p - c_p||^2  (Sec. 4.2, first step)
+//                    2. per-part sort by (key, center id) -> ranks  (Sec. 4.2)
+//                    3. the first batch of bridge vectors (a walk)
+//   main_kernel      the main loop of Algorithm 1: a shared min-queue of
+//                    reference vectors and the current bridge vector, the
+//                    visited set (Color), the result set R and the exact budget
+//                    T.  A query that has popped its whole first batch of
+//                    bridges is suspended.
+//   resume_kernel    suspended queries: tables and sort again, then the same
+//                    loop with further walks, to the end.
+// Why three: the loop is a chain of dependent steps (a warp collective takes
+// 30 to 40 cycles here, and a popped reference about 20 of them in a row), so
+// its rate is set by how many queries an SM holds.  With the walk in the same
+// kernel a query took 168 registers and, for its tables and walk lists, about
+// 8 KB more shared memory: 12 queries per SM.  Most queries need only the
+// first batch (21 of 10,000 are suspended at T = 371 on SIFT-shaped rows); the
+// loop alone holds 16 to 24 queries per SM.  And the resuming kernel, which
+// only sees queries that pop many bridges, sorts whole windows of bridges at
+// every budget.  One kernel against three, 10,000 queries, 1M SIFT-shaped rows:
+// T = 371 1.31 -> 0.92 ms, T = 2392 8.06 -> 6.06 ms; 2,000 GIST-shaped queries
+// with budgets of 64 to 8192 57.8 -> 29.6 ms; 1,792 queries of T = 339 among
+// 170-point components, which pop bridges all the time, 4.78 -> 2.56 ms.
 // Bridge vectors are produced in the order of the multi-sequence algorithm
 // (Sec. 3.3): ascending (bridge key, rank tuple).  A popped bridge vector
 // with an empty list discovers nothing and only makes the next one current,
@@ -43,8 +60,7 @@ namespace ann {
 // shared-memory layout of one warp
 // ---------------------------------------------------------------------------
 struct WarpLayout {
-    uint32_t q, tabD, rank, sk, sc, heap, hash, rbuf, bkey, bidx, pref, nodes, cand, ckey, wref, wkey, stage, misc,
-        total;
+    uint32_t q, tabD, rank, sc, heap, hash, rbuf, bkey, bidx, pref, nodes, cand, ckey, wref, wkey, stage, misc, stat, total;
     uint32_t heap_cap, hash_log, bcap, ncap, gcap, glist, stage_rows, stage_stride;
     uint32_t sc_parts;  // parts whose centers are kept in rank order (all of them when split walks may run)
 };
@@ -59,22 +75,29 @@ constexpr uint32_t kStageBytes = 4096;
 // so a query's shared-memory slice does not grow with the budget.
 constexpr uint32_t kSpillHeap = 512;
 
+// main_kernel: warps per CTA at most, and how many CTAs of that size an SM's
+// registers hold.  16 queries per SM (128 registers) is the faster shape until
+// the queries of a launch fill it; large-budget uint8 launches beyond that take
+// 24 (80 registers, with spills).  10,000 queries, SIFT-shaped 1M rows,
+// 16 / 20 / 24 per SM: T = 371 0.91 / 0.92 / 1.02 ms, T = 2392 6.67 / 6.43 /
+// 6.13 ms; the served burst, about 1000 queries per budget, 5.24 / 5.52 / 5.83 ms.
+constexpr int kMainWarps = 4, kMainCtas = 4, kMainCtasWide = 6;
+
 __host__ __device__ inline uint32_t align_up(uint32_t x, uint32_t a) { return (x + a - 1) / a * a; }
 
+// the layout of resume_kernel: everything
 __host__ __device__ inline WarpLayout make_layout(int dtype, int d, int P, int n, int PA, int capT,
                                                   int kmax, int bcap, int b, int R, bool stage = true,
                                                   bool grouped = false, bool spill = false,
-                                                  uint32_t spill_heap = kSpillHeap) {
+                                                  uint32_t spill_heap = kSpillHeap, bool split = false) {
     WarpLayout L;
     uint32_t o = 0;
     L.q = o;      o = align_up(o + (uint32_t)d * (dtype == ANN_U8 ? 1u : 4u), 16);
     L.tabD = o;   o = align_up(o + 4u * P * n, 16);
     L.rank = o;   o = align_up(o + (uint32_t)P * n, 16);
-    L.sk = 0;     // sorted keys are read as D[sc[r]]
-    // center id at each rank: the prefix parts, and with the large-budget
-    // layout every part (the suffix pass of a split walk reads them); below
-    // it the extra bytes would cost a resident query per SM
-    L.sc_parts = spill ? (uint32_t)P : (uint32_t)PA;
+    // center id at each rank: the prefix parts, and where split walks run every
+    // part (their suffix pass reads them)
+    L.sc_parts = spill || split ? (uint32_t)P : (uint32_t)PA;
     L.sc = o;     o = align_up(o + L.sc_parts * n, 16);
     uint32_t lpn = 1;
     while (lpn < (uint32_t)n) lpn <<= 1;  // the per-part sort borrows the heap region
@@ -119,10 +142,67 @@ __host__ __device__ inline WarpLayout make_layout(int dtype, int d, int P, int n
     L.wkey = o + align_up(4u * wb, 16);
     L.stage = o;
     o = align_up(o + ub, 16);
-    L.misc = o;   o = align_up(o + 16u * 4, 16);  // [0] emit count, [3] min suffix, [4] min last part, [8..10] walk counters
+    // [0] emit count, [3] min suffix, [4] min last part, [8..10] walk counters, [12..15] the query's counters
+    L.misc = o;   o = align_up(o + 16u * 4, 16);
+    L.stat = L.misc + 48;
     L.total = o;
     return L;
 }
+
+// the layout of prologue_kernel: no queue, visited set, results or staged rows
+__host__ __device__ inline WarpLayout prologue_layout(int dtype, int d, int P, int n, int PA, int bcap, bool grouped,
+                                                      bool spill) {
+    WarpLayout L = make_layout(dtype, d, P, n, PA, 32, 1, bcap, 1, 1, false, grouped, spill);
+    uint32_t o = align_up(L.sc + L.sc_parts * n, 16);
+    L.bkey = o;   o = align_up(o + 8u * bcap, 16);
+    L.bidx = o;   o = align_up(o + 4u * bcap, 16);
+    L.pref = o;
+    L.nodes = o + align_up(4u * (n + 1), 16);
+    L.glist = L.nodes + 16u * L.ncap;
+    o = align_up(L.glist + 20u * L.gcap, 16);
+    L.misc = o;
+    L.total = o + 64;
+    return L;
+}
+
+// the layout of main_kernel: no tables, walk lists or bridge batch.  The
+// bridge window, the candidates and the staged neighbour rows share a region:
+// window and candidates are written only after the copies in flight have landed.
+__host__ __device__ inline WarpLayout main_layout(int dtype, int d, int capT, int kmax, int b, int R, bool stage,
+                                                  bool spill, uint32_t spill_heap) {
+    WarpLayout L = make_layout(dtype, d, 1, 1, 1, capT, kmax, 1, b, R, stage, false, spill, spill_heap);
+    const uint32_t vb = (uint32_t)d * (dtype == ANN_U8 ? 1u : 4u), wb = align_up(128u * (uint32_t)b, 16);
+    uint32_t o = align_up(vb, 16);
+    L.heap = o;   o = align_up(o + 8u * L.heap_cap, 16);
+    L.hash = o;   o = align_up(o + (spill ? 0u : 4u * (1u << L.hash_log)), 16);
+    L.rbuf = o;   o = align_up(o + (kmax > 32 ? 8u * kmax : 0u), 16);
+    L.stat = o;   o += 16;
+    L.wref = o;
+    L.wkey = o + wb;
+    L.cand = o + 2 * wb;
+    L.ckey = o + 3 * wb;
+    L.stage = o;
+    const uint32_t stage_bytes = L.stage_rows * L.stage_stride;
+    L.total = align_up(o + (stage_bytes > 4 * wb ? stage_bytes : 4 * wb), 16);
+    return L;
+}
+
+// The prologue walks until it has this many bridges, the first of which is
+// popped at once: a query that pops no other one never needs another walk (on
+// the SIFT-shaped sets a walk's first window holds one or two bridges, and the
+// next bridge's key must be known while the first one's references are popped).
+constexpr uint32_t kFirstBridges = 1;
+
+// What the prologue leaves for a query, and what a suspended one needs to go on.
+struct QRec {
+    uint64_t lo;                          // the walk's state (WalkState)
+    uint32_t width, kmin, kmaxall, flags; // flags: 1 nothing produced yet, 2 all produced, 4 capacity error
+    uint32_t bcnt;                        // bridges of the first batch
+    uint32_t walks, nodes, leaves;        // counters of the walks so far
+    uint32_t slot;                        // where the suspended state lies (~0: start again)
+    uint32_t pad;
+};
+constexpr uint32_t kSaveHeader = 64 + 256;  // counters, then the register part of the result list
 
 struct SearchArgs {
     DevIndex ix;
@@ -139,10 +219,21 @@ struct SearchArgs {
     const int32_t *list;
     const int32_t *list_count;
     int64_t list_len;
-    // persistent mode: work ticket counter (nullable)
-    int32_t *ticket;
+    // this launch: queries base .. base + chunk of the selection
+    int64_t base, chunk;
+    // [0] main loop's ticket, [1] suspended queries, [2] resume ticket, [3] slots taken
+    int32_t *counters;
+    QRec *rec;        // per query of the chunk
+    uint64_t *bkeys;  // first batch: bstore keys and indexes per query of the chunk
+    uint32_t *bidxs;
+    int32_t *susp;    // suspended queries (position in the chunk)
+    // suspended states: header, result list (rbuf), heap, visited set, overflow
+    uint8_t *save;
+    uint32_t nslots;
+    uint64_t save_stride;
+    uint32_t save_rbuf, save_heap, save_hash, save_spill;
     int capT;
-    int bcap;
+    int bcap, bstore;
     WarpLayout L;
     // per-warp global scratch of the large-budget kernels, wstride bytes per
     // warp: sorted bridge windows (gcap x (2 keys + 2 values)) at 0, the
@@ -365,14 +456,21 @@ __device__ inline void heap_build(uint64_t *h, uint32_t sz) {
     for (int64_t i = (int64_t)(sz - 2) / 32; i >= 0; i--) heap_sift_down(h, sz, (uint32_t)i);
 }
 
+// what the two moves below change; they are rare, so they are called out of
+// line, and take and return values so that the loop's copies stay in registers
+struct SpillMove {
+    uint64_t tau;
+    uint32_t sz, nb;
+};
+
 // move the heap's entries >= t (a low sampled quantile) to the overflow
-__device__ inline void spill_shrink(uint64_t *h, uint32_t &sz, Spill &sp) {
+static __device__ __noinline__ SpillMove spill_shrink(uint64_t *h, uint32_t sz, uint64_t *B, uint32_t nb) {
     const int lane = lane_id();
     const unsigned lt = (1u << lane) - 1;
     uint64_t smp[1] = {h[(uint32_t)(((uint64_t)lane * sz) >> 5)]};
     reg_bitonic_sort_t<1, uint64_t>(smp);
     const uint64_t t = __shfl_sync(0xffffffffu, smp[0], 12);  // an entry of the heap: at least it moves
-    uint32_t w = 0, nb = sp.nb;
+    uint32_t w = 0;
     for (uint32_t base = 0; base < sz; base += 32) {
         const uint32_t i = base + lane;
         const bool valid = i < sz;
@@ -381,36 +479,34 @@ __device__ inline void spill_shrink(uint64_t *h, uint32_t &sz, Spill &sp) {
         const unsigned mk = __ballot_sync(0xffffffffu, keep), mv = __ballot_sync(0xffffffffu, valid && !keep);
         __syncwarp();
         if (keep) h[w + __popc(mk & lt)] = x;  // in place: never past what this step read
-        if (valid && !keep) sp.B[nb + __popc(mv & lt)] = x;
+        if (valid && !keep) B[nb + __popc(mv & lt)] = x;
         w += __popc(mk);
         nb += __popc(mv);
         __syncwarp();
     }
-    sz = w;
-    sp.nb = nb;
-    sp.tau = t;
-    heap_build(h, sz);
+    heap_build(h, w);
+    return SpillMove{t, w, nb};
 }
 
 // the heap is empty: take the smallest overflow entries back (at most hcap)
-__device__ inline void spill_refill(uint64_t *h, uint32_t &sz, Spill &sp, uint32_t hcap) {
+static __device__ __noinline__ SpillMove spill_refill(uint64_t *h, uint64_t *B, uint32_t nb, uint32_t hcap) {
     const int lane = lane_id();
     const unsigned lt = (1u << lane) - 1;
     uint64_t t = ~0ull;  // everything fits: take it all
-    if (sp.nb > hcap) {
-        uint64_t smp[1] = {sp.B[(uint32_t)(((uint64_t)lane * sp.nb) >> 5)]};
+    if (nb > hcap) {
+        uint64_t smp[1] = {B[(uint32_t)(((uint64_t)lane * nb) >> 5)]};
         reg_bitonic_sort_t<1, uint64_t>(smp);
-        int r = (int)((32u * (hcap / 2)) / sp.nb);  // the sample whose quantile is about hcap / 2 entries
+        int r = (int)((32u * (hcap / 2)) / nb);  // the sample whose quantile is about hcap / 2 entries
         if (r > 31) r = 31;
         for (;;) {
             t = __shfl_sync(0xffffffffu, smp[0], r) + 1;  // entries up to that sample move
             uint32_t c = 0;
-            for (uint32_t i = lane; i < sp.nb; i += 32) c += sp.B[i] < t;
+            for (uint32_t i = lane; i < nb; i += 32) c += B[i] < t;
             c = __reduce_add_sync(0xffffffffu, c);
             if (c <= hcap) break;
             if (r == 0) {
                 uint64_t m = ~0ull;  // the exact minimum: one entry always fits
-                for (uint32_t i = lane; i < sp.nb; i += 32) m = min(m, sp.B[i]);
+                for (uint32_t i = lane; i < nb; i += 32) m = min(m, B[i]);
                 t = warp_min64(m) + 1;
                 break;
             }
@@ -418,29 +514,33 @@ __device__ inline void spill_refill(uint64_t *h, uint32_t &sz, Spill &sp, uint32
         }
     }
     uint32_t na = 0, w = 0;
-    for (uint32_t base = 0; base < sp.nb; base += 32) {
+    for (uint32_t base = 0; base < nb; base += 32) {
         const uint32_t i = base + lane;
-        const bool valid = i < sp.nb;
-        const uint64_t x = valid ? sp.B[i] : ~0ull;
+        const bool valid = i < nb;
+        const uint64_t x = valid ? B[i] : ~0ull;
         const bool in = valid && x < t;
         const unsigned mi = __ballot_sync(0xffffffffu, in), mo = __ballot_sync(0xffffffffu, valid && !in);
         __syncwarp();
         if (in) h[na + __popc(mi & lt)] = x;
-        if (valid && !in) sp.B[w + __popc(mo & lt)] = x;  // compacted in place
+        if (valid && !in) B[w + __popc(mo & lt)] = x;  // compacted in place
         na += __popc(mi);
         w += __popc(mo);
         __syncwarp();
     }
-    sz = na;
-    sp.nb = w;
-    sp.tau = w == 0 ? ~0ull : t;
-    heap_build(h, sz);
+    heap_build(h, na);
+    return SpillMove{w == 0 ? ~0ull : t, na, w};
+}
+
+__device__ __forceinline__ void spill_moved(const SpillMove &r, uint32_t &sz, Spill &sp) {
+    sz = r.sz;
+    sp.nb = r.nb;
+    sp.tau = r.tau;
 }
 
 template <bool SP>
 __device__ __forceinline__ void queue_pop(uint64_t *h, uint32_t &sz, Spill &sp, uint32_t hcap) {
     heap_pop(h, sz);
-    if (SP && sz == 0 && sp.nb > 0) spill_refill(h, sz, sp, hcap);
+    if (SP && sz == 0 && sp.nb > 0) spill_moved(spill_refill(h, sp.B, sp.nb, hcap), sz, sp);
 }
 
 // push the entries of the lanes in mask (pos = the lane's rank in mask)
@@ -456,7 +556,7 @@ __device__ __forceinline__ void queue_push(uint64_t *h, uint32_t &sz, Spill &sp,
     const bool inm = (mask >> lane) & 1u;
     unsigned ma = __ballot_sync(0xffffffffu, inm && e < sp.tau);
     while (sz + __popc(ma) > hcap) {
-        spill_shrink(h, sz, sp);
+        spill_moved(spill_shrink(h, sz, sp.B, sp.nb), sz, sp);
         ma = __ballot_sync(0xffffffffu, inm && e < sp.tau);
     }
     const unsigned mb = mask & ~ma;
@@ -466,19 +566,21 @@ __device__ __forceinline__ void queue_push(uint64_t *h, uint32_t &sz, Spill &sp,
         __syncwarp();
     }
     if (ma) heap_push_masked(h, sz, e, ma, __popc(ma & lt));
-    if (sz == 0 && sp.nb > 0) spill_refill(h, sz, sp, hcap);
+    if (sz == 0 && sp.nb > 0) spill_moved(spill_refill(h, sp.B, sp.nb, hcap), sz, sp);
 }
 
 // ---------------------------------------------------------------------------
 // distances of candidate rows to the query.  cand[0..m) are row ids; keys go
 // to ckey[0..m).  A group of G lanes (G = 16-byte chunks per row, at most 32)
 // handles one row; all loads of several rows are issued before any is used.
+// Out of line: the staged rows of the next pop serve most steps, and inlined
+// twice this cost the main loop its registers and instruction cache (T = 371 on
+// SIFT-shaped rows 1.31 ms against 1.06 ms out of line, the loop not yet tuned).
 // ---------------------------------------------------------------------------
 template <int DT>
-__device__ void cand_distances(const DevIndex &ix, const uint8_t *qbytes, const uint32_t *cand, int m,
-                               uint32_t *ckey) {
+__device__ __noinline__ void cand_distances(const void *X, int vb, const uint8_t *qbytes, const uint32_t *cand, int m,
+                                            uint32_t *ckey) {
     const int lane = lane_id();
-    const int vb = ix.d * (DT == ANN_U8 ? 1 : 4);  // bytes per vector
     const int nc = vb >> 4;                          // 16-byte chunks
     int G = 1;
     while (G * 2 <= nc && G * 2 <= 32) G *= 2;
@@ -498,7 +600,7 @@ __device__ void cand_distances(const DevIndex &ix, const uint8_t *qbytes, const 
 #pragma unroll
             for (int u = 0; u < MAXL; u++) {
                 const int j = base + u * per_round + grp;
-                if (j < m) buf[u] = __ldg((const uint4 *)((const uint8_t *)ix.X + (int64_t)cand[j] * vb) + lig);
+                if (j < m) buf[u] = __ldg((const uint4 *)((const uint8_t *)X + (int64_t)cand[j] * vb) + lig);
             }
 #pragma unroll
             for (int u = 0; u < MAXL; u++) {
@@ -545,7 +647,7 @@ __device__ void cand_distances(const DevIndex &ix, const uint8_t *qbytes, const 
             int r = u / cpl, c = lig + (u % cpl) * G;
             int j = base + r * per_round + grp;
             if (r < rounds_per_batch && u < rounds_per_batch * cpl && j < m && c < nc)
-                buf[u] = __ldg((const uint4 *)((const uint8_t *)ix.X + (int64_t)cand[j] * vb) + c);
+                buf[u] = __ldg((const uint4 *)((const uint8_t *)X + (int64_t)cand[j] * vb) + c);
         }
         // reduce row by row
         for (int r = 0; r < rounds_per_batch; r++) {
@@ -574,7 +676,7 @@ __device__ void cand_distances(const DevIndex &ix, const uint8_t *qbytes, const 
             }
             // rows wider than MAXL chunks per lane: stream the rest
             if (cpl > MAXL && j < m) {
-                const uint4 *row = (const uint4 *)((const uint8_t *)ix.X + (int64_t)cand[j] * vb);
+                const uint4 *row = (const uint4 *)((const uint8_t *)X + (int64_t)cand[j] * vb);
                 for (int c = lig + MAXL * G; c < nc; c += G) {
                     uint4 a = __ldg(row + c), q = qv[c];
                     if (DT == ANN_U8) {
@@ -1487,32 +1589,141 @@ __device__ __forceinline__ void sort_parts(const uint32_t *D, uint8_t *rk, uint8
 }
 
 // ---------------------------------------------------------------------------
-// one query, one warp
+// steps 1 and 2: the query, its part tables and ranks (in shared memory)
 // ---------------------------------------------------------------------------
-template <int DT, bool WIN, bool GRP>
-__device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t qi, uint8_t *wscratch) {
-    constexpr bool SP = WIN;  // the large-budget kernels also spill the queue and the visited set
+template <int DT>
+__device__ __forceinline__ void load_query(const SearchArgs &A, uint8_t *qb, int64_t qi) {
+    const int vb = A.ix.d * (DT == ANN_U8 ? 1 : 4);
+    const uint4 *src = (const uint4 *)((const uint8_t *)A.queries + qi * (int64_t)vb);
+    for (int c = lane_id(); c < (vb >> 4); c += 32) ((uint4 *)qb)[c] = __ldg(src + c);
+}
+
+template <int DT>
+__device__ void build_tables(const SearchArgs &A, uint8_t *smem, uint32_t &kmin, uint32_t &kmaxall) {
+    const DevIndex &ix = A.ix;
+    const WarpLayout &L = A.L;
+    const int lane = lane_id(), n = ix.n, P = ix.P, dp = ix.d / ix.P;
+    const uint8_t *qb = smem + L.q;
+    uint32_t *D = (uint32_t *)(smem + L.tabD), *misc = (uint32_t *)(smem + L.misc);
+    if (lane < 12) misc[lane] = 0;  // the rest holds the query's counters
+    const bool wide = dp % (DT == ANN_U8 ? 16 : 4) == 0;  // parts start on 16-byte boundaries
+    for (int p = 0; p < P; p++)
+        for (int c = lane; c < n; c += 32)
+            D[p * n + c] = wide ? part_key_wide<DT>(qb, ix.C, p, c, n, dp) : part_key_lane<DT>(qb, ix.C, p, c, n, dp);
+    __syncwarp();
+    uint32_t first_keys[kMaxP], last_keys[kMaxP];
+    sort_parts<DT>(D, smem + L.rank, smem + L.sc, P, n, (int)L.sc_parts, dp, first_keys, last_keys);
+    __syncwarp();
+    // smallest / largest bridge keys (exact sums) and a lower bound of the
+    // smallest suffix sum
+    auto key_sum = [&](const uint32_t *v) -> uint32_t {
+        return KeyOps<DT>::sum4(v[0], v[1], P > 2 ? v[2] : 0u, P > 3 ? v[3] : 0u);
+    };
+    kmin = key_sum(first_keys);
+    kmaxall = key_sum(last_keys);
+    uint32_t msuf;
+    if (ix.PA == 1) {
+        msuf = first_keys[1];
+    } else {
+        msuf = first_keys[2];
+        for (int p = 3; p < P; p++) msuf = KeyOps<DT>::add_lo(msuf, first_keys[p]);
+    }
+    if (lane == 0) {
+        misc[3] = msuf;
+        misc[4] = first_keys[P - 1];
+    }
+    __syncwarp();
+}
+
+// position w of the selection -> query; false for one whose k or T is out of range
+__device__ __forceinline__ int64_t query_of(const SearchArgs &A, int64_t w) { return A.list ? A.list[w] : w; }
+__device__ __forceinline__ int64_t query_end(const SearchArgs &A) {
+    const int64_t count = A.list_count ? (int64_t)*A.list_count : (A.list ? A.list_len : A.nq);
+    return count < A.base + A.chunk ? count : A.base + A.chunk;
+}
+__device__ __forceinline__ bool query_args(const SearchArgs &A, int64_t qi, int &k, int &T) {
+    k = A.k ? A.k[qi] : A.k_all;
+    T = A.T ? A.T[qi] : A.T_all;
+    return k >= 0 && k <= A.kmax && T >= 0 && T <= A.capT;
+}
+
+// steps 1 to 3 for one query: its record and first batch of bridges
+template <int DT, bool GRP>
+__device__ void prologue_one(const SearchArgs &A, uint8_t *smem, int64_t w) {
     const DevIndex &ix = A.ix;
     const WarpLayout &L = A.L;
     const int lane = lane_id();
-    const int n = ix.n, P = ix.P, PA = ix.PA, dp = ix.d / ix.P;
-    const int k = A.k ? A.k[qi] : A.k_all;
-    const int T = A.T ? A.T[qi] : A.T_all;
-    int32_t *oid = A.out_ids + qi * A.kmax;
-    // per-query counters (registers; the walk keeps its own in shared memory)
-    uint32_t n_refpops = 0, n_brpops = 0, n_ready = 0;
-    if (k < 0 || k > A.kmax || T < 0 || T > A.capT) {
+    const int64_t qi = query_of(A, w), at = w - A.base;
+    int k, T;
+    if (!query_args(A, qi, k, T) || T == 0) return;  // the main loop reads no record of these
+    load_query<DT>(A, smem + L.q, qi);
+    __syncwarp();
+    WalkState ws;
+    ws.lo = 0;
+    ws.first = true;
+    ws.exhausted = ix.M == 0;
+    ws.gpos = ws.gcnt = 0;
+    ws.gbuf = 0;
+    build_tables<DT>(A, smem, ws.kmin, ws.kmaxall);
+    if (DT == ANN_U8) {
+        uint32_t w0 = ws.kmin >> 8;  // measured on the SIFT-shaped 1M index: narrow first windows walk fewest leaves
+        ws.width = w0 < 1 ? 1 : w0;
+    } else {
+        ws.width = 1u << 16;  // about 0.8% relative in float32 bit space
+    }
+    bool cap_err = false;
+    const uint64_t *bkey = (const uint64_t *)(smem + L.bkey);
+    const uint32_t *bidx = (const uint32_t *)(smem + L.bidx), *misc = (const uint32_t *)(smem + L.misc);
+    uint32_t bcnt = 0;
+    while (bcnt < kFirstBridges && !ws.exhausted && !cap_err) {
+        const uint32_t c = refill<DT, GRP>(ix, smem, L, ws, cap_err);
+        for (uint32_t i = lane; i < c; i += 32) {
+            A.bkeys[at * A.bstore + bcnt + i] = bkey[i];
+            A.bidxs[at * A.bstore + bcnt + i] = bidx[i];
+        }
+        bcnt += c;
+        __syncwarp();
+    }
+    if (lane == 0) {
+        QRec r;
+        r.lo = ws.lo;
+        r.width = ws.width;
+        r.kmin = ws.kmin;
+        r.kmaxall = ws.kmaxall;
+        r.flags = (ws.first ? 1u : 0u) | (ws.exhausted ? 2u : 0u) | (cap_err ? 4u : 0u);
+        r.bcnt = bcnt;
+        r.walks = misc[8];
+        r.nodes = misc[9];
+        r.leaves = misc[10];
+        r.slot = 0xffffffffu;
+        r.pad = 0;
+        A.rec[at] = r;
+    }
+    __syncwarp();
+}
+
+// ---------------------------------------------------------------------------
+// the main loop of one query.  FULL: with the tables in shared memory, so that
+// it can walk for further bridges (resume_kernel); otherwise it suspends the
+// query when the first batch is used up.
+// ---------------------------------------------------------------------------
+template <int DT, bool SP, bool GRP, bool FULL>
+__device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t w, uint8_t *wscratch) {
+    const DevIndex &ix = A.ix;
+    const WarpLayout &L = A.L;
+    const int lane = lane_id();
+    const int64_t qi = query_of(A, w), at = w - A.base;
+    int k, T;
+    constexpr uint32_t kNoKey = DT == ANN_U8 ? 0xffffffffu : 0x7f800000u;
+    if (!query_args(A, qi, k, T)) {
         for (int j = lane; j < A.kmax; j += 32) {
-            oid[j] = -1;
-            if (A.out_keys) ((uint32_t *)A.out_keys)[qi * A.kmax + j] = DT == ANN_U8 ? 0xffffffffu : 0x7f800000u;
+            A.out_ids[qi * A.kmax + j] = -1;
+            if (A.out_keys) ((uint32_t *)A.out_keys)[qi * A.kmax + j] = kNoKey;
         }
         if (A.out_status && lane == 0) A.out_status[qi] = ANN_ERR_ARG;
         return;
     }
     uint8_t *qb = smem + L.q;
-    uint32_t *D = (uint32_t *)(smem + L.tabD);
-    uint8_t *rk = smem + L.rank;
-    uint8_t *sc = smem + L.sc;
     uint64_t *heap = (uint64_t *)(smem + L.heap);
     uint32_t *H = SP ? (uint32_t *)(wscratch + A.hash_off) : (uint32_t *)(smem + L.hash);
     Spill sp{SP ? (uint64_t *)(wscratch + A.spill_off) : nullptr, 0u, ~0ull};
@@ -1522,74 +1733,35 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t qi, uint8
     uint32_t *cand = (uint32_t *)(smem + L.cand);
     uint32_t *ckey = (uint32_t *)(smem + L.ckey);
     uint32_t *misc = (uint32_t *)(smem + L.misc);
+    int32_t *wref = (int32_t *)(smem + L.wref);
+    uint32_t *wkey = (uint32_t *)(smem + L.wkey);
+    // the current batch of bridges: the prologue's, then (FULL) the one in shared memory
+    bool own = false;  // FULL: the batch in shared memory
+    auto bkey_of = [&](uint32_t i) { return FULL && own ? bkey[i] : A.bkeys[at * A.bstore + i]; };
+    auto bidx_of = [&](uint32_t i) { return FULL && own ? bidx[i] : A.bidxs[at * A.bstore + i]; };
 
-    // load the query
-    const int vb = ix.d * (DT == ANN_U8 ? 1 : 4);
-    {
-        const uint4 *src = (const uint4 *)((const uint8_t *)A.queries + qi * (int64_t)vb);
-        uint4 *dst = (uint4 *)qb;
-        for (int c = lane; c < (vb >> 4); c += 32) dst[c] = __ldg(src + c);
-    }
-    // clear the visited set and the walk counters
-    if (SP) {
-        for (uint32_t i = 4 * lane; i < (1u << L.hash_log); i += 128) *(uint4 *)(H + i) = make_uint4(0, 0, 0, 0);
-    } else {
-        for (uint32_t i = lane; i < (1u << L.hash_log); i += 32) H[i] = 0;
-    }
-    if (lane < 16) misc[lane] = 0;
-    __syncwarp();
-
-    // 1. part tables
-    for (int idx = lane; idx < P * n; idx += 32) {
-        int p = idx / n, c = idx % n;
-        D[idx] = part_key_lane<DT>(qb, ix.C, p, c, n, dp);
-    }
-    __syncwarp();
-    // 2. per-part sort by (key, center id); ranks for every part, sorted keys/ids for prefix parts
-    uint32_t msuf = 0, minlast = 0;
-    uint32_t kmin = 0, kmaxall = 0;
-    {
-        uint32_t first_keys[kMaxP], last_keys[kMaxP];
-        sort_parts<DT>(D, rk, sc, P, n, (int)L.sc_parts, dp, first_keys, last_keys);
-        __syncwarp();
-        // smallest / largest bridge keys (exact sums) and a lower bound of the
-        // smallest suffix sum
-        auto key_sum = [&](const uint32_t *v) -> uint32_t {
-            return KeyOps<DT>::sum4(v[0], v[1], P > 2 ? v[2] : 0u, P > 3 ? v[3] : 0u);
-        };
-        kmin = key_sum(first_keys);
-        kmaxall = key_sum(last_keys);
-        if (PA == 1) {
-            msuf = first_keys[1];
-        } else {
-            msuf = first_keys[2];
-            for (int p = 3; p < P; p++) msuf = KeyOps<DT>::add_lo(msuf, first_keys[p]);
-        }
-        minlast = first_keys[P - 1];
-    }
-    if (lane == 0) {
-        misc[3] = msuf;
-        misc[4] = minlast;
-    }
-    __syncwarp();
-
-    // 3. Algorithm 1
+    load_query<DT>(A, qb, qi);
+    uint32_t flags = 2, bcnt = 0, slot0 = 0xffffffffu;
     WalkState ws;
-    ws.gpos = ws.gcnt = 0;
-    ws.gbuf = 0;
-    ws.lo = 0;
-    ws.first = true;
-    ws.exhausted = ix.M == 0;
-    ws.kmin = kmin;
-    ws.kmaxall = kmaxall;
-    ws.msuf = msuf;
-    if (DT == ANN_U8) {
-        uint32_t w = kmin >> 8;  // measured on the SIFT-shaped 1M index: narrow first windows walk fewest leaves
-        ws.width = w < 1 ? 1 : w;
-    } else {
-        ws.width = 1u << 16;  // about 0.8% relative in float32 bit space
+    if (T > 0) {
+        const QRec *r = A.rec + at;
+        flags = r->flags;
+        bcnt = r->bcnt;
+        if (FULL) {
+            ws.lo = r->lo;
+            ws.width = r->width;
+            slot0 = r->slot;
+        }
     }
-    uint32_t bcur = 0, bcnt = 0;
+    bool cap_err = (flags & 4u) != 0;
+    bool exhausted = (flags & 2u) != 0;
+    if (FULL) {
+        ws.first = (flags & 1u) != 0;
+        ws.exhausted = exhausted;
+        ws.gpos = ws.gcnt = 0;
+        ws.gbuf = 0;
+    }
+    uint32_t bcur = 0;
     uint32_t wstart = 0, wcnt = 0;  // bridge window: batch entries [wstart, wstart + wcnt)
     uint32_t wsize = 1;             // next window size: 1, 2, 4, ... 32 bridges
     uint32_t hsz = 0;               // heap size (identical in every lane)
@@ -1597,11 +1769,59 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t qi, uint8
     uint64_t rreg = ~0ull;          // result list in registers when k <= 32: lane l holds rank l
     const bool rsmall = k <= 32;
     int t = 0;
-    bool cap_err = false;
-    int64_t maxq = 0;
+    // per-query counters, kept only for a caller that asks for them, in shared
+    // memory: the loop is short of registers
+    uint32_t *stat = (uint32_t *)(smem + L.stat);  // largest queue, reference pops, bridge pops, preloaded rows
+    const bool stats = A.out_stats != nullptr;
+    if (stats && lane < 4) stat[lane] = 0;
+    auto count = [&](int i) {
+        if (stats && lane == 0) stat[i]++;
+    };
     const int b = ix.b, R = ix.R;
-    int32_t *wref = (int32_t *)(smem + L.wref);
-    uint32_t *wkey = (uint32_t *)(smem + L.wkey);
+    if (FULL && slot0 != 0xffffffffu) {
+        const uint8_t *sv = A.save + (uint64_t)slot0 * A.save_stride;
+        // a suspended query goes on: its first batch is used up
+        const uint32_t *h = (const uint32_t *)sv;
+        t = (int)h[0];
+        hsz = h[1];
+        rlen = h[2];
+        wsize = h[3];
+        if (stats && lane < 4) stat[lane] = h[4 + lane];
+        bcur = bcnt;
+        rreg = ((const uint64_t *)(sv + 64))[lane];
+        if (!rsmall)
+            for (uint32_t i = lane; i < rlen; i += 32) rbuf[i] = ((const uint64_t *)(sv + A.save_rbuf))[i];
+        for (uint32_t i = lane; i < hsz; i += 32) heap[i] = ((const uint64_t *)(sv + A.save_heap))[i];
+        for (uint32_t i = 4 * lane; i < (1u << L.hash_log); i += 128)
+            *(uint4 *)(H + i) = *(const uint4 *)(sv + A.save_hash + 4 * i);
+        if (SP) {
+            sp.nb = h[8];
+            sp.tau = ((uint64_t)h[10] << 32) | h[9];
+            for (uint32_t i = lane; i < sp.nb; i += 32) sp.B[i] = ((const uint64_t *)(sv + A.save_spill))[i];
+        }
+    } else {
+        for (uint32_t i = 4 * lane; i < (1u << L.hash_log); i += 128) *(uint4 *)(H + i) = make_uint4(0, 0, 0, 0);
+    }
+    __syncwarp();
+    if (FULL && T > 0) {
+        build_tables<DT>(A, smem, ws.kmin, ws.kmaxall);
+        if (lane == 0) {
+            misc[8] = A.rec[at].walks;
+            misc[9] = A.rec[at].nodes;
+            misc[10] = A.rec[at].leaves;
+        }
+        __syncwarp();
+    }
+    // A reference is popped while its key is at most bkey_now: the current
+    // bridge's key or, when the batch is used up, the end of what has been
+    // walked (no further bridge lies below it, so its key is not needed yet).
+    auto next_bound = [&]() -> uint32_t {
+        if (bcur < bcnt) return (uint32_t)(bkey_of(bcur) >> 32);
+        if (FULL ? ws.exhausted : exhausted) return 0xffffffffu;
+        return FULL ? (uint32_t)(ws.lo >> 32) : (uint32_t)(A.rec[at].lo >> 32);
+    };
+    uint32_t bkey_now = next_bound();
+
     // The next pop, once known, is staged: its kNN row in registers (nx_row)
     // and, when stage_rows > 0, its unvisited neighbours' vectors copied into
     // shared memory by cp.async (nx_vec, nx_mask = which row entries are new,
@@ -1619,8 +1839,14 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t qi, uint8
     const int snc = vbytes >> 4;  // 16-byte chunks per row
     uint8_t *stage = smem + L.stage;
 
-    while (t < T) {
-        if (bcur >= bcnt && (!ws.exhausted || (WIN && ws.gpos < ws.gcnt))) {
+    while (t < T && !cap_err) {
+        const bool hr = hsz > 0;
+        const uint64_t top = hr ? heap[0] : ~0ull;
+        const bool take_ref = hr && (uint32_t)(top >> 32) <= bkey_now;
+        // the rest of a sorted window lies below the walk's end: it has to come first
+        const bool rest = FULL && bcur >= bcnt && ws.gpos < ws.gcnt;
+        if (rest || (!take_ref && bcur >= bcnt)) {
+            if (!rest && (FULL ? ws.exhausted : exhausted)) break;  // no bridge and no reference left
             // the walk reuses the staging region
             if (cp_out) {
                 cp_async_wait_all();
@@ -1628,19 +1854,48 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t qi, uint8
             }
             nx_vec = false;
             __syncwarp();
-            if (WIN) bcnt = refill_windowed<DT, GRP>(ix, smem, L, ws, cap_err, wscratch, A.gcap);
-            else bcnt = refill<DT, GRP>(ix, smem, L, ws, cap_err);
-            bcur = 0;
-            wstart = 0;
-            wcnt = 0;
-            if (cap_err) break;
+            if constexpr (FULL) {
+                bcnt = refill_windowed<DT, GRP>(ix, smem, L, ws, cap_err, wscratch, A.gcap);
+                bcur = 0;
+                wstart = 0;
+                wcnt = 0;
+                own = true;
+                if (cap_err) break;
+                bkey_now = next_bound();
+                continue;
+            } else {
+                // suspend: the state goes to a slot (none left: the query starts again)
+                uint32_t s = 0;
+                if (lane == 0) s = (uint32_t)atomicAdd(A.counters + 3, 1);
+                s = __shfl_sync(0xffffffffu, s, 0);
+                if (s < A.nslots) {
+                    uint8_t *sv = A.save + (uint64_t)s * A.save_stride;
+                    if (lane == 0) {
+                        uint32_t *h = (uint32_t *)sv;
+                        h[0] = (uint32_t)t;
+                        h[1] = hsz;
+                        h[2] = rlen;
+                        h[3] = wsize;
+                        for (int i = 0; i < 4; i++) h[4 + i] = stats ? stat[i] : 0u;
+                        h[8] = sp.nb;
+                        h[9] = (uint32_t)sp.tau;
+                        h[10] = (uint32_t)(sp.tau >> 32);
+                    }
+                    ((uint64_t *)(sv + 64))[lane] = rreg;
+                    if (!rsmall)
+                        for (uint32_t i = lane; i < rlen; i += 32) ((uint64_t *)(sv + A.save_rbuf))[i] = rbuf[i];
+                    for (uint32_t i = lane; i < hsz; i += 32) ((uint64_t *)(sv + A.save_heap))[i] = heap[i];
+                    for (uint32_t i = 4 * lane; i < (1u << L.hash_log); i += 128)
+                        *(uint4 *)(sv + A.save_hash + 4 * i) = SP ? __ldcg((const uint4 *)(H + i)) : *(const uint4 *)(H + i);
+                    if (SP)
+                        for (uint32_t i = lane; i < sp.nb; i += 32) ((uint64_t *)(sv + A.save_spill))[i] = sp.B[i];
+                    if (lane == 0) A.rec[at].slot = s;
+                }
+                if (lane == 0) A.susp[atomicAdd(A.counters + 1, 1)] = (int32_t)at;
+                __syncwarp();
+                return;
+            }
         }
-        bool hb = bcur < bcnt;
-        bool hr = hsz > 0;
-        if (!hb && !hr) break;
-        uint64_t top = hr ? heap[0] : ~0ull;
-        uint64_t bc = hb ? bkey[bcur] : ~0ull;
-        bool take_ref = hr && (!hb || (uint32_t)(top >> 32) <= (uint32_t)(bc >> 32));
         int32_t x = -1;
         uint32_t xkey = 0;
         bool have_key = false;
@@ -1653,10 +1908,10 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t qi, uint8
             if (p == nx_id) {
                 x = nx_row;
                 staged = nx_vec;
-                n_ready++;
+                count(3);
             } else if (p == sp_id) {
                 x = sp_row;
-                n_ready++;
+                count(3);
             } else if (lane < R) {
                 x = __ldg(ix.G + (int64_t)p * R + lane);
             }
@@ -1668,7 +1923,7 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t qi, uint8
             } else {
                 sp_id = kNone;
             }
-            n_refpops++;
+            count(1);
         } else {
             // the bridge window reuses the staging region
             if (cp_out) {
@@ -1683,7 +1938,7 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t qi, uint8
                 wcnt = min(wsize, bcnt - bcur);
                 if (wsize < 32) wsize <<= 1;
                 for (int e = lane; e < (int)wcnt * b; e += 32) {
-                    uint32_t j = bidx[wstart + e / b];
+                    uint32_t j = bidx_of(wstart + e / b);
                     int32_t r = __ldg(ix.brefs + (int64_t)j * b + (e % b));
                     bool keep = r >= 0 && r < ix.N &&
                                 !(SP ? ghash_has(H, L.hash_log, (uint32_t)r) : hash_has(H, L.hash_log, (uint32_t)r));
@@ -1703,20 +1958,21 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t qi, uint8
                     nc += __popc(mk);
                 }
                 __syncwarp();
-                cand_distances<DT>(ix, qb, cand, nc, ckey);
+                cand_distances<DT>(ix.X, vbytes, qb, cand, nc, ckey);
                 for (int e = lane; e < (int)wcnt * b; e += 32)
                     if (wref[e] >= 0) wkey[e] = ckey[wkey[e]];
                 __syncwarp();
             }
             uint32_t wi = (bcur - wstart) * b;
             bcur++;
+            bkey_now = next_bound();
             alen = b;
             if (lane < b) {
                 x = wref[wi + lane];
                 xkey = wkey[wi + lane];
             }
             have_key = true;
-            n_brpops++;
+            count(2);
         }
         // the new references of this adjacency list, in list order, cut to the budget
         unsigned mask;
@@ -1737,30 +1993,42 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t qi, uint8
         const int pos = __popc(mask & ((1u << lane) - 1));
         uint64_t mine = ~0ull;
         if (m > 0) {
-            // mark them visited: the lowest lane among those whose probe ended on
-            // the same empty slot stores there; the others insert by CAS after it
-            const unsigned peers = __match_any_sync(0xffffffffu, inm ? slot : 0xfffffffeu);
-            const bool direct = inm && slot != kNone && (peers & ((1u << lane) - 1)) == 0;
-            if (direct) H[slot] = (uint32_t)x + 1;
-            __syncwarp();
+            // mark them visited: one lane among those whose probe ended on the
+            // same empty slot stores there; the others insert by CAS after it
+            bool direct;
+            if (SP) {
+                const unsigned peers = __match_any_sync(0xffffffffu, inm ? slot : 0xfffffffeu);
+                direct = inm && slot != kNone && (peers & ((1u << lane) - 1)) == 0;
+                if (direct) H[slot] = (uint32_t)x + 1;
+                __syncwarp();
+            } else {
+                // all store, the one that stays has it (a match over the warp takes 120 cycles)
+                if (inm && slot != kNone) H[slot] = (uint32_t)x + 1;
+                __syncwarp();
+                direct = inm && slot != kNone && H[slot] == (uint32_t)x + 1;
+                __syncwarp();
+            }
             if (inm && !direct) hash_add(H, L.hash_log, (uint32_t)x);
             uint32_t key = xkey;
             if (!have_key) {
-                if (staged) {
+                // candidates share their region with the staged rows
+                if (cp_out) {
                     cp_async_wait_all();
                     cp_out = false;
-                    __syncwarp();
+                }
+                __syncwarp();
+                if (staged) {
                     if (inm) key = row_key_smem<DT>(stage + (size_t)pos * L.stage_stride, qb, vbytes);
                 } else {
                     if (inm) cand[pos] = (uint32_t)x;
                     __syncwarp();
-                    cand_distances<DT>(ix, qb, cand, m, ckey);
+                    cand_distances<DT>(ix.X, vbytes, qb, cand, m, ckey);
                     if (inm) key = ckey[pos];
                 }
             }
             mine = inm ? (((uint64_t)key << 32) | (uint32_t)x) : ~0ull;
             queue_push<SP>(heap, hsz, sp, L.heap_cap, mine, mask, pos);
-            if ((int64_t)hsz + sp.nb + 1 > maxq) maxq = (int64_t)hsz + sp.nb + 1;
+            if (stats && lane == 0) stat[0] = max(stat[0], hsz + sp.nb + 1);
         }
         // The next pop is known now.  When it is a reference, take its kNN row
         // (usually the speculative one) and start copying its unvisited
@@ -1768,8 +2036,7 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t qi, uint8
         // next pop.
         if (t + m < T && hsz > 0) {
             const uint64_t ntop = heap[0];
-            const bool maybe_ref = bcur >= bcnt || (uint32_t)(ntop >> 32) <= (uint32_t)(bkey[bcur] >> 32);
-            if (maybe_ref) {
+            if ((uint32_t)(ntop >> 32) <= bkey_now) {
                 const uint32_t nid = (uint32_t)ntop;
                 if (nid != nx_id) {
                     nx_row = nid == sp_id ? sp_row : (lane < R ? __ldg(ix.G + (int64_t)nid * R + lane) : -1);
@@ -1777,7 +2044,7 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t qi, uint8
                 }
                 // vectors only when the next step is certainly this pop (no
                 // refill first) and no bridge-window entries are still pending
-                const bool refill_next = bcur >= bcnt && (!ws.exhausted || (WIN && ws.gpos < ws.gcnt));
+                const bool refill_next = FULL && bcur >= bcnt && ws.gpos < ws.gcnt;
                 if (L.stage_rows && !refill_next && bcur >= wstart + wcnt) {
                     uint32_t s2 = kNone;
                     bool nw = false;
@@ -1813,10 +2080,10 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t qi, uint8
                     uint64_t e = __shfl_sync(0xffffffffu, mine, j);
                     kth = __shfl_sync(0xffffffffu, rreg, k - 1);
                     if (e >= kth) continue;
-                    int pos = __popc(__ballot_sync(0xffffffffu, rreg < e));
+                    int rpos = __popc(__ballot_sync(0xffffffffu, rreg < e));
                     uint64_t up = __shfl_up_sync(0xffffffffu, rreg, 1);
-                    if (lane == pos) rreg = e;
-                    else if (lane > pos) rreg = up;
+                    if (lane == rpos) rreg = e;
+                    else if (lane > rpos) rreg = up;
                     if ((int)rlen < k) rlen++;
                 }
             }
@@ -1827,7 +2094,7 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t qi, uint8
                 // position = number of entries smaller than e
                 int cntless = 0;
                 for (int i = lane; i < (int)rlen; i += 32) cntless += rbuf[i] < e;
-                for (int off = 16; off > 0; off >>= 1) cntless += __shfl_xor_sync(0xffffffffu, cntless, off);
+                cntless = __reduce_add_sync(0xffffffffu, cntless);
                 int newlen = (int)rlen < k ? (int)rlen + 1 : k;
                 // shift [cntless, newlen-1) up by one, top-down in chunks of 32
                 for (int top_i = newlen - 1; top_i > cntless; top_i -= 32) {
@@ -1849,66 +2116,79 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t qi, uint8
     // nothing may still land in shared memory once this query ends
     if (cp_out) cp_async_wait_all();
     __syncwarp();
-    if (rsmall) {
-        if (lane < k) rbuf[lane] = rreg;
-        __syncwarp();
-    }
-    __syncwarp();
     // outputs
     for (int j = lane; j < A.kmax; j += 32) {
-        bool have = j < (int)rlen && j < k;
-        oid[j] = have ? (int32_t)(uint32_t)rbuf[j] : -1;
-        if (A.out_keys) {
-            uint32_t kv = have ? (uint32_t)(rbuf[j] >> 32) : (DT == ANN_U8 ? 0xffffffffu : 0x7f800000u);
-            ((uint32_t *)A.out_keys)[qi * A.kmax + j] = kv;
-        }
+        const bool have = j < (int)rlen && j < k;
+        const uint64_t e = !have ? 0ull : (rsmall ? rreg : rbuf[j]);
+        A.out_ids[qi * A.kmax + j] = have ? (int32_t)(uint32_t)e : -1;
+        if (A.out_keys) ((uint32_t *)A.out_keys)[qi * A.kmax + j] = have ? (uint32_t)(e >> 32) : kNoKey;
     }
     if (lane == 0) {
         if (A.out_status) A.out_status[qi] = cap_err ? ANN_ERR_CAPACITY : ANN_OK;
         if (A.out_stats) {
             int64_t *o = A.out_stats + qi * ANN_NSTATS;
+            const QRec *r = A.rec + at;
             o[ANN_STAT_DISCOVERED] = t;
-            o[ANN_STAT_REF_POPS] = n_refpops;
-            o[ANN_STAT_BRIDGE_POPS] = n_brpops;
-            o[ANN_STAT_WALKS] = misc[8];
-            o[ANN_STAT_WALK_NODES] = misc[9];
-            o[ANN_STAT_WALK_LEAVES] = misc[10];
-            o[ANN_STAT_MAX_Q] = maxq;
-            o[ANN_STAT_PRELOADED] = n_ready;
+            o[ANN_STAT_REF_POPS] = stat[1];
+            o[ANN_STAT_BRIDGE_POPS] = stat[2];
+            o[ANN_STAT_WALKS] = FULL ? misc[8] : (T > 0 ? r->walks : 0u);
+            o[ANN_STAT_WALK_NODES] = FULL ? misc[9] : (T > 0 ? r->nodes : 0u);
+            o[ANN_STAT_WALK_LEAVES] = FULL ? misc[10] : (T > 0 ? r->leaves : 0u);
+            o[ANN_STAT_MAX_Q] = stat[0];
+            o[ANN_STAT_PRELOADED] = stat[3];
         }
     }
     __syncwarp();
 }
 
-template <int DT, bool WIN, bool GRP>
-__global__ void __launch_bounds__(192, 2) search_kernel(SearchArgs A) {
+template <int DT, bool GRP>
+__global__ void __launch_bounds__(128, 4) prologue_kernel(const __grid_constant__ SearchArgs A) {
+    extern __shared__ __align__(16) uint8_t smem_all[];
+    const int warp = threadIdx.x >> 5;
+    if (blockIdx.x == 0 && threadIdx.x < 4) A.counters[threadIdx.x] = 0;  // for the two kernels that follow
+    uint8_t *smem = smem_all + (size_t)warp * A.L.total;
+    const int64_t end = query_end(A), step = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t w = A.base + (int64_t)blockIdx.x * (blockDim.x >> 5) + warp; w < end; w += step)
+        prologue_one<DT, GRP>(A, smem, w);
+}
+
+// queries are pulled from a ticket: their lengths differ
+template <int DT, bool SP, int CTAS>
+__global__ void __launch_bounds__(32 * kMainWarps, CTAS) main_kernel(const __grid_constant__ SearchArgs A) {
     extern __shared__ __align__(16) uint8_t smem_all[];
     const int warp = threadIdx.x >> 5;
     uint8_t *smem = smem_all + (size_t)warp * A.L.total;
-    uint8_t *wscratch = WIN ? A.gscratch + ((size_t)blockIdx.x * (blockDim.x >> 5) + warp) * A.wstride : nullptr;
-    const int64_t count = A.list_count ? (int64_t)*A.list_count : (A.list ? A.list_len : A.nq);
-    if (A.ticket) {
-        // persistent: pull queries from the device work queue
-        for (;;) {
-            int32_t w = 0;
-            if (lane_id() == 0) w = atomicAdd(A.ticket, 1);
-            w = __shfl_sync(0xffffffffu, w, 0);
-            if (w >= count) break;
-            int64_t qi = A.list ? A.list[w] : w;
-            search_one<DT, WIN, GRP>(A, smem, qi, wscratch);
-        }
-    } else {
-        const int64_t gw = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
-        const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-        for (int64_t w = gw; w < count; w += nw) {
-            int64_t qi = A.list ? A.list[w] : w;
-            search_one<DT, WIN, GRP>(A, smem, qi, wscratch);
-        }
+    uint8_t *wscratch = SP ? A.gscratch + ((size_t)blockIdx.x * (blockDim.x >> 5) + warp) * A.wstride : nullptr;
+    const int64_t count = query_end(A) - A.base;
+    for (;;) {
+        int32_t w = 0;
+        if (lane_id() == 0) w = atomicAdd(A.counters, 1);
+        w = __shfl_sync(0xffffffffu, w, 0);
+        if (w >= count) break;
+        search_one<DT, SP, false, false>(A, smem, A.base + w, wscratch);
+    }
+}
+
+template <int DT, bool SP, bool GRP>
+__global__ void __launch_bounds__(192, 2) resume_kernel(const __grid_constant__ SearchArgs A) {
+    extern __shared__ __align__(16) uint8_t smem_all[];
+    const int warp = threadIdx.x >> 5;
+    uint8_t *smem = smem_all + (size_t)warp * A.L.total;
+    uint8_t *wscratch = A.gscratch + ((size_t)blockIdx.x * (blockDim.x >> 5) + warp) * A.wstride;
+    const int32_t count = A.counters[1];
+    for (;;) {
+        int32_t i = 0;
+        if (lane_id() == 0) i = atomicAdd(A.counters + 2, 1);
+        i = __shfl_sync(0xffffffffu, i, 0);
+        if (i >= count) break;
+        search_one<DT, SP, GRP, true>(A, smem, A.base + A.susp[i], wscratch);
     }
 }
 
 // Launch helpers of the kernels with the c2 group level (ann_search_grp.cu).
-cudaError_t config_grouped(int dtype, bool win, size_t smem, int threads, int *blocks_per_sm);
-void launch_grouped(int dtype, bool win, dim3 grid, dim3 block, size_t smem, cudaStream_t s, const SearchArgs &A);
+cudaError_t config_grouped(int dtype, bool sp, size_t smem, int threads, int *blocks_per_sm);
+cudaError_t config_grouped_prologue(int dtype, size_t smem, int threads, int *blocks_per_sm);
+void launch_grouped(int dtype, bool sp, dim3 grid, dim3 block, size_t smem, cudaStream_t s, const SearchArgs &A);
+void launch_grouped_prologue(int dtype, dim3 grid, dim3 block, size_t smem, cudaStream_t s, const SearchArgs &A);
 
 }  // namespace ann
