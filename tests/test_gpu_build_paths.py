@@ -146,3 +146,49 @@ def test_u8_tensor_knn_tile_edges_and_extreme_rows(ann, kind, N, nq, d, k):
     np.testing.assert_array_equal(ids.cpu().numpy(), want_ids)
     np.testing.assert_array_equal(ann.keys_as_uint32(keys).astype(np.float64),
                                   np.where(np.isinf(want_keys), 4294967295.0, want_keys))
+
+
+@pytest.mark.parametrize("m,dp,ks,w,T,L,shift", [(16, 8, 256, 6, 100, 10**9, 0), (8, 5, 37, 1, 128, 900, 0),
+                                                 (2, 4, 101, 3, 1, 5000, 0), (12, 3, 100, 5, 128, 10**9, 0),
+                                                 (5, 12, 16, 4, 33, 3333, 0), (16, 4, 256, 5, 128, 10**9, 4),
+                                                 (3, 4, 1, 4, 77, 10**9, 0)])
+def test_adc_rerank_is_bit_exact_in_its_stated_order(ann, m, dp, ks, w, T, L, shift):
+    # the float32 operations of ann.h in their order, with numpy; lists of up to 3,000 members (the buffer is cut
+    # several times), a list visited twice, absent lists, codes off their natural alignment, one codeword (all keys tie)
+    rng = np.random.default_rng(m * 1000 + ks)
+    d, N, K, nq = m * dp, 9000, 7, 5
+    C = rng.standard_normal((K, d)).astype(np.float32)
+    books = rng.standard_normal((m, ks, dp)).astype(np.float32)
+    codes = rng.integers(0, ks, (N, m)).astype(np.uint8)
+    assign = np.sort(rng.choice(K, N, p=[.34, .3, .2, .1, .05, .009, .001]))
+    members = np.argsort(assign, kind="stable").astype(np.int32)
+    offsets = np.concatenate([[0], np.cumsum(np.bincount(assign, minlength=K))]).astype(np.int64)
+    Q = rng.standard_normal((nq, d)).astype(np.float32)
+    lists = np.stack([rng.permutation(K)[:w] for _ in range(nq)]).astype(np.int32)
+    lists[0, -1] = lists[0, 0]
+    lists[1, 0] = -1
+    flat = torch.empty(codes.size + shift, dtype=torch.uint8, device="cuda")
+    flat[shift:] = dev(codes.reshape(-1))
+    ids, keys, seen = ann.ann_adc_rerank(dev(Q), dev(lists), dev(offsets), dev(members), dev(C),
+                                         flat[shift:].view(N, m), dev(books), L, T)
+    for i in range(nq):
+        got, total = [np.zeros(0, np.uint64)], 0
+        for c in lists[i]:
+            if c < 0 or total >= L:
+                continue
+            x = members[offsets[c]:offsets[c + 1]][:L - total]
+            total += len(x)
+            r = (Q[i] - C[c]).reshape(m, 1, dp)
+            table = np.zeros((m, ks), np.float32)
+            for t in range(dp):
+                e = r[:, :, t] - books[:, :, t]
+                table = table + e * e
+            key = np.zeros(len(x), np.float32)
+            for j in range(m):
+                key = key + table[j, codes[x, j]]
+            got.append(np.stack([key.view(np.uint32).astype(np.uint64) << 32 | x.astype(np.uint64)]).reshape(-1))
+        best = np.sort(np.concatenate(got))[:T]
+        assert int(seen[i]) == total
+        np.testing.assert_array_equal(ids[i].cpu().numpy()[:len(best)], (best & 0xffffffff).astype(np.int32))
+        np.testing.assert_array_equal(keys[i].cpu().numpy().view(np.uint32)[:len(best)], (best >> 32).astype(np.uint32))
+        assert np.all(ids[i].cpu().numpy()[len(best):] == -1)
