@@ -137,6 +137,24 @@ int search_num_buckets();
 // implemented in ann_knn_tc.cu: exact k-NN of uint8 rows on the tensor cores, d in {64, 128}, k <= 32
 int knn_u8_tensor(const uint8_t *refs, int64_t N, const uint8_t *queries, int64_t nq, int d, int k,
                   int exclude_self, int32_t *out_ids, uint32_t *out_keys, cudaStream_t s);
+// The leaf step of the approximate graph on the tensor cores (d in {64, 128}):
+// in every round the rows in leaf order (ids ascending inside a leaf) against
+// their leaf-mates.  round() leaves two sorted lists of R (key << 32 | id)
+// values (~0 padded) per position in `lists`; *err is set when a wait timed
+// out, the lists then being undefined.
+struct LeafTc {
+    AsyncBufs bufs;
+    int64_t N = 0;
+    int d = 0, R = 0, levels = 0, nsm = 0;
+    uint64_t *lists = nullptr;
+    uint16_t *rb = nullptr, *rslab = nullptr, *qslab = nullptr;
+    uint32_t *norm = nullptr, *limit = nullptr, *ids = nullptr;
+    int *err = nullptr, *pend_col = nullptr;
+    float4 *pend = nullptr;
+    explicit LeafTc(cudaStream_t s) : bufs(s) {}
+    int prepare(int64_t N, int d, int R, int levels, cudaStream_t s);
+    int round(const uint8_t *X, const uint64_t *order, uint64_t idmask, const uint64_t *graph, cudaStream_t s);
+};
 // implemented in ann_index.cu
 int build_bridge_index_from_host(ann_index *ix, int64_t M, const uint64_t *ids,
                                  const int64_t *offsets, const int32_t *refs);

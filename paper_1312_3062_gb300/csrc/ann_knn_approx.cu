@@ -10,10 +10,13 @@
 //     of the 64-bit keys (segment, <u, x> + bias, id) over all N positions:
 //     a segment's members occupy the same positions before and after, so a
 //     global sort is the per-segment sort.
-//  2. Leaf step: every point is offered every other leaf member.  A leaf that
-//     fits in shared memory is staged whole by one CTA (one warp per point);
-//     a larger one (d <= 128) is streamed through shared memory by CTAs of
-//     32 members each, two per warp.
+//  2. Leaf step: every point is offered every other leaf member.  For d 64 and
+//     128 and leaves of more than leaf_tc_from(R) points the keys come from the
+//     tensor cores (LeafTc: rows gathered in leaf order, 128 of a leaf against
+//     the leaf, the two lists of a row merged into the graph); other leaves
+//     that fit in shared memory are staged whole by one CTA (one warp per
+//     point), larger ones (d <= 128) are streamed through shared memory by CTAs
+//     of 32 members each, two per warp.
 //  3. `iters` propagation steps (one warp per point): row i is offered the
 //     rows of its neighbours, read from the previous step's graph.
 // A row is a warp-held ascending list of packed (key << 32 | id) values, one
@@ -39,6 +42,12 @@ constexpr int TILE_THREADS = 512;
 constexpr int TILE_I = 2 * TILE_THREADS / 32;  // members per CTA of the streamed leaf kernel
 constexpr int TILE_J = 256;                    // leaf rows per shared-memory pass
 constexpr unsigned FULL = 0xffffffffu;
+// The tensor cores take leaves of more than this many points.  What they pay
+// beyond the tiles grows with the insertions into a row's list.  500,000 rows
+// of 128 bytes, 2 rounds, other kernels / tensor cores: R = 8, leaves of 122
+// 5.3 / 5.9, 244 5.6 / 5.4 ms; R = 20, 244 6.6 / 7.3, 488 7.9 / 7.8, 976
+// 14.0 / 8.2, 7812 57 / 10.8 ms; R = 32, 488 9.1 / 9.9, 976 16.1 / 11.0 ms.
+inline int64_t leaf_tc_from(int R) { return std::max(96, 24 * R); }
 
 // sum of x_b * u_b over 4 byte pairs: x unsigned, u signed (PTX dp4a with
 // mixed operand types)
@@ -114,13 +123,47 @@ __global__ void rp_key_kernel(const uint8_t *__restrict__ X, int64_t N, int d, c
     out[p] = (s << seg_shift) | ((uint64_t)(uint32_t)(acc + bias) << id_bits) | id;
 }
 
+// key of position p after the last level: (leaf, id), so that ids ascend inside
+// a leaf (the tensor-core leaf step breaks ties by position)
+__global__ void rp_leaf_key_kernel(int64_t N, int levels, const uint64_t *__restrict__ prev, uint64_t idmask, int id_bits,
+                                   uint64_t *__restrict__ out) {
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= N) return;
+    int64_t lo = 0, hi = N;
+    uint64_t s = 0;
+    for (int k = 0; k < levels; k++) {
+        const int64_t m = lo + (hi - lo) / 2;
+        const bool right = p >= m;
+        lo = right ? m : lo;
+        hi = right ? hi : m;
+        s = 2 * s + right;
+    }
+    out[p] = (s << id_bits) | (prev ? prev[p] & idmask : (uint64_t)p);
+}
+
+// offer the two lists of every position to the row of its id
+__global__ void __launch_bounds__(256) rp_merge_kernel(int64_t N, int R, const uint32_t *__restrict__ ids,
+                                                       const uint64_t *__restrict__ lists, const int *__restrict__ err,
+                                                       uint64_t *__restrict__ rows) {
+    const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = lane_id();
+    if (p >= N || *err) return;  // whole warps
+    const uint32_t id = ids[p];
+    uint64_t mine = lane < R ? rows[(int64_t)id * R + lane] : ~0ull;
+    for (int h = 0; h < 2; h++)
+        offer_lanes(mine, lane < R ? lists[(p * 2 + h) * R + lane] : ~0ull, R);
+    if (lane < R) rows[(int64_t)id * R + lane] = mine;
+}
+
 // one CTA per leaf: stage the leaf's rows, offer every leaf-mate to each
 // member's row (rows: N*R packed values, updated in place; a point lies in
 // exactly one leaf per round)
 __global__ void __launch_bounds__(LEAF_THREADS) rp_leaf_kernel(const uint8_t *__restrict__ X, int64_t N, int d,
                                                                int R, int levels, const uint64_t *__restrict__ sorted,
-                                                               uint64_t idmask, uint64_t *__restrict__ rows) {
+                                                               uint64_t idmask, uint64_t *__restrict__ rows,
+                                                               const int *__restrict__ only_if) {
     extern __shared__ __align__(16) uint8_t sm[];
+    if (only_if && !*only_if) return;
     const int64_t leaf = blockIdx.x;
     int64_t lo = 0, hi = N;
     for (int k = levels - 1; k >= 0; k--) {
@@ -182,8 +225,10 @@ __device__ __forceinline__ uint32_t dot16(uint4 a, uint4 b, uint32_t acc) {
 __global__ void __launch_bounds__(TILE_THREADS) rp_leaf_tiled_kernel(const uint8_t *__restrict__ X, int64_t N,
                                                                      int d, int R, int levels, int chunks,
                                                                      const uint64_t *__restrict__ sorted,
-                                                                     uint64_t idmask, uint64_t *__restrict__ rows) {
+                                                                     uint64_t idmask, uint64_t *__restrict__ rows,
+                                                                     const int *__restrict__ only_if) {
     extern __shared__ __align__(16) uint8_t sm[];
+    if (only_if && !*only_if) return;
     const int64_t leaf = blockIdx.x / chunks;
     const int chunk = (int)(blockIdx.x % chunks);
     int64_t lo = 0, hi = N;
@@ -264,21 +309,24 @@ __global__ void __launch_bounds__(TILE_THREADS) rp_leaf_tiled_kernel(const uint8
     if (v2 && lane < R) rows[(int64_t)g2 * R + lane] = m2;
 }
 
-// one warp per point: offer the rows of its neighbours (from rin) to its row
+// One warp per point: offer the rows of its neighbours (from rin) to its row.
+// The candidates not yet in the row are packed, and G lanes read one of them
+// together (G = 16-byte chunks of a row, a power of two): with each lane reading
+// a row of its own every load touched 32 lines.  1M x 128 bytes, R = 16: 7.1 ms
+// then, 1.4 ms less now (the gather of R^2 rows per point from L2 remains).
 __global__ void __launch_bounds__(PROP_THREADS) rp_prop_kernel(const uint8_t *__restrict__ X, int64_t N, int d, int R,
-                                                               const uint64_t *__restrict__ rin,
+                                                               int G, const uint64_t *__restrict__ rin,
                                                                uint64_t *__restrict__ rout) {
+    __shared__ uint32_t s_id[PROP_THREADS], s_key[PROP_THREADS];  // 32 per warp
     const int lane = lane_id();
     const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (i >= N) return;  // whole warps
+    uint32_t *cid = s_id + (threadIdx.x & ~31u), *ckey = s_key + (threadIdx.x & ~31u);
     const uint64_t orig = lane < R ? rin[i * R + lane] : ~0ull;
     uint64_t mine = orig;
-    const int W = d / 16;
+    const int W = d / 16, lig = lane & (G - 1), per = 32 / G;  // candidates per step
     const uint4 *xi = (const uint4 *)(X + i * d);
-    uint4 a[8];
-#pragma unroll
-    for (int w = 0; w < 8; w++)
-        if (w < W) a[w] = __ldg(xi + w);
+    const uint4 a = __ldg(xi + lig);  // G <= W
     const int RR = R * R;
     for (int e0 = 0; e0 < RR; e0 += 32) {
         const int e = e0 + lane;
@@ -288,17 +336,23 @@ __global__ void __launch_bounds__(PROP_THREADS) rp_prop_kernel(const uint8_t *__
         if (e < RR && j != 0xffffffffu) c = (uint32_t)__ldg(rin + (int64_t)j * R + (e - jj * R));
         bool fresh = c != 0xffffffffu && c != (uint32_t)i;
         for (int q = 0; q < R; q++)  // already in the row: nothing to compute
-            if ((uint32_t)__shfl_sync(FULL, mine, q) == c) fresh = false;
-        uint64_t v = ~0ull;
-        if (fresh) {
-            const uint4 *xc = (const uint4 *)(X + (int64_t)c * d);
-            uint32_t acc = 0;
-#pragma unroll
-            for (int w = 0; w < 8; w++)
-                if (w < W) acc = sqd16(a[w], __ldg(xc + w), acc);
-            for (int w = 8; w < W; w++) acc = sqd16(__ldg(xi + w), __ldg(xc + w), acc);
-            v = ((uint64_t)acc << 32) | c;
+            if (__shfl_sync(FULL, (uint32_t)mine, q) == c) fresh = false;
+        const unsigned fm = __ballot_sync(FULL, fresh);
+        const int nf = __popc(fm);
+        if (!nf) continue;
+        if (fresh) cid[__popc(fm & ((1u << lane) - 1))] = c;
+        __syncwarp();
+        for (int f0 = 0; f0 < nf; f0 += per) {
+            const int f = f0 + lane / G;
+            const uint4 *xc = (const uint4 *)(X + (int64_t)cid[f < nf ? f : 0] * d);
+            uint32_t acc = sqd16(a, __ldg(xc + lig), 0u);
+            for (int w = lig + G; w < W; w += G) acc = sqd16(__ldg(xi + w), __ldg(xc + w), acc);
+            for (int off = G >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(FULL, acc, off);
+            if (f < nf && lig == 0) ckey[f] = acc;
         }
+        __syncwarp();
+        const uint64_t v = lane < nf ? ((uint64_t)ckey[lane] << 32) | cid[lane] : ~0ull;
+        __syncwarp();
         offer_lanes(mine, v, R);
     }
     if (lane < R) rout[i * R + lane] = mine;
@@ -380,7 +434,8 @@ extern "C" int ann_build_knn_graph_approx(const void *data, int dtype, int64_t N
     } while (0)
     AP_CUDA(cudaMallocAsync((void **)&ra, sizeof(uint64_t) * (size_t)N * R, s));
     if (iters > 0) AP_CUDA(cudaMallocAsync((void **)&rb, sizeof(uint64_t) * (size_t)N * R, s));
-    if (levels > 0) {
+    const bool tensor = (d == 64 || d == 128) && largest > leaf_tc_from(R);
+    if (levels > 0 || tensor) {
         AP_CUDA(cudaMallocAsync((void **)&k0, sizeof(uint64_t) * (size_t)N, s));
         AP_CUDA(cudaMallocAsync((void **)&k1, sizeof(uint64_t) * (size_t)N, s));
         cub::DoubleBuffer<uint64_t> probe(k0, k1);
@@ -391,6 +446,14 @@ extern "C" int ann_build_knn_graph_approx(const void *data, int dtype, int64_t N
     if (tiled) AP_CUDA(cudaFuncSetAttribute(rp_leaf_tiled_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             (int)smem));
     else AP_CUDA(cudaFuncSetAttribute(rp_leaf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    LeafTc tc(s);
+    if (tensor) {
+        const int rc = tc.prepare(N, d, R, levels, s);
+        if (rc != ANN_OK) {
+            release();
+            return rc;
+        }
+    }
     const int64_t nseg = nleaves - 1;
     const unsigned gridN = (unsigned)((N + 255) / 256);
     for (int r = 0; r < rounds; r++) {
@@ -407,17 +470,39 @@ extern "C" int ann_build_knn_graph_approx(const void *data, int dtype, int64_t N
             AP_CUDA(cub::DeviceRadixSort::SortKeys(temp, tb, keys, (int)N, 0, l + proj_bits + id_bits, s));
         }
         const uint64_t *sorted = levels > 0 ? keys.Current() : nullptr;
+        if (tensor) {
+            // ids ascending inside a leaf, then the leaves' keys
+            uint64_t *out = levels > 0 ? keys.Alternate() : keys.Current();
+            rp_leaf_key_kernel<<<gridN, 256, 0, s>>>(N, levels, sorted, idmask, id_bits, out);
+            AP_CUDA(cudaGetLastError());
+            if (levels > 0) {
+                keys.selector ^= 1;
+                size_t tb = temp_bytes;
+                AP_CUDA(cub::DeviceRadixSort::SortKeys(temp, tb, keys, (int)N, 0, levels + id_bits, s));
+            }
+            sorted = keys.Current();
+            const int rc = tc.round((const uint8_t *)data, sorted, idmask, ra, s);
+            if (rc != ANN_OK) {
+                release();
+                return rc;
+            }
+            rp_merge_kernel<<<(unsigned)((N * 32 + 255) / 256), 256, 0, s>>>(N, R, tc.ids, tc.lists, tc.err, ra);
+        }
+        // other shapes, or (decided on the device) a tensor-core step that gave up
+        const int *only_if = tensor ? tc.err : nullptr;
         if (tiled)
             rp_leaf_tiled_kernel<<<(unsigned)(nleaves * chunks), TILE_THREADS, smem, s>>>(
-                (const uint8_t *)data, N, d, R, levels, chunks, sorted, idmask, ra);
+                (const uint8_t *)data, N, d, R, levels, chunks, sorted, idmask, ra, only_if);
         else
             rp_leaf_kernel<<<(unsigned)nleaves, LEAF_THREADS, smem, s>>>((const uint8_t *)data, N, d, R, levels,
-                                                                         sorted, idmask, ra);
+                                                                         sorted, idmask, ra, only_if);
         AP_CUDA(cudaGetLastError());
     }
     const unsigned gridW = (unsigned)((N * 32 + PROP_THREADS - 1) / PROP_THREADS);
     for (int it = 0; it < iters; it++) {
-        rp_prop_kernel<<<gridW, PROP_THREADS, 0, s>>>((const uint8_t *)data, N, d, R, ra, rb);
+        int G = 1;
+        while (2 * G <= d / 16 && G < 32) G *= 2;
+        rp_prop_kernel<<<gridW, PROP_THREADS, 0, s>>>((const uint8_t *)data, N, d, R, G, ra, rb);
         AP_CUDA(cudaGetLastError());
         std::swap(ra, rb);
     }

@@ -39,6 +39,8 @@
 // distances, 1340 with the slab); 138 ms with norms added and sorted insertions
 // into shared memory in the epilogue.  10,000 queries against 1M rows, k = 10:
 // 2.4 ms, 9.7 before (79 CTAs, no ranges).
+// The leaf step of the approximate graph (knn_u8_leaves) is the same kernel with
+// other items: rows in leaf order, and 128 rows of a leaf against that leaf.
 // Every mbarrier wait is bounded; on timeout the CTA records an error and
 // every role leaves its loop, so the kernel always returns and frees TMEM.
 #include <cuda.h>
@@ -67,6 +69,8 @@ struct Params {
     int64_t nq, N;
     int d, k, exclude_self;
     int nsplit;                   // ranges of reference tiles per block of query rows
+    int levels, leaf_blocks;      // leaves: halvings of [0, N), 128-row blocks of the largest leaf
+    const uint32_t *ids;          // leaves: the id of the row at each position
     const uint32_t *qnorm;
     uint32_t *row_limit;          // per query row: the smallest k-th key of its lists so far
     uint64_t *lists;              // [row][2 * nsplit][k], ascending, ~0 padded
@@ -217,7 +221,50 @@ struct RowList {
     }
 };
 
-template <int K>
+// leaf `s` of `levels` halvings of [0, N): its positions [lo, hi)
+__device__ __forceinline__ void leaf_range(int64_t N, int levels, int64_t s, int64_t &lo, int64_t &hi) {
+    lo = 0;
+    hi = N;
+    for (int k = levels - 1; k >= 0; k--) {
+        const int64_t m = lo + (hi - lo) / 2;
+        if ((s >> k) & 1) lo = m;
+        else hi = m;
+    }
+}
+
+// One item: query rows [row0, row1), at most BM of them, against the
+// references [ref0, ref1).
+struct Item {
+    int64_t row0, row1, ref0, ref1, split;
+    __device__ __forceinline__ int64_t tiles() const { return (ref1 - ref0 + BN - 1) / BN; }
+};
+
+template <bool LEAF>
+__device__ __forceinline__ int64_t num_items(const Params &p) {
+    return LEAF ? ((int64_t)p.leaf_blocks << p.levels) : (p.nq + BM - 1) / BM * p.nsplit;
+}
+
+// false: there is nothing to do (a leaf with fewer blocks than the largest)
+template <bool LEAF>
+__device__ __forceinline__ bool get_item(const Params &p, int64_t it, Item &I) {
+    if (LEAF) {
+        leaf_range(p.N, p.levels, it / p.leaf_blocks, I.ref0, I.ref1);
+        I.row0 = I.ref0 + it % p.leaf_blocks * BM;
+        I.row1 = I.ref1;
+        I.split = 0;
+        return I.row0 < I.ref1;
+    }
+    // split-major: CTAs of one wave share their tiles
+    const int64_t nblocks = (p.nq + BM - 1) / BM, per = ((p.N + BN - 1) / BN + p.nsplit - 1) / p.nsplit;
+    I.split = it / nblocks;
+    I.row0 = it % nblocks * BM;
+    I.row1 = p.nq;
+    I.ref0 = I.split * per * BN;
+    I.ref1 = I.ref0 + per * BN < p.N ? I.ref0 + per * BN : p.N;
+    return true;
+}
+
+template <int K, bool LEAF>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
     knn_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapAs,
                   const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapBs, Params prm) {
@@ -244,10 +291,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     __shared__ float s_half[4][2][BM];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t nblocks = (prm.nq + BM - 1) / BM;
-    const int64_t ntiles = (prm.N + BN - 1) / BN;
-    const int64_t per = (ntiles + prm.nsplit - 1) / prm.nsplit;  // tiles per split
-    const int64_t nitems = nblocks * prm.nsplit;                 // split-major: CTAs of one wave share their tiles
+    const int64_t nitems = num_items<LEAF>(prm);
+    Item I;
 
     if (threadIdx.x == 0) {
         s_err = 0;
@@ -283,17 +328,18 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             int64_t last_use[STAGES];
             for (int s = 0; s < STAGES; s++) last_use[s] = -1;
             int64_t a_loads = 0;
-            for (int64_t it = blockIdx.x; it < nitems && !*err; it += gridDim.x, nb++) {
-                const int64_t blk = it % nblocks, t0 = it / nblocks * per;
-                const int64_t t1 = t0 + per < ntiles ? t0 + per : ntiles;
+            for (int64_t it = blockIdx.x; it < nitems && !*err; it += gridDim.x) {
+                if (!get_item<LEAF>(prm, it, I)) continue;
+                const int64_t nt = I.tiles();
                 if (nb > 0 && !mbar_wait(aempty, (uint32_t)((nb - 1) & 1), err)) break;
                 mbar_expect_tx(afull, (uint32_t)Smem::a_bytes(d));
                 for (int c = 0; c < kch; c++)
-                    tma_load_2d(sA + c * BM * 128, &mapA, afull, c * BK, (int)(blk * BM));
+                    tma_load_2d(sA + c * BM * 128, &mapA, afull, c * BK, (int)I.row0);
                 tma_load_2d(sA + kch * BM * 128, &mapAs, afull, 0, 0);
                 a_loads++;
+                nb++;
                 bool ok = true;
-                for (int64_t t = t0; t < t1; t++, g++) {
+                for (int64_t t = 0; t < nt; t++, g++) {
                     const int s = (int)(g % STAGES);
                     const int64_t use = g / STAGES;
                     if (use > 0 && !mbar_wait(&empty[s], (uint32_t)((use - 1) & 1), err)) {
@@ -303,8 +349,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     uint8_t *dst = sB + s * Smem::b_bytes(d);
                     mbar_expect_tx(&full[s], (uint32_t)Smem::b_bytes(d));
                     for (int c = 0; c < kch; c++)
-                        tma_load_2d(dst + c * BN * 128, &mapB, &full[s], c * BK, (int)(t * BN));
-                    tma_load_2d(dst + kch * BN * 128, &mapBs, &full[s], 0, (int)(t * BN));
+                        tma_load_2d(dst + c * BN * 128, &mapB, &full[s], c * BK, (int)(I.ref0 + t * BN));
+                    tma_load_2d(dst + kch * BN * 128, &mapBs, &full[s], 0, (int)(I.ref0 + t * BN));
                     last_use[s] = use;
                 }
                 if (!ok) break;
@@ -321,13 +367,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             const uint32_t idesc = instr_desc(BM, BN);
             int64_t g = 0, u = 0;  // ring position, accumulator use counter
             int64_t nb = 0;
-            for (int64_t it = blockIdx.x; it < nitems && !*err; it += gridDim.x, nb++) {
-                const int64_t t0 = it / nblocks * per;
-                const int64_t t1 = t0 + per < ntiles ? t0 + per : ntiles;
+            for (int64_t it = blockIdx.x; it < nitems && !*err; it += gridDim.x) {
+                if (!get_item<LEAF>(prm, it, I)) continue;
+                const int64_t nt = I.tiles();
                 if (!mbar_wait(afull, (uint32_t)(nb & 1), err)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                nb++;
                 bool ok = true;
-                for (int64_t t = t0; t < t1; t++, g++, u++) {
+                for (int64_t t = 0; t < nt; t++, g++, u++) {
                     const int s = (int)(g % STAGES);
                     const int acc = (int)(u & 1);
                     const int64_t ause = u >> 1;
@@ -370,14 +417,15 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         const int k2 = K - k + (k + 1) / 2 - 1;  // list entry of the ceil(k/2)-th best
         int64_t u = 0;
         uint32_t n_it = 0;
-        for (int64_t it = blockIdx.x; it < nitems && !*err; it += gridDim.x, n_it++) {
+        for (int64_t it = blockIdx.x; it < nitems && !*err; it += gridDim.x) {
+            if (!get_item<LEAF>(prm, it, I)) continue;
             volatile float *my_half = &s_half[n_it & 3][half][row], *other_half = &s_half[n_it & 3][half ^ 1][row];
             *(volatile float *)&s_half[(n_it + 2) & 3][half][row] = inf;
             float own_half = inf;
-            const int64_t blk = it % nblocks, sp = it / nblocks;
-            const int64_t t0 = sp * per, t1 = t0 + per < ntiles ? t0 + per : ntiles;
-            const int64_t qrow = blk * BM + row;
-            const bool valid_row = qrow < prm.nq;
+            n_it++;
+            const int64_t nt = I.tiles();
+            const int64_t qrow = I.row0 + row;
+            const bool valid_row = qrow < I.row1;
             const uint32_t qn = valid_row ? prm.qnorm[qrow] : 0u;
             const float qnf = (float)qn;
             uint32_t *limit = prm.row_limit + (valid_row ? qrow : 0);
@@ -386,6 +434,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             int cnt = 0;                           // pending entries
             // accumulators above lim may belong to the k best; rows past the end take none
             float lim = valid_row ? -inf : inf;
+            if (valid_row && *(volatile uint32_t *)limit != 0xffffffffu)
+                lim = -0.5f * ((float)(*(volatile uint32_t *)limit + 1) - qnf);
             auto flush = [&]() {
                 const int most = __reduce_max_sync(0xffffffffu, cnt);
                 const uint32_t other = *(volatile uint32_t *)limit;  // arrives while the entries go in
@@ -405,7 +455,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     }
 #pragma unroll
                     for (int j = 0; j < 4; j++)
-                        if (c + j >= prm.N || (prm.exclude_self && c + j == qrow)) a[j] = -inf;
+                        if (c + j >= I.ref1 || (prm.exclude_self && c + j == qrow)) a[j] = -inf;
                     for (;;) {  // the best of the four first, the lower id of equal ones
                         const float b = fmaxf(fmaxf(a[0], a[1]), fmaxf(a[2], a[3]));
                         const float v = -2.0f * b;  // -inf becomes an infinite key, which goes nowhere
@@ -432,7 +482,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             };
             bool ok = true;
             int64_t next = 1;  // tiles after which the buffers are emptied next
-            for (int64_t t = t0; t < t1; t++, u++) {
+            for (int64_t t = 0; t < nt; t++, u++) {
                 const int acc = (int)(u & 1);
                 if (!mbar_wait(&tfull[acc], (uint32_t)((u >> 1) & 1), err)) {
                     ok = false;
@@ -444,9 +494,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 lim = fmaxf(lim, -0.5f * fmaxf(own_half, *other_half) - 0.5f);
                 const uint32_t tcol =
                     tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * BN + half * (BN / 2));
-                const int rid0 = (int)(t * BN) + half * (BN / 2);
+                const int rid0 = (int)(I.ref0 + t * BN) + half * (BN / 2);
                 const int kk = k + (prm.exclude_self ? 1 : 0);
-                if (t == t0 && rid0 + BN / 2 <= prm.N && kk <= 32) {
+                if (t == 0 && rid0 + BN / 2 <= I.ref1 && kk <= 32) {
                     // k distinct references (and the row itself) lie at or above the kk-th group maximum
                     float gm[32];
 #pragma unroll
@@ -474,7 +524,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     float bound = gm[0];
 #pragma unroll
                     for (int i = 1; i < 32; i++) bound = i == kk - 1 ? gm[i] : bound;
-                    if (valid_row) lim = bound - 0.5f;  // accumulators are multiples of 1/2
+                    if (valid_row) lim = fmaxf(lim, bound - 0.5f);  // accumulators are multiples of 1/2
                 }
                 auto take = [&](const uint32_t (&v)[32], int cb) __attribute__((always_inline)) {
                     float m[8];
@@ -512,20 +562,21 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 if (lane == 0) mbar_arrive(&tempty[acc]);
                 take(vb, 96);
                 // a tile adds up to 32 groups
-                if (t + 1 - t0 == next || t + 1 == t1 || __any_sync(0xffffffffu, cnt > CAP - BN / 8)) {
-                    if (t + 1 - t0 == next) next *= 2;
+                if (t + 1 == next || t + 1 == nt || __any_sync(0xffffffffu, cnt > CAP - BN / 8)) {
+                    if (t + 1 == next) next *= 2;
                     flush();
                 }
             }
             if (!ok) break;
             // this warp's list for its rows and column half; merged by a second kernel
             if (valid_row) {
-                uint64_t *dst = prm.lists + ((size_t)qrow * 2 * prm.nsplit + 2 * sp + half) * k;
+                uint64_t *dst = prm.lists + ((size_t)qrow * 2 * prm.nsplit + 2 * I.split + half) * k;
 #pragma unroll
                 for (int i = 0; i < K; i++)
                     if (i >= K - k)
                         dst[i - (K - k)] = list.key[i] < inf
-                                               ? ((uint64_t)(uint32_t)(list.key[i] + qnf) << 32) | (uint32_t)list.id[i]
+                                               ? ((uint64_t)(uint32_t)(list.key[i] + qnf) << 32) |
+                                                     (LEAF ? prm.ids[list.id[i]] : (uint32_t)list.id[i])
                                                : ~0ull;
             }
         }
@@ -570,13 +621,18 @@ __global__ void merge_lists_kernel(const uint64_t *lists, int64_t nq, int nl, in
 }
 
 // Rows as bf16 (bytes are exact), their squared norms and, for references, the
-// slab of norm pieces.  Four bytes per thread, d / 4 threads per row.
-__global__ void prep_rows_kernel(const uint8_t *X, int64_t N, int d, uint16_t *rows, uint32_t *norm, uint16_t *slab) {
+// slab of norm pieces.  Four bytes per thread, d / 4 threads per row.  With an
+// order (leaves), row r is the one of id order[r] & idmask; its id and the
+// largest key of its list so far (graph: R per id) go out too.
+__global__ void prep_rows_kernel(const uint8_t *X, int64_t N, int d, uint16_t *rows, uint32_t *norm, uint16_t *slab,
+                                 const uint64_t *order = nullptr, uint64_t idmask = 0, const uint64_t *graph = nullptr,
+                                 int R = 0, uint32_t *ids = nullptr, uint32_t *limit = nullptr) {
     const int tpr = d / 4;  // 16 or 32
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t r = i / tpr;
     const int w = (int)(i - r * tpr);
-    const uint32_t v = r < N ? __ldg((const uint32_t *)X + i) : 0u;
+    const int64_t src = r >= N ? 0 : (order ? (int64_t)(order[r] & idmask) : r);
+    const uint32_t v = r < N ? __ldg((const uint32_t *)X + src * tpr + w) : 0u;
     uint32_t s = __dp4a(v, v, 0u);
     for (int off = tpr / 2; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
     if (r >= N) return;
@@ -585,6 +641,10 @@ __global__ void prep_rows_kernel(const uint8_t *X, int64_t N, int d, uint16_t *r
     const uint32_t b2 = bf((float)((v >> 16) & 255u)), b3 = bf((float)(v >> 24));
     *(uint2 *)(rows + 4 * i) = make_uint2(b0 | (b1 << 16), b2 | (b3 << 16));
     if (w == 0) norm[r] = s;
+    if (ids && w == 1) {
+        ids[r] = (uint32_t)src;
+        limit[r] = (uint32_t)(graph[src * R + R - 1] >> 32);
+    }
     if (slab && w < 2) {
         const uint32_t hi = bf((float)(s >> 16) * 32768.0f), mid = bf((float)((s >> 8) & 255u) * 128.0f);
         const uint32_t low = bf((float)(s & 255u) * 0.5f);
@@ -661,11 +721,21 @@ int choose_split(int64_t nblocks, int64_t ntiles, int nsm, int k) {
     return best;
 }
 
-template <int K>
-cudaError_t launch_tc(unsigned grid, size_t smem, cudaStream_t s, const CUtensorMap *m, const Params &prm) {
-    const cudaError_t e = cudaFuncSetAttribute(knn_tc_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) knn_tc_kernel<K><<<grid, NUM_THREADS, smem, s>>>(m[0], m[1], m[2], m[3], prm);
+template <int K, bool LEAF>
+cudaError_t launch_k(unsigned grid, size_t smem, cudaStream_t s, const CUtensorMap *m, const Params &prm) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(knn_tc_kernel<K, LEAF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) knn_tc_kernel<K, LEAF><<<grid, NUM_THREADS, smem, s>>>(m[0], m[1], m[2], m[3], prm);
     return e;
+}
+
+// list capacity 8, 16, 24 or 32
+template <bool LEAF>
+cudaError_t launch_tc(unsigned grid, size_t smem, cudaStream_t s, const CUtensorMap *m, const Params &prm) {
+    return prm.k <= 8    ? launch_k<8, LEAF>(grid, smem, s, m, prm)
+           : prm.k <= 16 ? launch_k<16, LEAF>(grid, smem, s, m, prm)
+           : prm.k <= 24 ? launch_k<24, LEAF>(grid, smem, s, m, prm)
+                         : launch_k<32, LEAF>(grid, smem, s, m, prm);
 }
 
 }  // namespace tc
@@ -717,11 +787,8 @@ int knn_u8_tensor(const uint8_t *refs, int64_t N, const uint8_t *queries, int64_
     if (r == ANN_OK) r = make_map(&m[2], rb, N, d, BN);
     if (r == ANN_OK) r = make_map(&m[3], rslab, N, SLAB, BN);
     if (r != ANN_OK) return r;
-    Params prm{nq, N, d, k, exclude_self, nsplit, qn, limit, lists, pend, pend_col, derr};
-    cudaError_t e = k <= 8    ? launch_tc<8>(grid, smem, s, m, prm)
-                    : k <= 16 ? launch_tc<16>(grid, smem, s, m, prm)
-                    : k <= 24 ? launch_tc<24>(grid, smem, s, m, prm)
-                              : launch_tc<32>(grid, smem, s, m, prm);
+    Params prm{nq, N, d, k, exclude_self, nsplit, 0, 0, nullptr, qn, limit, lists, pend, pend_col, derr};
+    const cudaError_t e = launch_tc<false>(grid, smem, s, m, prm);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(knn_tc_kernel)");
     merge_lists_kernel<<<(unsigned)((nq * 32 + 255) / 256), 256, 0, s>>>(lists, nq, nl, k, out_ids, out_keys);
     ANN_CUDA(cudaGetLastError());
@@ -729,6 +796,51 @@ int knn_u8_tensor(const uint8_t *refs, int64_t N, const uint8_t *queries, int64_
     ANN_CUDA(cudaMemcpyAsync(&herr, derr, sizeof(int), cudaMemcpyDeviceToHost, s));
     ANN_CUDA(cudaStreamSynchronize(s));
     if (herr) return fail(ANN_ERR_TIMEOUT, "knn_tc_kernel: a pipeline wait timed out");
+    return ANN_OK;
+}
+
+// ---- the leaf step of the approximate graph ----
+
+int LeafTc::prepare(int64_t N_, int d_, int R_, int levels_, cudaStream_t s) {
+    using namespace tc;
+    N = N_, d = d_, R = R_, levels = levels_;
+    int dev = 0;
+    ANN_CUDA(cudaGetDevice(&dev));
+    ANN_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    ANN_CUDA(bufs.alloc(&lists, (size_t)N * 2 * R * 8));
+    ANN_CUDA(bufs.alloc(&rb, (size_t)N * d * 2));
+    ANN_CUDA(bufs.alloc(&rslab, (size_t)N * SLAB * 2));
+    ANN_CUDA(bufs.alloc(&qslab, (size_t)BM * SLAB * 2));
+    ANN_CUDA(bufs.alloc(&norm, (size_t)N * 4));
+    ANN_CUDA(bufs.alloc(&limit, (size_t)N * 4));
+    ANN_CUDA(bufs.alloc(&ids, (size_t)N * 4));
+    ANN_CUDA(bufs.alloc(&err, sizeof(int)));
+    ANN_CUDA(bufs.alloc(&pend, (size_t)nsm * 8 * CAP * 32 * sizeof(float4)));
+    ANN_CUDA(bufs.alloc(&pend_col, (size_t)nsm * 8 * CAP * 32 * 4));
+    ANN_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
+    query_slab_kernel<<<(BM * SLAB + 255) / 256, 256, 0, s>>>(qslab);
+    ANN_CUDA(cudaGetLastError());
+    return ANN_OK;
+}
+
+int LeafTc::round(const uint8_t *X, const uint64_t *order, uint64_t idmask, const uint64_t *graph, cudaStream_t s) {
+    using namespace tc;
+    const int tpr = d / 4;
+    prep_rows_kernel<<<(unsigned)((N * tpr + 255) / 256), 256, 0, s>>>(X, N, d, rb, norm, rslab, order, idmask, graph, R,
+                                                                       ids, limit);
+    CUtensorMap m[4];
+    int r = make_map(&m[0], rb, N, d, BM);
+    if (r == ANN_OK) r = make_map(&m[1], qslab, BM, SLAB, BM);
+    if (r == ANN_OK) r = make_map(&m[2], rb, N, d, BN);
+    if (r == ANN_OK) r = make_map(&m[3], rslab, N, SLAB, BN);
+    if (r != ANN_OK) return r;
+    const int64_t largest = (N + (1ll << levels) - 1) >> levels;
+    const int blocks = (int)((largest + BM - 1) / BM);
+    Params prm{N, N, d, R, 1, 1, levels, blocks, ids, norm, limit, lists, pend, pend_col, err};
+    const unsigned grid = (unsigned)std::min<int64_t>((int64_t)blocks << levels, nsm);
+    const cudaError_t e = launch_tc<true>(grid, smem_bytes(d), s, m, prm);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(knn_tc_kernel)");
+    ANN_CUDA(cudaGetLastError());
     return ANN_OK;
 }
 

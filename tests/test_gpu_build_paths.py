@@ -192,3 +192,20 @@ def test_adc_rerank_is_bit_exact_in_its_stated_order(ann, m, dp, ks, w, T, L, sh
         np.testing.assert_array_equal(ids[i].cpu().numpy()[:len(best)], (best & 0xffffffff).astype(np.int32))
         np.testing.assert_array_equal(keys[i].cpu().numpy().view(np.uint32)[:len(best)], (best >> 32).astype(np.uint32))
         assert np.all(ids[i].cpu().numpy()[len(best):] == -1)
+
+
+@pytest.mark.parametrize("kind,N,d,R,rounds,levels,iters", [
+    ("mix", 193, 64, 8, 1, 0, 0), ("mix", 1539, 128, 32, 2, 1, 0), ("mix", 4100, 128, 20, 3, 3, 1),
+    ("mix", 5003, 64, 16, 2, 3, 1), ("mix", 3001, 128, 1, 2, 4, 0), ("mix", 5099, 128, 25, 3, 3, 0),
+    ("equal", 1500, 64, 12, 2, 2, 1), ("few", 5000, 128, 24, 3, 3, 1), ("mix", 97, 64, 8, 1, 0, 0)])
+def test_approx_graph_leaves_on_the_tensor_cores(ann, kind, N, d, R, rounds, levels, iters):
+    X = datagen.mixture(N, N, d, 11, np.uint8)
+    if kind == "equal":      # every key equal: ids decide
+        X[:] = X[0]
+    elif kind == "few":      # many equal rows, so equal keys in one leaf and across rounds
+        X = np.ascontiguousarray(X[np.random.default_rng(1).integers(0, 30, N)])
+    dirs = datagen.rp_directions(N, rounds, levels, d)
+    gi, gk = ann.ann_build_knn_graph_approx(dev(X), R, dev(dirs), iters)
+    oi, ok = oracle.knn_graph_approx(X, R, dirs, iters)
+    np.testing.assert_array_equal(gi.cpu().numpy(), oi)
+    np.testing.assert_array_equal(gk.cpu().numpy().view(np.uint32), ok.astype(np.uint32))
