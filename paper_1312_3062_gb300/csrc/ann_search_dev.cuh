@@ -61,7 +61,7 @@ namespace ann {
 // ---------------------------------------------------------------------------
 struct WarpLayout {
     uint32_t q, tabD, rank, sc, heap, hash, rbuf, bkey, bidx, pref, nodes, cand, ckey, wref, wkey, stage, misc, stat, total;
-    uint32_t heap_cap, hash_log, bcap, ncap, gcap, glist, stage_rows, stage_stride;
+    uint32_t heap_cap, hash_log, hash_slots, bcap, ncap, gcap, glist, stage_rows, stage_stride;
     uint32_t sc_parts;  // parts whose centers are kept in rank order (all of them when split walks may run)
 };
 
@@ -108,7 +108,10 @@ __host__ __device__ inline WarpLayout make_layout(int dtype, int d, int P, int n
     uint32_t hl = 5;
     while ((1u << hl) < 2u * (uint32_t)capT) hl++;
     L.hash_log = hl;
-    L.hash = o;   o = align_up(o + (spill ? 0u : 4u * (1u << hl)), 16);  // spilling: in global scratch
+    // spilling: in global scratch, of any size (1.6 slots per entry): what the
+    // resident queries' tables take of the L2 decides how long a probe is
+    L.hash_slots = spill ? (8u * (uint32_t)capT / 5u + 71u) / 8u * 8u : 1u << hl;
+    L.hash = o;   o = align_up(o + (spill ? 0u : 4u * (1u << hl)), 16);
     L.rbuf = o;   o = align_up(o + 8u * kmax, 16);
     L.bcap = (uint32_t)bcap;
     L.bkey = o;   o = align_up(o + 8u * bcap, 16);
@@ -238,7 +241,7 @@ struct SearchArgs {
     // per-warp global scratch of the large-budget kernels, wstride bytes per
     // warp: sorted bridge windows (gcap x (2 keys + 2 values)) at 0, the
     // queue's overflow (capT entries) at spill_off, the visited set
-    // (2^hash_log slots) at hash_off
+    // (hash_slots) at hash_off
     uint8_t *gscratch;
     uint32_t gcap;
     uint64_t wstride, spill_off, hash_off;
@@ -284,15 +287,16 @@ __device__ __forceinline__ void hash_add(uint32_t *H, uint32_t log, uint32_t x) 
     }
 }
 
-// The same open-addressing table in global memory (large-budget kernels):
+// The same open-addressing table in global memory (large-budget kernels), of n
+// slots, a multiple of eight:
 // one probe step reads the aligned 32-byte sector of eight slots holding the
 // current slot, so an insertion or a lookup usually costs one memory round
 // trip.  Only the owning warp reads and writes its table; plain loads and
 // stores ordered by __syncwarp keep it coherent.  Returns as hash_find.
-__device__ __forceinline__ bool ghash_find(const uint32_t *G, uint32_t log, uint32_t x, uint32_t &slot) {
-    const uint32_t mask = (1u << log) - 1;
-    uint32_t h = hslot(x, log), seen = 0;
-    while (seen <= mask) {
+__device__ __forceinline__ uint32_t gslot(uint32_t x, uint32_t n) { return __umulhi(x * 2654435761u, n); }
+__device__ __forceinline__ bool ghash_find(const uint32_t *G, uint32_t n, uint32_t x, uint32_t &slot) {
+    uint32_t h = gslot(x, n), seen = 0;
+    while (seen <= n) {
         const uint32_t base = h & ~7u;
         const uint4 *p = (const uint4 *)(G + base);
         const uint4 a = __ldcg(p), b = __ldcg(p + 1);  // at L2: insertions by CAS bypass L1
@@ -311,14 +315,22 @@ __device__ __forceinline__ bool ghash_find(const uint32_t *G, uint32_t log, uint
             return (eq >> j) & 1u;
         }
         seen += 8 - from;
-        h = (base + 8) & mask;
+        h = base + 8 < n ? base + 8 : 0u;
     }
     slot = 0xffffffffu;
     return false;
 }
-__device__ __forceinline__ bool ghash_has(const uint32_t *G, uint32_t log, uint32_t x) {
+__device__ __forceinline__ bool ghash_has(const uint32_t *G, uint32_t n, uint32_t x) {
     uint32_t slot;
-    return ghash_find(G, log, x, slot);
+    return ghash_find(G, n, x, slot);
+}
+__device__ __forceinline__ void ghash_add(uint32_t *G, uint32_t n, uint32_t x) {
+    uint32_t h = gslot(x, n);
+    for (uint32_t i = 0; i < n; i++) {
+        const uint32_t prev = atomicCAS(&G[h], 0u, x + 1);
+        if (prev == 0 || prev == x + 1) return;
+        h = h + 1 < n ? h + 1 : 0u;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1792,7 +1804,7 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t w, uint8_
         if (!rsmall)
             for (uint32_t i = lane; i < rlen; i += 32) rbuf[i] = ((const uint64_t *)(sv + A.save_rbuf))[i];
         for (uint32_t i = lane; i < hsz; i += 32) heap[i] = ((const uint64_t *)(sv + A.save_heap))[i];
-        for (uint32_t i = 4 * lane; i < (1u << L.hash_log); i += 128)
+        for (uint32_t i = 4 * lane; i < L.hash_slots; i += 128)
             *(uint4 *)(H + i) = *(const uint4 *)(sv + A.save_hash + 4 * i);
         if (SP) {
             sp.nb = h[8];
@@ -1800,7 +1812,7 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t w, uint8_
             for (uint32_t i = lane; i < sp.nb; i += 32) sp.B[i] = ((const uint64_t *)(sv + A.save_spill))[i];
         }
     } else {
-        for (uint32_t i = 4 * lane; i < (1u << L.hash_log); i += 128) *(uint4 *)(H + i) = make_uint4(0, 0, 0, 0);
+        for (uint32_t i = 4 * lane; i < L.hash_slots; i += 128) *(uint4 *)(H + i) = make_uint4(0, 0, 0, 0);
     }
     __syncwarp();
     if (FULL && T > 0) {
@@ -1885,7 +1897,7 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t w, uint8_
                     if (!rsmall)
                         for (uint32_t i = lane; i < rlen; i += 32) ((uint64_t *)(sv + A.save_rbuf))[i] = rbuf[i];
                     for (uint32_t i = lane; i < hsz; i += 32) ((uint64_t *)(sv + A.save_heap))[i] = heap[i];
-                    for (uint32_t i = 4 * lane; i < (1u << L.hash_log); i += 128)
+                    for (uint32_t i = 4 * lane; i < L.hash_slots; i += 128)
                         *(uint4 *)(sv + A.save_hash + 4 * i) = SP ? __ldcg((const uint4 *)(H + i)) : *(const uint4 *)(H + i);
                     if (SP)
                         for (uint32_t i = lane; i < sp.nb; i += 32) ((uint64_t *)(sv + A.save_spill))[i] = sp.B[i];
@@ -1941,7 +1953,7 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t w, uint8_
                     uint32_t j = bidx_of(wstart + e / b);
                     int32_t r = __ldg(ix.brefs + (int64_t)j * b + (e % b));
                     bool keep = r >= 0 && r < ix.N &&
-                                !(SP ? ghash_has(H, L.hash_log, (uint32_t)r) : hash_has(H, L.hash_log, (uint32_t)r));
+                                !(SP ? ghash_has(H, L.hash_slots, (uint32_t)r) : hash_has(H, L.hash_log, (uint32_t)r));
                     wref[e] = keep ? r : -1;
                 }
                 __syncwarp();
@@ -1983,7 +1995,7 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t w, uint8_
         } else {
             bool isnew = false;
             if (lane < alen && x >= 0 && x < ix.N)
-                isnew = !(SP ? ghash_find(H, L.hash_log, (uint32_t)x, slot) : hash_find(H, L.hash_log, (uint32_t)x, slot));
+                isnew = !(SP ? ghash_find(H, L.hash_slots, (uint32_t)x, slot) : hash_find(H, L.hash_log, (uint32_t)x, slot));
             mask = __ballot_sync(0xffffffffu, isnew);
             int room = T - t;
             while (__popc(mask) > room) mask &= ~(1u << (31 - __clz(mask)));  // keep the first `room` in list order
@@ -2008,7 +2020,10 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t w, uint8_
                 direct = inm && slot != kNone && H[slot] == (uint32_t)x + 1;
                 __syncwarp();
             }
-            if (inm && !direct) hash_add(H, L.hash_log, (uint32_t)x);
+            if (inm && !direct) {
+                if (SP) ghash_add(H, L.hash_slots, (uint32_t)x);
+                else hash_add(H, L.hash_log, (uint32_t)x);
+            }
             uint32_t key = xkey;
             if (!have_key) {
                 // candidates share their region with the staged rows
@@ -2049,7 +2064,7 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t w, uint8_
                     uint32_t s2 = kNone;
                     bool nw = false;
                     if (lane < R && nx_row >= 0 && nx_row < ix.N)
-                        nw = !(SP ? ghash_find(H, L.hash_log, (uint32_t)nx_row, s2)
+                        nw = !(SP ? ghash_find(H, L.hash_slots, (uint32_t)nx_row, s2)
                                   : hash_find(H, L.hash_log, (uint32_t)nx_row, s2));
                     unsigned mk = __ballot_sync(0xffffffffu, nw);
                     const int room2 = T - (t + m);
@@ -2142,7 +2157,7 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t w, uint8_
 }
 
 template <int DT, bool GRP>
-__global__ void __launch_bounds__(128, 4) prologue_kernel(const __grid_constant__ SearchArgs A) {
+__global__ void __launch_bounds__(128, 5) prologue_kernel(const __grid_constant__ SearchArgs A) {
     extern __shared__ __align__(16) uint8_t smem_all[];
     const int warp = threadIdx.x >> 5;
     if (blockIdx.x == 0 && threadIdx.x < 4) A.counters[threadIdx.x] = 0;  // for the two kernels that follow
