@@ -1015,7 +1015,9 @@ __device__ uint32_t walk(const DevIndex &ix, uint8_t *smem, const WarpLayout &L,
     const uint32_t *D = (const uint32_t *)(smem + L.tabD);
     const uint8_t *rk = smem + L.rank;
     const uint8_t *sc = smem + L.sc;
-    auto sk = [&](int i) -> uint32_t { return D[(i / n) * n + sc[i]]; };  // sorted key of prefix rank
+    // sorted key of a rank of part 0 and of part 1
+    auto sk0 = [&](int r) -> uint32_t { return D[sc[r]]; };
+    auto sk1 = [&](int r) -> uint32_t { return D[n + sc[n + r]]; };
     uint32_t *pref = (uint32_t *)(smem + L.pref);
     uint32_t *nodes = (uint32_t *)(smem + L.nodes);  // 4 words per node: start, count, kpre, rpre
     uint64_t *bkey = (uint64_t *)(smem + L.bkey);
@@ -1041,7 +1043,7 @@ __device__ uint32_t walk(const DevIndex &ix, uint8_t *smem, const WarpLayout &L,
     uint32_t theta = 0, bound2 = 0;
     bool pass2 = false;
     if (can_split) {
-        const uint32_t minA = PA == 1 ? sk(0) : KeyOps<DT>::add_lo(sk(0), sk(n));
+        const uint32_t minA = PA == 1 ? sk0(0) : KeyOps<DT>::add_lo(sk0(0), sk1(0));
         if (DT == ANN_U8) {
             int64_t ex = (int64_t)hik - (int64_t)minA - (int64_t)msuf;
             if (ex < 0) ex = 0;
@@ -1071,16 +1073,16 @@ __device__ uint32_t walk(const DevIndex &ix, uint8_t *smem, const WarpLayout &L,
     for (int r0 = lane; r0 < n; r0 += 32) {
         uint32_t c1, c2 = 0;
         if (PA == 1) {
-            c1 = admit1(sk(r0)) ? 1u : 0u;
-            c2 = can_split && admit2(sk(r0)) ? 1u : 0u;
+            c1 = admit1(sk0(r0)) ? 1u : 0u;
+            c2 = can_split && admit2(sk0(r0)) ? 1u : 0u;
         } else {
-            const uint32_t a0 = sk(r0);
+            const uint32_t a0 = sk0(r0);
             auto count = [&](bool two) -> uint32_t {
-                if (!(two ? admit2(KeyOps<DT>::add_lo(a0, sk(n))) : admit1(KeyOps<DT>::add_lo(a0, sk(n))))) return 0;
+                if (!(two ? admit2(KeyOps<DT>::add_lo(a0, sk1(0))) : admit1(KeyOps<DT>::add_lo(a0, sk1(0))))) return 0;
                 int lo1 = 1, hi1 = n;  // answer in [1, n]
                 while (lo1 < hi1) {
                     const int mid = (lo1 + hi1 + 1) >> 1;
-                    const uint32_t kA = KeyOps<DT>::add_lo(a0, sk(n + mid - 1));
+                    const uint32_t kA = KeyOps<DT>::add_lo(a0, sk1(mid - 1));
                     if (two ? admit2(kA) : admit1(kA)) lo1 = mid;
                     else hi1 = mid - 1;
                 }
