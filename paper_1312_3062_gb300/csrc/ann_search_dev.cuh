@@ -726,6 +726,7 @@ __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc) {
     const uint32_t s = (uint32_t)__cvta_generic_to_shared(smem_dst);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gsrc) : "memory");
 }
+__device__ __forceinline__ void prefetch_l1(const void *p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
@@ -1840,12 +1841,10 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t w, uint8_
     // and, when stage_rows > 0, its unvisited neighbours' vectors copied into
     // shared memory by cp.async (nx_vec, nx_mask = which row entries are new,
     // cut to the budget).  The vectors and mask stay valid only while nothing
-    // else is discovered, i.e. for the very next step.  Right after every
-    // reference pop the new heap root's row is loaded speculatively (sp_row):
-    // it is the next pop unless the expansion finds a smaller key.
+    // else is discovered, i.e. for the very next step.
     constexpr uint32_t kNone = 0xffffffffu;
-    uint32_t nx_id = kNone, sp_id = kNone;
-    int32_t nx_row = -1, sp_row = -1;
+    uint32_t nx_id = kNone;
+    int32_t nx_row = -1;
     bool nx_vec = false, cp_out = false;
     unsigned nx_mask = 0;
     uint32_t nx_slot = kNone;  // where this lane's staged id goes in the visited set
@@ -1923,20 +1922,15 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t w, uint8_
                 x = nx_row;
                 staged = nx_vec;
                 count(3);
-            } else if (p == sp_id) {
-                x = sp_row;
-                count(3);
             } else if (lane < R) {
                 x = __ldg(ix.G + (int64_t)p * R + lane);
             }
             nx_id = kNone;
             nx_vec = false;
-            if (hsz > 0) {
-                sp_id = (uint32_t)heap[0];
-                sp_row = lane < R ? __ldg(ix.G + (int64_t)sp_id * R + lane) : -1;
-            } else {
-                sp_id = kNone;
-            }
+            // The new root's row (one line or two) is needed at the end of the
+            // step unless the expansion finds a smaller key.  A prefetch and
+            // not a load: the next __syncwarp waits for every load issued.
+            if (hsz > 0 && lane < 2) prefetch_l1(ix.G + (int64_t)(uint32_t)heap[0] * R + lane * (R - 1));
             count(1);
         } else {
             // the bridge window reuses the staging region
@@ -2056,7 +2050,7 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t w, uint8_
             if ((uint32_t)(ntop >> 32) <= bkey_now) {
                 const uint32_t nid = (uint32_t)ntop;
                 if (nid != nx_id) {
-                    nx_row = nid == sp_id ? sp_row : (lane < R ? __ldg(ix.G + (int64_t)nid * R + lane) : -1);
+                    nx_row = lane < R ? __ldg(ix.G + (int64_t)nid * R + lane) : -1;
                     nx_id = nid;
                 }
                 // vectors only when the next step is certainly this pop (no
