@@ -171,7 +171,7 @@ static int plan_launch(const SearchArgs &base, int capT, const int32_t *list, co
     A.capT = capT;
     // bridge batch: budgets below the windowed kernels pop few bridges
     A.bcap = win ? 128 : 64;
-    A.bstore = A.bcap + (int)kFirstBridges;
+    A.bstore = 2 * A.bcap;
     A.list = list;
     A.list_count = list_count;
     A.list_len = list_len;

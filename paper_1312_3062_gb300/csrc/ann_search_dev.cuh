@@ -17,8 +17,7 @@
 // its rate is set by how many queries an SM holds.  With the walk in the same
 // kernel a query took 168 registers and, for its tables and walk lists, about
 // 8 KB more shared memory: 12 queries per SM.  Most queries need only the
-// first batch (21 of 10,000 are suspended at T = 371 on SIFT-shaped rows); the
-// loop alone holds 16 to 24 queries per SM.  And the resuming kernel, which
+// first batch; the loop alone holds 16 to 24 queries per SM.  And the resuming kernel, which
 // only sees queries that pop many bridges, sorts whole windows of bridges at
 // every budget.  One kernel against three, 10,000 queries, 1M SIFT-shaped rows:
 // T = 371 1.31 -> 0.92 ms, T = 2392 8.06 -> 6.06 ms; 2,000 GIST-shaped queries
@@ -190,11 +189,16 @@ __host__ __device__ inline WarpLayout main_layout(int dtype, int d, int capT, in
     return L;
 }
 
-// The prologue walks until it has this many bridges, the first of which is
-// popped at once: a query that pops no other one never needs another walk (on
-// the SIFT-shaped sets a walk's first window holds one or two bridges, and the
-// next bridge's key must be known while the first one's references are popped).
-constexpr uint32_t kFirstBridges = 1;
+// The prologue walks to the first bridge and, in launches of kReachFrom queries
+// or more, on to kReach times the distance of that bridge's nearest reference
+// (or a full batch): references up to about that distance are popped, and a
+// query that needs a walk beyond has to be resumed, one whole query's length
+// after the batch.  Suspended of 10,000 queries with kReach = 0 / 1 / 1.3: T =
+// 371 21 / 4 / 0, T = 2392 503 / 22 / 1; times 0.88 / 0.81 / 0.79 and 5.75 /
+// 5.72 / 4.98 ms (1.6: the same, 2: 0.86 ms).  Few queries gain nothing by it: a
+// served burst over an index of 4,096 bridges took 4.06 instead of 2.23 ms.
+constexpr float kReach = 1.3f;
+constexpr int64_t kReachFrom = 512;
 
 // What the prologue leaves for a query, and what a suspended one needs to go on.
 struct QRec {
@@ -1690,7 +1694,9 @@ __device__ void prologue_one(const SearchArgs &A, uint8_t *smem, int64_t w) {
     const uint64_t *bkey = (const uint64_t *)(smem + L.bkey);
     const uint32_t *bidx = (const uint32_t *)(smem + L.bidx), *misc = (const uint32_t *)(smem + L.misc);
     uint32_t bcnt = 0;
-    while (bcnt < kFirstBridges && !ws.exhausted && !cap_err) {
+    uint32_t reach = 0;  // walk at least to this key
+    while ((bcnt == 0 || ((uint32_t)(ws.lo >> 32) < reach && bcnt < L.bcap)) && !ws.exhausted && !cap_err) {
+        const bool begin = bcnt == 0;
         const uint32_t c = refill<DT, GRP>(ix, smem, L, ws, cap_err);
         for (uint32_t i = lane; i < c; i += 32) {
             A.bkeys[at * A.bstore + bcnt + i] = bkey[i];
@@ -1698,6 +1704,20 @@ __device__ void prologue_one(const SearchArgs &A, uint8_t *smem, int64_t w) {
         }
         bcnt += c;
         __syncwarp();
+        if (begin && c > 0 && A.chunk >= kReachFrom) {
+            // the nearest reference of the first bridge: the search pops
+            // references up to about its distance
+            uint32_t *cand = (uint32_t *)(smem + L.pref), *ckey = cand + 32;
+            const int32_t r = lane < ix.b ? __ldg(ix.brefs + (int64_t)bidx[0] * ix.b + lane) : -1;
+            const unsigned have = __ballot_sync(0xffffffffu, r >= 0 && r < ix.N);
+            if ((have >> lane) & 1u) cand[__popc(have & ((1u << lane) - 1))] = (uint32_t)r;
+            __syncwarp();
+            const int m = __popc(have);
+            cand_distances<DT>(ix.X, ix.d * (DT == ANN_U8 ? 1 : 4), smem + L.q, cand, m, ckey);
+            const uint32_t d = __reduce_min_sync(0xffffffffu, lane < m ? ckey[lane] : 0xffffffffu);
+            if (m) reach = DT == ANN_U8 ? (uint32_t)((float)d * kReach) : __float_as_uint(__uint_as_float(d) * kReach);
+            __syncwarp();
+        }
     }
     if (lane == 0) {
         QRec r;
