@@ -143,15 +143,16 @@ struct LaunchCfg {
     uint64_t main_stride, res_stride;  // global scratch per warp (large budgets)
     uint64_t main_spill, main_hash, res_spill, res_hash;
     bool win, wide;
+    bool whole;                        // resume_kernel alone
     int64_t total, chunk;              // queries, and queries per pass over the three kernels
     // offsets into the workspace
     size_t o_rec, o_bk, o_bi, o_susp, o_save, o_scratch, bytes;
 };
 
 // A pass holds the records and first bridge batches of at most kChunk queries
-// (0.9 to 1.7 KB each), and states of suspended ones up to kSaveBytes; queries
+// (4.7 KB each), and states of suspended ones up to kSaveBytes; queries
 // that find no room there start again when they are resumed.
-static const int64_t kChunk = 65536;
+static const int64_t kChunk = 32768;
 static const size_t kSaveBytes = (size_t)256 << 20;
 
 static int plan_launch(const SearchArgs &base, int capT, const int32_t *list, const int32_t *list_count,
@@ -171,7 +172,7 @@ static int plan_launch(const SearchArgs &base, int capT, const int32_t *list, co
     A.capT = capT;
     // bridge batch: budgets below the windowed kernels pop few bridges
     A.bcap = win ? 128 : 64;
-    A.bstore = 2 * A.bcap;
+    A.bstore = (int)(kFirstEnough + kFirstCap);
     A.list = list;
     A.list_count = list_count;
     A.list_len = list_len;
@@ -179,7 +180,7 @@ static int plan_launch(const SearchArgs &base, int capT, const int32_t *list, co
     cfg.wide = list_len > (int64_t)g_num_sms * kMainWarps * kMainCtas;
     cfg.total = list_len;
     cfg.chunk = std::min(list_len, kChunk);
-    cfg.pro.L = prologue_layout(ix.dtype, ix.d, ix.P, ix.n, ix.PA, A.bcap, grouped, win);
+    cfg.pro.L = prologue_layout(ix.dtype, ix.d, ix.P, ix.n, ix.PA, (int)kFirstCap, grouped, win);
     cfg.main.L = main_layout(ix.dtype, ix.d, capT, A.kmax, ix.b, ix.R, tn.stage, win, (uint32_t)tn.spill_heap);
     cfg.res.L = make_layout(ix.dtype, ix.d, ix.P, ix.n, ix.PA, capT, A.kmax, A.bcap, ix.b, ix.R, true, grouped, win,
                             (uint32_t)tn.spill_heap, true);
@@ -195,6 +196,12 @@ static int plan_launch(const SearchArgs &base, int capT, const int32_t *list, co
             return resume_occupancy(ix, win, smem, threads, blocks);
         });
     if (r != ANN_OK) return r;
+    // One kernel while it holds all queries at once: the others only pay when
+    // there are more queries than that, and a suspended one would come after
+    // all that were not.  SIFT-shaped rows, P = 2 x n = 64, 600 queries, T = 64 /
+    // 256 / 2048: three kernels 232 / 298 / 1406 us, one 207 / 252 / 1186 us.
+    cfg.whole = cfg.res.warps >= list_len;
+    A.whole = cfg.whole;
     auto al = [](uint64_t x) { return (x + 255) & ~(uint64_t)255; };
     // a sorted window serves many batches of bridges
     const uint32_t gcap = (uint32_t)std::min(8192, std::max(1024, 2 * capT));
@@ -241,6 +248,7 @@ static int do_launch(LaunchCfg &cfg, uint8_t *ws, cudaStream_t stream, int first
     A.gscratch = ws + cfg.o_scratch;
     A.chunk = cfg.chunk;
     for (A.base = 0; A.base < cfg.total; A.base += cfg.chunk) {
+        if (cfg.whole) first = last = 2;
         if (first <= 0) {
             const Shape &s = cfg.pro;
             A.L = s.L;
@@ -497,6 +505,10 @@ static int autotune(PlanCache *pc, const SearchArgs &A, int64_t nq, const int32_
         LaunchCfg c0;
         rc = plan_launch(A, capT, list, nullptr, hc[bkt], c0, &cands[0]);
         if (rc != ANN_OK) break;
+        if (c0.whole) {  // the main loop's shape is not used
+            pc->tuned[{bucket_cap(bkt), A.kmax}] = cands[0];
+            continue;
+        }
         const int64_t ntune = std::min<int64_t>(std::min<int64_t>(hc[bkt], kChunk), 4 * (int64_t)c0.main.warps);
         float best_ms = 0.f;
         int best = -1;

@@ -11,7 +11,8 @@
 //                    T.  A query that has popped its whole first batch of
 //                    bridges is suspended.
 //   resume_kernel    suspended queries: tables and sort again, then the same
-//                    loop with further walks, to the end.
+//                    loop with further walks, to the end.  Alone, from the
+//                    start, when all queries of a launch fit it at once.
 // Why three: the loop is a chain of dependent steps (a warp collective takes
 // 30 to 40 cycles here, and a popped reference about 20 of them in a row), so
 // its rate is set by how many queries an SM holds.  With the walk in the same
@@ -189,16 +190,16 @@ __host__ __device__ inline WarpLayout main_layout(int dtype, int d, int capT, in
     return L;
 }
 
-// The prologue walks to the first bridge and, in launches of kReachFrom queries
-// or more, on to kReach times the distance of that bridge's nearest reference
-// (or a full batch): references up to about that distance are popped, and a
-// query that needs a walk beyond has to be resumed, one whole query's length
-// after the batch.  Suspended of 10,000 queries with kReach = 0 / 1 / 1.3: T =
-// 371 21 / 4 / 0, T = 2392 503 / 22 / 1; times 0.88 / 0.81 / 0.79 and 5.75 /
-// 5.72 / 4.98 ms (1.6: the same, 2: 0.86 ms).  Few queries gain nothing by it: a
-// served burst over an index of 4,096 bridges took 4.06 instead of 2.23 ms.
+// The prologue walks to the first bridge and on to kReach times the distance of
+// that bridge's nearest reference (or kFirstEnough bridges): references up to
+// about that distance are popped, and a query that needs a walk beyond has to be
+// resumed, one whole query's length after the batch.  Suspended of 10,000
+// queries with kReach = 0 / 1 / 1.3: T = 371 21 / 4 / 0, T = 2392 503 / 22 / 1;
+// times 0.88 / 0.81 / 0.79 and 5.75 / 5.72 / 4.98 ms (1.6: the same, 2: 0.86 ms).
 constexpr float kReach = 1.3f;
-constexpr int64_t kReachFrom = 512;
+// bridges that end the prologue's walks whatever their reach, and the most one
+// walk of it returns
+constexpr uint32_t kFirstEnough = 128, kFirstCap = 256;
 
 // What the prologue leaves for a query, and what a suspended one needs to go on.
 struct QRec {
@@ -226,6 +227,7 @@ struct SearchArgs {
     const int32_t *list;
     const int32_t *list_count;
     int64_t list_len;
+    bool whole;  // resume_kernel: every query of the selection, from the start
     // this launch: queries base .. base + chunk of the selection
     int64_t base, chunk;
     // [0] main loop's ticket, [1] suspended queries, [2] resume ticket, [3] slots taken
@@ -1666,6 +1668,13 @@ __device__ __forceinline__ bool query_args(const SearchArgs &A, int64_t qi, int 
     return k >= 0 && k <= A.kmax && T >= 0 && T <= A.capT;
 }
 
+// the first window's width: narrow ones walk fewest leaves (measured on the
+// SIFT-shaped 1M index); float32: about 0.8% relative, in bit space
+template <int DT>
+__device__ __forceinline__ uint32_t first_width(uint32_t kmin) {
+    return DT == ANN_U8 ? max(1u, kmin >> 8) : 1u << 16;
+}
+
 // steps 1 to 3 for one query: its record and first batch of bridges
 template <int DT, bool GRP>
 __device__ void prologue_one(const SearchArgs &A, uint8_t *smem, int64_t w) {
@@ -1684,18 +1693,13 @@ __device__ void prologue_one(const SearchArgs &A, uint8_t *smem, int64_t w) {
     ws.gpos = ws.gcnt = 0;
     ws.gbuf = 0;
     build_tables<DT>(A, smem, ws.kmin, ws.kmaxall);
-    if (DT == ANN_U8) {
-        uint32_t w0 = ws.kmin >> 8;  // measured on the SIFT-shaped 1M index: narrow first windows walk fewest leaves
-        ws.width = w0 < 1 ? 1 : w0;
-    } else {
-        ws.width = 1u << 16;  // about 0.8% relative in float32 bit space
-    }
+    ws.width = first_width<DT>(ws.kmin);
     bool cap_err = false;
     const uint64_t *bkey = (const uint64_t *)(smem + L.bkey);
     const uint32_t *bidx = (const uint32_t *)(smem + L.bidx), *misc = (const uint32_t *)(smem + L.misc);
     uint32_t bcnt = 0;
     uint32_t reach = 0;  // walk at least to this key
-    while ((bcnt == 0 || ((uint32_t)(ws.lo >> 32) < reach && bcnt < L.bcap)) && !ws.exhausted && !cap_err) {
+    while ((bcnt == 0 || ((uint32_t)(ws.lo >> 32) < reach && bcnt < kFirstEnough)) && !ws.exhausted && !cap_err) {
         const bool begin = bcnt == 0;
         const uint32_t c = refill<DT, GRP>(ix, smem, L, ws, cap_err);
         for (uint32_t i = lane; i < c; i += 32) {
@@ -1704,7 +1708,7 @@ __device__ void prologue_one(const SearchArgs &A, uint8_t *smem, int64_t w) {
         }
         bcnt += c;
         __syncwarp();
-        if (begin && c > 0 && A.chunk >= kReachFrom) {
+        if (begin && c > 0) {
             // the nearest reference of the first bridge: the search pops
             // references up to about its distance
             uint32_t *cand = (uint32_t *)(smem + L.pref), *ckey = cand + 32;
@@ -1778,7 +1782,12 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t w, uint8_
     load_query<DT>(A, qb, qi);
     uint32_t flags = 2, bcnt = 0, slot0 = 0xffffffffu;
     WalkState ws;
-    if (T > 0) {
+    const bool whole = FULL && A.whole;
+    if (FULL && whole) {
+        flags = 1u | (ix.M == 0 ? 2u : 0u);
+        ws.lo = 0;
+        ws.width = 0;  // set from the smallest key
+    } else if (T > 0) {
         const QRec *r = A.rec + at;
         flags = r->flags;
         bcnt = r->bcnt;
@@ -1840,7 +1849,8 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t w, uint8_
     __syncwarp();
     if (FULL && T > 0) {
         build_tables<DT>(A, smem, ws.kmin, ws.kmaxall);
-        if (lane == 0) {
+        if (whole) ws.width = first_width<DT>(ws.kmin);
+        if (lane == 0 && !whole) {
             misc[8] = A.rec[at].walks;
             misc[9] = A.rec[at].nodes;
             misc[10] = A.rec[at].leaves;
@@ -2206,6 +2216,12 @@ __global__ void __launch_bounds__(192, 2) resume_kernel(const __grid_constant__ 
     const int warp = threadIdx.x >> 5;
     uint8_t *smem = smem_all + (size_t)warp * A.L.total;
     uint8_t *wscratch = A.gscratch + ((size_t)blockIdx.x * (blockDim.x >> 5) + warp) * A.wstride;
+    if (A.whole) {  // no more queries than warps
+        const int64_t end = query_end(A), step = (int64_t)gridDim.x * (blockDim.x >> 5);
+        for (int64_t w = A.base + (int64_t)blockIdx.x * (blockDim.x >> 5) + warp; w < end; w += step)
+            search_one<DT, SP, GRP, true>(A, smem, w, wscratch);
+        return;
+    }
     const int32_t count = A.counters[1];
     for (;;) {
         int32_t i = 0;

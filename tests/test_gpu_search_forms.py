@@ -1,0 +1,66 @@
+"""Launches of more queries than one kernel holds run as prologue, main loop and
+resumed queries; smaller ones as one kernel from start to end.  Both give the
+same results, counters included, and the oracle's on a sample."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+import oracle  # noqa: E402
+from paper_1312_3062_gb300 import datagen  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def ann():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_1312_3062_gb300 import _build
+    _build.build()
+    from paper_1312_3062_gb300 import ann as mod
+    return mod
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+# the last uint8 cases pop more bridges than the prologue leaves: nearly every query is resumed, with budgets of 8192
+# more of them than there are slots for their states
+@pytest.mark.parametrize("dtype,N,d,comps,P,n,R,T,k,mode", [
+    (np.uint8, 4000, 128, 4, 4, 16, 16, 300, 10, 0), (np.uint8, 4000, 64, 40, 2, 64, 20, 900, 100, 1),
+    (np.uint8, 4000, 128, 40, 4, 24, 10, 1024, 33, 0), (np.float32, 3000, 96, 20, 3, 20, 20, 700, 10, 1),
+    (np.float32, 3000, 512, 20, 4, 12, 16, 1500, 1, 0), (np.uint8, 9000, 32, 3, 2, 128, 8, 8192, 10, 0),
+    (np.uint8, 2500, 48, 60, 3, 33, 32, 31, 5, 1)])
+def test_many_queries_equal_few_and_the_oracle(ann, dtype, N, d, comps, P, n, R, T, k, mode):
+    rng = np.random.default_rng(N + T)
+    X = datagen.mixture(T, N, d, comps, dtype)
+    nq = 6000
+    Q = datagen.mixture(T, nq, d, comps, dtype)
+    C = ann.ann_train_centers(dev(X), P, n, 2, rng.permutation(N)[:n])
+    G, _ = ann.ann_build_knn_graph(dev(X), R)
+    ix = ann.Index.create(dev(X), G, C, t=100, b=5)
+
+    def search(q, m):
+        st = torch.zeros((len(q), ann.ANN_NSTATS), dtype=torch.int64, device="cuda")
+        ids, keys, status = ann.ann_search_batch(ix, q, k, T, mode=m, out_stats=st)
+        torch.cuda.synchronize()
+        cols = [ann.STAT_NAMES.index(s) for s in ("discovered", "ref_pops", "bridge_pops", "max_q")]
+        return [x.cpu().numpy() for x in (ids, keys, status, st[:, cols])]
+
+    Qd = dev(Q)
+    many = search(Qd, mode)
+    few = [np.concatenate(x) for x in zip(*(search(Qd[i:i + 150].contiguous(), 0) for i in range(0, nq, 150)))]
+    for a, b in zip(many, few):
+        np.testing.assert_array_equal(a, b)
+    sel = rng.permutation(nq)[:24]
+    ids, refs = ix.bridges()
+    bg = dict(bridges=ids, offsets=np.concatenate([[0], np.cumsum((refs >= 0).sum(1))]).astype(np.int64),
+              refs=refs[refs >= 0])
+    wi, wk, ws = oracle.search(X, G.cpu().numpy(), C.cpu().numpy(), bg, Q[sel], k, T, kmax=k, nthreads=8)
+    np.testing.assert_array_equal(many[0][sel], wi)
+    np.testing.assert_array_equal(many[3][sel, 1], ws["ref_pops"])
+    np.testing.assert_array_equal(many[3][sel, 2], ws["nonempty_bridge_pops"])
