@@ -258,13 +258,15 @@ enum {
  * names one bridge and halving a window always separates them: the check
  * only guards against a corrupted index).
  * out_stats (optional) int64[nq*ANN_NSTATS].
- * mode ANN_MODE_PLAIN: one kernel launch for this batch on `stream`, sized
- * for the largest budget (per-query T costs one device max and a host sync).
+ * mode ANN_MODE_PLAIN: the kernels of this batch on `stream`, sized for the
+ * largest budget (per-query T costs one device max and a host sync), with a
+ * stream-ordered workspace of about 5 KB per query (passes of 32768 queries)
+ * and up to 256 MB for the states of queries that pop many bridges.
  * mode ANN_MODE_PERSISTENT: queries are bucketed by budget (128 * 2^i) and
- * each bucket is run by a kernel sized for it, pulling queries from a device
- * ticket or taking fixed shares; the sequence is captured once per (index,
- * pointers, sizes, stream) into a CUDA graph and replayed (at most 32 plans
- * per index, least recently used evicted after its stream finished).  The
+ * each bucket is run by kernels sized for it, the buckets side by side; the
+ * sequence is captured once per (index, pointers, sizes, stream) into a CUDA
+ * graph and replayed (at most 32 plans and 16 GB of workspaces per index,
+ * least recently used evicted after its stream finished).  The
  * first call that meets a (budget bucket, kmax) measures candidate launch
  * shapes on the batch itself and keeps the fastest for the index; that call
  * synchronizes `stream` and runs the batch a few times.

@@ -37,10 +37,9 @@ static int device_props() {
     return ANN_OK;
 }
 
-// Budgets from this size on use per-warp global scratch: sorted bridge windows
-// (one walk then serves many batches, which pays off when queries pop many
-// bridges), and the queue's overflow and the visited set, so the shared-memory
-// slice of a query no longer grows with its budget.
+// Budgets from this size on, in launches with more queries than fit otherwise,
+// keep the queue's overflow and the visited set in per-warp global scratch, so
+// the shared-memory slice of a query no longer grows with its budget.
 static const int kWindowedFromT = 1024;
 
 // Launch shape of the main loop for a budget bucket.
@@ -157,6 +156,8 @@ static const size_t kSaveBytes = (size_t)256 << 20;
 
 static int plan_launch(const SearchArgs &base, int capT, const int32_t *list, const int32_t *list_count,
                        int64_t list_len, LaunchCfg &cfg, const Tune *tune = nullptr) {
+    // the buckets of a batch (their counts are on the device) share its queries
+    const size_t save_bytes = list_count ? kSaveBytes / 4 : kSaveBytes;
     SearchArgs A = base;
     const DevIndex &ix = A.ix;
     const bool grouped = ix.ngroups > 0;
@@ -221,7 +222,7 @@ static int plan_launch(const SearchArgs &base, int capT, const int32_t *list, co
     A.save_hash = align_up(A.save_heap + 8u * cfg.main.L.heap_cap, 16);
     A.save_spill = A.save_hash + 4u * cfg.main.L.hash_slots;
     A.save_stride = al(A.save_spill + (win ? 8ull * (uint64_t)capT : 0ull));
-    A.nslots = (uint32_t)std::min<int64_t>(cfg.chunk, (int64_t)(kSaveBytes / A.save_stride));
+    A.nslots = (uint32_t)std::min<int64_t>(cfg.chunk, (int64_t)(save_bytes / A.save_stride));
     size_t o = 256;  // counters
     cfg.o_rec = o;   o = al(o + sizeof(QRec) * (size_t)cfg.chunk);
     cfg.o_bk = o;    o = al(o + 8 * (size_t)A.bstore * cfg.chunk);
@@ -324,11 +325,13 @@ struct Plan {
     cudaGraphExec_t exec = nullptr;
     int32_t *scratch = nullptr;   // counts[kBuckets], then lists[kBuckets*nq]
     uint8_t *wscratch = nullptr;  // the buckets' workspaces, one after another
+    size_t bytes = 0;             // of the workspaces
     uint64_t last_use = 0;        // for evicting the least recently used plan
 };
 
-// plans kept per index; the least recently used one goes beyond this
-static const size_t kMaxPlans = 32;
+// plans kept per index, and bytes of their workspaces; beyond either the least
+// recently used ones go
+static const size_t kMaxPlans = 32, kMaxPlanBytes = (size_t)16 << 30;
 
 struct PlanKey {
     const void *queries;
@@ -407,8 +410,15 @@ struct ForkSet {
     }
 };
 
+// one bucket's launch: the whole batch in order, or (per-query T) its list
+static int plan_bucket(const SearchArgs &A, int64_t nq, const int32_t *T, int32_t *scratch, int bkt, int capT,
+                       LaunchCfg &cfg, const Tune *tn) {
+    if (!T) return plan_launch(A, capT, nullptr, nullptr, nq, cfg, tn);
+    return plan_launch(A, capT, scratch + kBuckets + (int64_t)bkt * nq, scratch + bkt, nq, cfg, tn);
+}
+
 static int record_persistent(const PlanCache *pc, const SearchArgs &A, int64_t nq, const int32_t *T, int32_t T_all,
-                             int32_t *scratch, uint8_t *wscratch, cudaStream_t s, ForkSet &fs) {
+                             int32_t *scratch, uint8_t *wscratch, size_t wbytes, cudaStream_t s, ForkSet &fs) {
     int32_t *counts = scratch, *lists = scratch + kBuckets;
     if (T) {
         ANN_CUDA(cudaMemsetAsync(counts, 0, sizeof(int32_t) * kBuckets, s));
@@ -422,11 +432,15 @@ static int record_persistent(const PlanCache *pc, const SearchArgs &A, int64_t n
         const int capT = sized_for(bkt, T, T_all);
         const Tune *tn = tuned_for(pc, bucket_cap(bkt), A.kmax);
         LaunchCfg cfg;
-        rc = T ? plan_launch(A, capT, lists + (int64_t)bkt * nq, counts + bkt, nq, cfg, tn)
-               : plan_launch(A, capT, nullptr, nullptr, nq, cfg, tn);
+        rc = plan_bucket(A, nq, T, scratch, bkt, capT, cfg, tn);
         if (rc != ANN_OK) break;
+        if (cfg.bytes > wbytes) {
+            rc = fail(ANN_ERR_CAPACITY, "search workspace smaller than its kernels need");
+            break;
+        }
         uint8_t *ws = wscratch;
         wscratch += cfg.bytes;
+        wbytes -= cfg.bytes;
         if (b0 == b1) {
             rc = do_launch(cfg, ws, s);
             continue;
@@ -636,8 +650,8 @@ extern "C" int ann_search_batch(const ann_index *index, const void *queries, int
     PlanKey key{queries, nq, k, T, k_all, T_all, kmax, out_ids, out_keys, out_status, out_stats, s};
     std::lock_guard<std::mutex> g(pc->mu);
     auto it = pc->plans.find(key);
-    if (it == pc->plans.end() && pc->plans.size() >= kMaxPlans) {
-        // evict the least recently used plan once its stream has finished with it
+    // evict the least recently used plan once its stream has finished with it
+    auto evict = [pc]() -> int {
         auto old = pc->plans.begin();
         for (auto jt = pc->plans.begin(); jt != pc->plans.end(); ++jt)
             if (jt->second.last_use < old->second.last_use) old = jt;
@@ -646,6 +660,11 @@ extern "C" int ann_search_batch(const ann_index *index, const void *queries, int
         cudaFree(old->second.scratch);
         if (old->second.wscratch) cudaFree(old->second.wscratch);
         pc->plans.erase(old);
+        return ANN_OK;
+    };
+    if (it == pc->plans.end() && pc->plans.size() >= kMaxPlans) {
+        const int er = evict();
+        if (er != ANN_OK) return er;
     }
     if (it == pc->plans.end()) {
         Plan p;
@@ -661,7 +680,7 @@ extern "C" int ann_search_batch(const ann_index *index, const void *queries, int
             bucket_range(T, T_all, b0, b1);
             for (int bkt = b0; bkt <= b1; bkt++) {
                 LaunchCfg cfg;
-                r = plan_launch(A, sized_for(bkt, T, T_all), nullptr, p.scratch, nq, cfg,
+                r = plan_bucket(A, nq, T, p.scratch, bkt, sized_for(bkt, T, T_all), cfg,
                                 tuned_for(pc, bucket_cap(bkt), kmax));
                 if (r != ANN_OK) {
                     cudaFree(p.scratch);
@@ -669,6 +688,19 @@ extern "C" int ann_search_batch(const ann_index *index, const void *queries, int
                 }
                 need += cfg.bytes;
             }
+            size_t held = need;
+            for (auto &kv : pc->plans) held += kv.second.bytes;
+            while (held > kMaxPlanBytes && !pc->plans.empty()) {
+                size_t left = need;
+                r = evict();
+                if (r != ANN_OK) {
+                    cudaFree(p.scratch);
+                    return r;
+                }
+                for (auto &kv : pc->plans) left += kv.second.bytes;
+                held = left;
+            }
+            p.bytes = need;
             if (need) {
                 cudaError_t ae = cudaMalloc(&p.wscratch, need);
                 if (ae != cudaSuccess) {
@@ -697,7 +729,7 @@ extern "C" int ann_search_batch(const ann_index *index, const void *queries, int
         int rr;
         {
             ForkSet fs;
-            rr = record_persistent(pc, A, nq, T, T_all, p.scratch, p.wscratch, cap, fs);
+            rr = record_persistent(pc, A, nq, T, T_all, p.scratch, p.wscratch, p.bytes, cap, fs);
             ce = cudaStreamEndCapture(cap, &graph);
         }
         cudaStreamDestroy(cap);

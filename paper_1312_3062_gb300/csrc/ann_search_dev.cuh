@@ -14,16 +14,17 @@
 //                    loop with further walks, to the end.  Alone, from the
 //                    start, when all queries of a launch fit it at once.
 // Why three: the loop is a chain of dependent steps (a warp collective takes
-// 30 to 40 cycles here, and a popped reference about 20 of them in a row), so
-// its rate is set by how many queries an SM holds.  With the walk in the same
-// kernel a query took 168 registers and, for its tables and walk lists, about
-// 8 KB more shared memory: 12 queries per SM.  Most queries need only the
-// first batch; the loop alone holds 16 to 24 queries per SM.  And the resuming kernel, which
-// only sees queries that pop many bridges, sorts whole windows of bridges at
-// every budget.  One kernel against three, 10,000 queries, 1M SIFT-shaped rows:
-// T = 371 1.31 -> 0.92 ms, T = 2392 8.06 -> 6.06 ms; 2,000 GIST-shaped queries
-// with budgets of 64 to 8192 57.8 -> 29.6 ms; 1,792 queries of T = 339 among
-// 170-point components, which pop bridges all the time, 4.78 -> 2.56 ms.
+// 30 to 40 cycles here, and a popped reference about 20 of them in a row, some
+// 690 instructions in all), so its rate is set by how many queries an SM holds.
+// With the walk in the same kernel a query took 168 registers and, for its
+// tables and walk lists, about 8 KB more shared memory: 12 queries per SM.
+// Most queries need only the first batch; the loop alone holds 16 to 24
+// queries per SM.  And the resuming kernel, which only sees queries that pop
+// many bridges, sorts whole windows of bridges at every budget.  One kernel
+// against three, 10,000 queries, 1M SIFT-shaped rows: T = 371 1.31 -> 0.79 ms,
+// T = 2392 8.06 -> 4.97 ms; 2,000 GIST-shaped queries with budgets of 64 to
+// 8192 57.8 -> 25.7 ms; 1,792 queries of T = 339 among 170-point components,
+// which pop bridges all the time, 4.78 -> 2.39 ms.
 // Bridge vectors are produced in the order of the multi-sequence algorithm
 // (Sec. 3.3): ascending (bridge key, rank tuple).  A popped bridge vector
 // with an empty list discovers nothing and only makes the next one current,
@@ -79,8 +80,9 @@ constexpr uint32_t kSpillHeap = 512;
 // registers hold.  16 queries per SM (128 registers) is the faster shape until
 // the queries of a launch fill it; large-budget uint8 launches beyond that take
 // 24 (80 registers, with spills).  10,000 queries, SIFT-shaped 1M rows,
-// 16 / 20 / 24 per SM: T = 371 0.91 / 0.92 / 1.02 ms, T = 2392 6.67 / 6.43 /
-// 6.13 ms; the served burst, about 1000 queries per budget, 5.24 / 5.52 / 5.83 ms.
+// 16 / 20 / 24 per SM, when the choice was made: T = 371 0.91 / 0.92 / 1.02 ms,
+// T = 2392 6.67 / 6.43 / 6.13 ms; the served burst, about 1000 queries per
+// budget, 5.24 / 5.52 / 5.83 ms.
 constexpr int kMainWarps = 4, kMainCtas = 4, kMainCtasWide = 6;
 
 __host__ __device__ inline uint32_t align_up(uint32_t x, uint32_t a) { return (x + a - 1) / a * a; }
@@ -200,6 +202,8 @@ constexpr float kReach = 1.3f;
 // bridges that end the prologue's walks whatever their reach, and the most one
 // walk of it returns
 constexpr uint32_t kFirstEnough = 128, kFirstCap = 256;
+// a walk trims its buffer, of 32 entries or more, until a step's 64 leaves fit in
+static_assert(kFirstCap >= 64 + 32, "the prologue's walks could not trim their buffer");
 
 // What the prologue leaves for a query, and what a suspended one needs to go on.
 struct QRec {
@@ -1027,8 +1031,6 @@ __device__ uint32_t walk(const DevIndex &ix, uint8_t *smem, const WarpLayout &L,
     auto sk1 = [&](int r) -> uint32_t { return D[n + sc[n + r]]; };
     uint32_t *pref = (uint32_t *)(smem + L.pref);
     uint32_t *nodes = (uint32_t *)(smem + L.nodes);  // 4 words per node: start, count, kpre, rpre
-    uint64_t *bkey = (uint64_t *)(smem + L.bkey);
-    uint32_t *bidx = (uint32_t *)(smem + L.bidx);
     uint32_t *cnt = (uint32_t *)(smem + L.misc);
     uint32_t hik = (uint32_t)(hi >> 32);  // lowered, with hi, when the output buffer fills
     const bool pow2n = (n & (n - 1)) == 0;
@@ -2172,9 +2174,9 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t w, uint8_
             o[ANN_STAT_DISCOVERED] = t;
             o[ANN_STAT_REF_POPS] = stat[1];
             o[ANN_STAT_BRIDGE_POPS] = stat[2];
-            o[ANN_STAT_WALKS] = FULL ? misc[8] : (T > 0 ? r->walks : 0u);
-            o[ANN_STAT_WALK_NODES] = FULL ? misc[9] : (T > 0 ? r->nodes : 0u);
-            o[ANN_STAT_WALK_LEAVES] = FULL ? misc[10] : (T > 0 ? r->leaves : 0u);
+            o[ANN_STAT_WALKS] = T == 0 ? 0u : (FULL ? misc[8] : r->walks);
+            o[ANN_STAT_WALK_NODES] = T == 0 ? 0u : (FULL ? misc[9] : r->nodes);
+            o[ANN_STAT_WALK_LEAVES] = T == 0 ? 0u : (FULL ? misc[10] : r->leaves);
             o[ANN_STAT_MAX_Q] = stat[0];
             o[ANN_STAT_PRELOADED] = stat[3];
         }
