@@ -234,7 +234,15 @@ extern "C" int ann_exact_knn(const void *refs, int64_t N, const void *queries, i
     ANN_ARG(!exclude_self || (queries == refs && nq == N), "exclude_self needs queries == refs");
     if (nq == 0) return ANN_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    if (dtype == ANN_U8 && (d == 64 || d == 128))
+    // the tensor-core form reads its error word back, which a capturing stream
+    // does not allow: there the largest k of the widest rows keeps the SIMT form
+    bool tensor = dtype == ANN_U8 && (d == 64 || d == 128);
+    if (tensor && d == 128 && k > 30) {
+        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+        ANN_CUDA(cudaStreamIsCapturing(s, &st));
+        tensor = st == cudaStreamCaptureStatusNone;
+    }
+    if (tensor)
         return knn_u8_tensor((const uint8_t *)refs, N, (const uint8_t *)queries, nq, d, k, exclude_self, out_ids,
                              (uint32_t *)out_keys, s);
     // float32 at scale: candidates from tensor-core dot products, exact keys

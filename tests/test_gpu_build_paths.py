@@ -209,3 +209,31 @@ def test_approx_graph_leaves_on_the_tensor_cores(ann, kind, N, d, R, rounds, lev
     oi, ok = oracle.knn_graph_approx(X, R, dirs, iters)
     np.testing.assert_array_equal(gi.cpu().numpy(), oi)
     np.testing.assert_array_equal(gk.cpu().numpy().view(np.uint32), ok.astype(np.uint32))
+
+
+def test_widest_lists_and_plain_searches_can_be_captured(ann):
+    """Calls that wait for nothing on the host: recorded into a CUDA graph once, replayed on other queries."""
+    N, nq, d, k, T = 3000, 5000, 128, 32, 200
+    X, Q = datagen.mixture(3, N, d, 9, np.uint8), datagen.mixture(4, nq, d, 9, np.uint8)
+    Xd, Qd = dev(X), dev(Q)
+    G, _ = ann.ann_build_knn_graph(Xd, 10)
+    C = ann.ann_train_centers(Xd, 4, 16, 2, np.arange(16))
+    ix = ann.Index.create(Xd, G, C, t=100, b=5)
+
+    def calls(q):
+        s = torch.cuda.current_stream()
+        return (*ann.ann_exact_knn(Xd, q[:200], k, stream=s), *ann.ann_search_batch(ix, q, 10, T, mode=0, stream=s)[:2],
+                *ann.ann_search_batch(ix, q[:64], 10, 2000, mode=0, stream=s)[:2])
+
+    want = [x.cpu().numpy() for x in calls(Qd)]
+    buf = torch.zeros_like(Qd)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, capture_error_mode="thread_local"):
+        got = calls(buf)
+    for _ in range(2):
+        buf.copy_(Qd)
+        g.replay()
+        for a, b in zip(got, want):
+            np.testing.assert_array_equal(a.cpu().numpy(), b)
+            a.zero_()
