@@ -6,10 +6,10 @@
 //  1. `rounds` random partitions.  Positions [0, N) are halved recursively
 //     `levels` times (segment [lo, hi) -> [lo, m), [m, hi), m = lo + (hi-lo)/2).
 //     At level l every segment s reorders its members ascending by
-//     (<u, x>, id), u = dirs[round][2^l - 1 + s].  One level is one radix sort
-//     of the 64-bit keys (segment, <u, x> + bias, id) over all N positions:
-//     a segment's members occupy the same positions before and after, so a
-//     global sort is the per-segment sort.
+//     (<u, x>, id), u = dirs[round][2^l - 1 + s].  One level is one stable radix
+//     sort of the 64-bit keys (segment, <u, x> + bias, id), taken in id order,
+//     by the bits above the id: a segment's members occupy the same positions
+//     before and after, so a global sort is the per-segment sort.
 //  2. Leaf step: every point is offered every other leaf member.  For d 64 and
 //     128 and leaves of more than leaf_tc_from(R) points the keys come from the
 //     tensor cores (LeafTc: rows gathered in leaf order, 128 of a leaf against
@@ -91,7 +91,10 @@ __device__ __forceinline__ void offer_lanes(uint64_t &mine, uint64_t v, int R) {
     }
 }
 
-// key of position p at level l: (segment, <u, x> + bias, id)
+// key of position p at level l: (segment, <u, x> + bias, id), written at its id:
+// a stable sort of the array in id order needs to look at the bits above the id
+// only, 4 digits instead of 7 (a 1M x 128 build, 4 rounds of 10 levels, 25.0 ->
+// 22.8 ms; the scattered 8-byte writes stay in L2)
 __global__ void rp_key_kernel(const uint8_t *__restrict__ X, int64_t N, int d, const int8_t *__restrict__ u_level,
                               int l, const uint64_t *__restrict__ prev, uint64_t idmask, int id_bits, int seg_shift,
                               int bias, uint64_t *__restrict__ out) {
@@ -120,11 +123,11 @@ __global__ void rp_key_kernel(const uint8_t *__restrict__ X, int64_t N, int d, c
         acc = dp4a_us(xv.z, uv.z, acc);
         acc = dp4a_us(xv.w, uv.w, acc);
     }
-    out[p] = (s << seg_shift) | ((uint64_t)(uint32_t)(acc + bias) << id_bits) | id;
+    out[id] = (s << seg_shift) | ((uint64_t)(uint32_t)(acc + bias) << id_bits) | id;
 }
 
-// key of position p after the last level: (leaf, id), so that ids ascend inside
-// a leaf (the tensor-core leaf step breaks ties by position)
+// key of position p after the last level: (leaf, id), written at its id, so that
+// ids ascend inside a leaf (the tensor-core leaf step breaks ties by position)
 __global__ void rp_leaf_key_kernel(int64_t N, int levels, const uint64_t *__restrict__ prev, uint64_t idmask, int id_bits,
                                    uint64_t *__restrict__ out) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -138,7 +141,8 @@ __global__ void rp_leaf_key_kernel(int64_t N, int levels, const uint64_t *__rest
         hi = right ? hi : m;
         s = 2 * s + right;
     }
-    out[p] = (s << id_bits) | (prev ? prev[p] & idmask : (uint64_t)p);
+    const uint64_t id = prev ? prev[p] & idmask : (uint64_t)p;
+    out[id] = (s << id_bits) | id;
 }
 
 // offer the two lists of every position to the row of its id
@@ -467,7 +471,7 @@ extern "C" int ann_build_knn_graph_approx(const void *data, int dtype, int64_t N
             AP_CUDA(cudaGetLastError());
             if (l > 0) keys.selector ^= 1;
             size_t tb = temp_bytes;
-            AP_CUDA(cub::DeviceRadixSort::SortKeys(temp, tb, keys, (int)N, 0, l + proj_bits + id_bits, s));
+            AP_CUDA(cub::DeviceRadixSort::SortKeys(temp, tb, keys, (int)N, id_bits, l + proj_bits + id_bits, s));
         }
         const uint64_t *sorted = levels > 0 ? keys.Current() : nullptr;
         if (tensor) {
@@ -478,7 +482,7 @@ extern "C" int ann_build_knn_graph_approx(const void *data, int dtype, int64_t N
             if (levels > 0) {
                 keys.selector ^= 1;
                 size_t tb = temp_bytes;
-                AP_CUDA(cub::DeviceRadixSort::SortKeys(temp, tb, keys, (int)N, 0, levels + id_bits, s));
+                AP_CUDA(cub::DeviceRadixSort::SortKeys(temp, tb, keys, (int)N, id_bits, levels + id_bits, s));
             }
             sorted = keys.Current();
             const int rc = tc.round((const uint8_t *)data, sorted, idmask, ra, s);
