@@ -370,49 +370,56 @@ __global__ void km_store_kernel(int total, int dtype, const double *C, void *out
 // no particular order: the sort by bridge that follows does not need one.
 // Issue-bound (the part tables and sorts, then one pass over the candidates).
 // Sorting all candidates by one warp in shared memory took 210 ms for
-// 200,000 x 128 bytes, P = 4, n = 256, t = 100; this takes 5.3 ms.
-constexpr int BG_WARPS = 4;
+// 200,000 x 128 bytes, P = 4, n = 256, t = 100; this takes about 5 ms.  Tables
+// stay in registers and only the ranks below t are kept, so that an SM holds
+// more warps; whole index build with buffers of 1024 / 768 / 512 / 384: 10.1 /
+// 9.9 / 9.5 / 9.7 ms.
+constexpr int BG_WARPS = 4, BG_CAP = 512;
 
-// sort part p's keys by (key, center id) in registers: the keys in rank order
-// over the unsorted ones, the center id at each rank
-template <int EPL, bool PACK>
-__device__ __forceinline__ void bg_sort_part(uint32_t *key, uint8_t *cid, int n) {
+// part p's table and its sort by (key, center id), both in registers: the ns
+// smallest keys and their center ids, in rank order
+template <int DT, int EPL, bool PACK>
+__device__ __forceinline__ void bg_sort_part(const uint8_t *qb, const void *C, int p, int n, int dp, bool wide,
+                                             uint32_t *key, uint8_t *cid, int ns) {
     const int lane = lane_id();
     using K = typename std::conditional<PACK, uint32_t, uint64_t>::type;
     constexpr int SH = PACK ? 8 : 32;
     K v[EPL];
 #pragma unroll
     for (int s = 0; s < EPL; s++) {
-        const int c = lane * EPL + s;
-        v[s] = c < n ? (((K)key[c]) << SH) | (K)c : ~(K)0;
+        const int c = s * 32 + lane;
+        v[s] = ~(K)0;
+        if (c < n)
+            v[s] = ((K)(wide ? part_key_wide<DT>(qb, C, p, c, n, dp) : part_key_lane<DT>(qb, C, p, c, n, dp)) << SH) |
+                   (K)c;
     }
     reg_bitonic_sort_t<EPL, K>(v);
-    __syncwarp();
 #pragma unroll
     for (int s = 0; s < EPL; s++) {
         const int r = lane * EPL + s;
-        if (r < n) {
+        if (r < ns) {
             key[r] = (uint32_t)(v[s] >> SH);
             cid[r] = (uint8_t)(v[s] & (PACK ? 0xffu : 0xffffffffu));
         }
     }
 }
 
-template <bool PACK>
-__device__ __forceinline__ void bg_sort_any(uint32_t *key, uint8_t *cid, int n) {
-    if (n <= 32) bg_sort_part<1, PACK>(key, cid, n);
-    else if (n <= 64) bg_sort_part<2, PACK>(key, cid, n);
-    else if (n <= 128) bg_sort_part<4, PACK>(key, cid, n);
-    else bg_sort_part<8, PACK>(key, cid, n);
+template <int DT, bool PACK>
+__device__ __forceinline__ void bg_sort_any(const uint8_t *qb, const void *C, int p, int n, int dp, bool wide,
+                                            uint32_t *key, uint8_t *cid, int ns) {
+    if (n <= 32) bg_sort_part<DT, 1, PACK>(qb, C, p, n, dp, wide, key, cid, ns);
+    else if (n <= 64) bg_sort_part<DT, 2, PACK>(qb, C, p, n, dp, wide, key, cid, ns);
+    else if (n <= 128) bg_sort_part<DT, 4, PACK>(qb, C, p, n, dp, wide, key, cid, ns);
+    else bg_sort_part<DT, 8, PACK>(qb, C, p, n, dp, wide, key, cid, ns);
 }
 
 // (key, ranks) of a packed rank tuple; ~0 when its key is above limk
 // (float32: a bound taken downwards first, the exact sum only below it)
 template <int DT>
-__device__ __forceinline__ uint64_t bg_composite(const uint32_t *skey, int P, int n, uint32_t rr, uint32_t limk) {
+__device__ __forceinline__ uint64_t bg_composite(const uint32_t *skey, int P, int ns, uint32_t rr, uint32_t limk) {
     uint32_t s[kMaxP];
 #pragma unroll
-    for (int p = 0; p < kMaxP; p++) s[p] = p < P ? skey[p * n + ((rr >> (8 * (P - 1 - p))) & 255u)] : 0u;
+    for (int p = 0; p < kMaxP; p++) s[p] = p < P ? skey[p * ns + ((rr >> (8 * (P - 1 - p))) & 255u)] : 0u;
     if (DT == ANN_F32) {
         const uint32_t low = KeyOps<DT>::add_lo(KeyOps<DT>::add_lo(s[0], s[1]), KeyOps<DT>::add_lo(s[2], s[3]));
         if (__uint_as_float(low) > __uint_as_float(limk)) return ~0ull;  // a NaN goes on to the exact sum
@@ -423,14 +430,14 @@ __device__ __forceinline__ uint64_t bg_composite(const uint32_t *skey, int P, in
 
 // how many candidates lie at or below lim; the first cap of them to buf
 template <int DT>
-__device__ __forceinline__ uint32_t bg_collect(const uint32_t *skey, int P, int n, const uint32_t *cands, int ncand,
+__device__ __forceinline__ uint32_t bg_collect(const uint32_t *skey, int P, int ns, const uint32_t *cands, int ncand,
                                                uint64_t lim, uint64_t *buf, uint32_t cap) {
     const int lane = lane_id();
     uint32_t c = 0;
     for (int i0 = 0; i0 < ncand; i0 += 32) {
         const int i = i0 + lane;
         const uint64_t v =
-            i < ncand ? bg_composite<DT>(skey, P, n, __ldg(cands + i), (uint32_t)(lim >> 32)) : ~0ull;
+            i < ncand ? bg_composite<DT>(skey, P, ns, __ldg(cands + i), (uint32_t)(lim >> 32)) : ~0ull;
         const bool in = v <= lim && i < ncand && v != ~0ull;
         const unsigned m = __ballot_sync(0xffffffffu, in);
         const uint32_t pos = c + __popc(m & ((1u << lane) - 1));
@@ -445,7 +452,7 @@ template <int DT>
 __global__ void __launch_bounds__(32 * BG_WARPS) bg_topt_kernel(const void *X, int64_t N, int d, int P, int n,
                                                                 const void *C, const uint32_t *cands, int ncand,
                                                                 const uint32_t *bound, int nbound, uint32_t cap,
-                                                                int t_eff, uint32_t slice, uint64_t *out_keys,
+                                                                int t_eff, uint32_t slice, int kb, uint64_t *out_keys,
                                                                 uint32_t *out_vals) {
     extern __shared__ __align__(16) uint8_t smem_all[];
     const int warp = threadIdx.x >> 5, lane = lane_id();
@@ -453,8 +460,9 @@ __global__ void __launch_bounds__(32 * BG_WARPS) bg_topt_kernel(const void *X, i
     const int vb = d * (DT == ANN_U8 ? 1 : 4);
     uint8_t *qb = sm;
     uint32_t *skey = (uint32_t *)(sm + align_up16(vb));
-    uint8_t *scid = (uint8_t *)(skey + P * n);
-    uint64_t *buf = (uint64_t *)(sm + align_up16(align_up16(vb) + 5 * P * n));
+    const int ns = min(n, t_eff);  // a rank of t or more is in no candidate
+    uint8_t *scid = (uint8_t *)(skey + P * ns);
+    uint64_t *buf = (uint64_t *)(sm + align_up16(align_up16(vb) + 5 * P * ns));
     const int dp = d / P;
     const bool wide = dp % (DT == ANN_U8 ? 16 : 4) == 0;
     const bool pack = DT == ANN_U8 && (uint64_t)dp * 65025u < (1u << 24);
@@ -464,27 +472,22 @@ __global__ void __launch_bounds__(32 * BG_WARPS) bg_topt_kernel(const void *X, i
         const uint4 *src = (const uint4 *)((const uint8_t *)X + i * (int64_t)vb);
         for (int c = lane; c < (vb >> 4); c += 32) ((uint4 *)qb)[c] = __ldg(src + c);
         __syncwarp();
-        for (int idx = lane; idx < P * n; idx += 32) {
-            const int p = idx / n, c = idx - p * n;
-            skey[idx] = wide ? part_key_wide<DT>(qb, C, p, c, n, dp) : part_key_lane<DT>(qb, C, p, c, n, dp);
-        }
-        __syncwarp();
         for (int p = 0; p < P; p++) {
-            if (pack) bg_sort_any<true>(skey + p * n, scid + p * n, n);
-            else bg_sort_any<false>(skey + p * n, scid + p * n, n);
+            if (pack) bg_sort_any<DT, true>(qb, C, p, n, dp, wide, skey + p * ns, scid + p * ns, ns);
+            else bg_sort_any<DT, false>(qb, C, p, n, dp, wide, skey + p * ns, scid + p * ns, ns);
         }
         __syncwarp();
         uint32_t limk = 0xffffffffu;
         for (int c = lane; c < nbound; c += 32)
-            limk = min(limk, (uint32_t)(bg_composite<DT>(skey, P, n, __ldg(bound + c), limk) >> 32));
+            limk = min(limk, (uint32_t)(bg_composite<DT>(skey, P, ns, __ldg(bound + c), limk) >> 32));
         limk = __reduce_min_sync(0xffffffffu, limk);
         // at or below hi there are at least t candidates, at or below lo fewer
-        uint64_t lo = bg_composite<DT>(skey, P, n, 0u, 0xffffffffu), hi = ((uint64_t)limk << 32) | 0xffffffffull;
+        uint64_t lo = bg_composite<DT>(skey, P, ns, 0u, 0xffffffffu), hi = ((uint64_t)limk << 32) | 0xffffffffull;
         if (t_eff == 1) hi = lo;
-        uint32_t c = bg_collect<DT>(skey, P, n, cands, ncand, hi, buf, cap);
+        uint32_t c = bg_collect<DT>(skey, P, ns, cands, ncand, hi, buf, cap);
         while (c > cap) {
             const uint64_t mid = lo + (hi - lo) / 2;
-            const uint32_t cm = bg_collect<DT>(skey, P, n, cands, ncand, mid, buf, cap);
+            const uint32_t cm = bg_collect<DT>(skey, P, ns, cands, ncand, mid, buf, cap);
             if (cm < (uint32_t)t_eff) {
                 lo = mid;
             } else {
@@ -515,9 +518,9 @@ __global__ void __launch_bounds__(32 * BG_WARPS) bg_topt_kernel(const void *X, i
             if (keep) {
                 const uint32_t rr = (uint32_t)v;
                 uint64_t bid = 0;
-                for (int p = 0; p < P; p++) bid = bid * (uint64_t)n + scid[p * n + ((rr >> (8 * (P - 1 - p))) & 255u)];
+                for (int p = 0; p < P; p++) bid = bid * (uint64_t)n + scid[p * ns + ((rr >> (8 * (P - 1 - p))) & 255u)];
                 const int64_t o = i * t_eff + at + __popc(m & ((1u << lane) - 1));
-                out_keys[o] = (bid << 32) | (v >> 32);
+                out_keys[o] = (bid << kb) | (v >> 32);
                 out_vals[o] = (uint32_t)i;
             }
             at += __popc(m);
@@ -526,27 +529,27 @@ __global__ void __launch_bounds__(32 * BG_WARPS) bg_topt_kernel(const void *X, i
     }
 }
 
-__global__ void bg_keep_kernel(const uint64_t *keys, int64_t m, int b, uint8_t *flags) {
+__global__ void bg_keep_kernel(const uint64_t *keys, int64_t m, int kb, int b, uint8_t *flags) {
     int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= m) return;
-    flags[j] = (j < b) || ((keys[j - b] >> 32) != (keys[j] >> 32));
+    flags[j] = (j < b) || ((keys[j - b] >> kb) != (keys[j] >> kb));
 }
 
-__global__ void bg_first_kernel(const uint64_t *keys, int64_t m, uint32_t *first) {
+__global__ void bg_first_kernel(const uint64_t *keys, int64_t m, int kb, uint32_t *first) {
     int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= m) return;
-    first[j] = (j == 0 || (keys[j - 1] >> 32) != (keys[j] >> 32)) ? 1u : 0u;
+    first[j] = (j == 0 || (keys[j - 1] >> kb) != (keys[j] >> kb)) ? 1u : 0u;
 }
 
 // seg = inclusive scan of first, minus one
 __global__ void bg_scatter_kernel(const uint64_t *keys, const uint32_t *vals, const uint32_t *seg_incl,
-                                  const uint32_t *first, int64_t m, uint32_t *ustart, uint32_t *ubid) {
+                                  const uint32_t *first, int64_t m, int kb, uint32_t *ustart, uint32_t *ubid) {
     int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= m) return;
     if (first[j]) {
         uint32_t s = seg_incl[j] - 1;
         ustart[s] = (uint32_t)j;
-        ubid[s] = (uint32_t)(keys[j] >> 32);
+        ubid[s] = (uint32_t)(keys[j] >> kb);
     }
 }
 
@@ -660,6 +663,14 @@ __global__ void mark_refs_kernel(const int32_t *brefs, int64_t total, uint8_t *m
     if (r >= 0) mark[r] = 1;
 }
 
+__global__ void count_marks_kernel(const uint8_t *mark, int64_t N, unsigned long long *sum) {
+    unsigned c = 0;
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < N; j += (int64_t)gridDim.x * blockDim.x)
+        c += mark[j];
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (lane_id() == 0 && c) atomicAdd(sum, (unsigned long long)c);
+}
+
 static inline unsigned nblk(int64_t m, int t = 256) { return (unsigned)((m + t - 1) / t); }
 
 static int64_t ipow(int64_t a, int e) {
@@ -674,12 +685,15 @@ static int count_bridged(ann_index *ix, cudaStream_t s) {
     ANN_CUDA(cudaMemsetAsync(mark.p, 0, ix->dev.N, s));
     int64_t tot = ix->dev.M * ix->dev.b;
     if (tot > 0) mark_refs_kernel<<<nblk(tot), 256, 0, s>>>(ix->brefs, tot, mark.p);
-    std::vector<uint8_t> h(ix->dev.N);
-    ANN_CUDA(cudaMemcpyAsync(h.data(), mark.p, ix->dev.N, cudaMemcpyDeviceToHost, s));
+    unsigned long long *sum = nullptr, c = 0;
+    AsyncBufs bufs(s);
+    ANN_CUDA(bufs.alloc(&sum, sizeof(*sum)));
+    ANN_CUDA(cudaMemsetAsync(sum, 0, sizeof(*sum), s));
+    count_marks_kernel<<<(unsigned)std::min<int64_t>(nblk(ix->dev.N), 1024), 256, 0, s>>>(mark.p, ix->dev.N, sum);
+    ANN_CUDA(cudaGetLastError());
+    ANN_CUDA(cudaMemcpyAsync(&c, sum, sizeof(c), cudaMemcpyDeviceToHost, s));
     ANN_CUDA(cudaStreamSynchronize(s));
-    int64_t c = 0;
-    for (uint8_t v : h) c += v;
-    ix->bridged_refs = c;
+    ix->bridged_refs = (int64_t)c;
     return ANN_OK;
 }
 
@@ -845,12 +859,21 @@ static int build_bridges_gpu(ann_index *ix, cudaStream_t s) {
     // room for every candidate in shared memory is still what limits t
     if (align_up16(align_up16(align_up16(vb) + 9 * P * n) + 8 * std::max(Lc, Lp)) > (uint32_t)optin)
         return fail(ANN_ERR_CAPACITY, "bridge builder: per-reference state exceeds shared memory");
-    const uint32_t cap = Lc <= 1024 ? (uint32_t)Lc : (uint32_t)std::max(1024, t_eff);
-    const uint32_t slice = align_up16(align_up16(align_up16(vb) + 5 * P * n) + 8 * cap);
+    const uint32_t cap = Lc <= BG_CAP ? (uint32_t)Lc : (uint32_t)std::max(BG_CAP, t_eff);
+    const uint32_t slice = align_up16(align_up16(align_up16(vb) + 5 * P * std::min(n, t_eff)) + 8 * cap);
     const int warps = std::max(1, std::min(BG_WARPS, (int)(optin / slice)));
     size_t smem = (size_t)warps * slice;
     ANN_CUDA(cudaFuncSetAttribute(bg_topt_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int64_t m = N * t_eff;
+    // sort keys: the bridge id over the kb bits that a key can have; the radix
+    // sort reads no digits above (55 bits of 64 for 128 bytes, n^P = 2^32)
+    auto bits = [](uint64_t v) {
+        int c = 0;
+        for (; v; v >>= 1) c++;
+        return c;
+    };
+    const int kb = DT == ANN_U8 ? std::min(32, bits((uint64_t)65025 * dv.d)) : 32;
+    const int kend = kb + std::max(1, bits((uint64_t)nb - 1));
     DBuf<uint64_t> k0, k1;
     DBuf<uint32_t> v0, v1;
     ANN_CUDA_ALLOC(k0, m);
@@ -860,27 +883,34 @@ static int build_bridges_gpu(ann_index *ix, cudaStream_t s) {
     int64_t blocks = std::min<int64_t>((N + warps - 1) / warps, (int64_t)nsm * 16);
     if (N > 0)
         bg_topt_kernel<DT><<<(unsigned)blocks, warps * 32, smem, s>>>(dv.X, N, dv.d, P, n, dv.C, dcand.p, ncand,
-                                                                       dbound.p, nbound, cap, t_eff, slice, k0.p,
+                                                                       dbound.p, nbound, cap, t_eff, slice, kb, k0.p,
                                                                        v0.p);
     ANN_CUDA(cudaGetLastError());
     // sort by (bridge id, key); stable, so references stay in id order within ties
+    // (both buffers are given to the sort: no third copy in its workspace)
+    cub::DoubleBuffer<uint64_t> kd(k0.p, k1.p);
+    cub::DoubleBuffer<uint32_t> vd(v0.p, v1.p);
     size_t tb = 0;
-    ANN_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, tb, k0.p, k1.p, v0.p, v1.p, m, 0, 64, s));
+    ANN_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, tb, kd, vd, m, 0, kend, s));
     DBuf<uint8_t> temp;
     ANN_CUDA_ALLOC(temp, tb);
-    ANN_CUDA(cub::DeviceRadixSort::SortPairs(temp.p, tb, k0.p, k1.p, v0.p, v1.p, m, 0, 64, s));
+    ANN_CUDA(cub::DeviceRadixSort::SortPairs(temp.p, tb, kd, vd, m, 0, kend, s));
+    const uint64_t *ks = kd.Current();
+    const uint32_t *vs = vd.Current();
+    uint64_t *kk = kd.Alternate();
+    uint32_t *vk = vd.Alternate();
     // keep the first b of every bridge
     DBuf<uint8_t> flags;
     ANN_CUDA_ALLOC(flags, m);
-    if (m > 0) bg_keep_kernel<<<nblk(m), 256, 0, s>>>(k1.p, m, b, flags.p);
+    if (m > 0) bg_keep_kernel<<<nblk(m), 256, 0, s>>>(ks, m, kb, b, flags.p);
     DBuf<int64_t> nsel;
     ANN_CUDA_ALLOC(nsel, 1);
     size_t tb2 = 0;
-    ANN_CUDA(cub::DeviceSelect::Flagged(nullptr, tb2, k1.p, flags.p, k0.p, nsel.p, m, s));
+    ANN_CUDA(cub::DeviceSelect::Flagged(nullptr, tb2, ks, flags.p, kk, nsel.p, m, s));
     DBuf<uint8_t> temp2;
     ANN_CUDA_ALLOC(temp2, tb2);
-    ANN_CUDA(cub::DeviceSelect::Flagged(temp2.p, tb2, k1.p, flags.p, k0.p, nsel.p, m, s));
-    ANN_CUDA(cub::DeviceSelect::Flagged(temp2.p, tb2, v1.p, flags.p, v0.p, nsel.p, m, s));
+    ANN_CUDA(cub::DeviceSelect::Flagged(temp2.p, tb2, ks, flags.p, kk, nsel.p, m, s));
+    ANN_CUDA(cub::DeviceSelect::Flagged(temp2.p, tb2, vs, flags.p, vk, nsel.p, m, s));
     int64_t mk = 0;
     ANN_CUDA(cudaMemcpyAsync(&mk, nsel.p, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     ANN_CUDA(cudaStreamSynchronize(s));
@@ -888,7 +918,7 @@ static int build_bridges_gpu(ann_index *ix, cudaStream_t s) {
     DBuf<uint32_t> first, seg;
     ANN_CUDA_ALLOC(first, mk);
     ANN_CUDA_ALLOC(seg, mk);
-    if (mk > 0) bg_first_kernel<<<nblk(mk), 256, 0, s>>>(k0.p, mk, first.p);
+    if (mk > 0) bg_first_kernel<<<nblk(mk), 256, 0, s>>>(kk, mk, kb, first.p);
     size_t tb3 = 0;
     ANN_CUDA(cub::DeviceScan::InclusiveSum(nullptr, tb3, first.p, seg.p, mk, s));
     DBuf<uint8_t> temp3;
@@ -905,8 +935,8 @@ static int build_bridges_gpu(ann_index *ix, cudaStream_t s) {
     ANN_CUDA_ALLOC(brefs, M * b);
     ANN_CUDA(cudaMemsetAsync(brefs.p, 0xff, sizeof(int32_t) * std::max<int64_t>(M * b, 1), s));
     if (mk > 0) {
-        bg_scatter_kernel<<<nblk(mk), 256, 0, s>>>(k0.p, v0.p, seg.p, first.p, mk, ustart.p, ubid.p);
-        bg_refs_kernel<<<nblk(mk), 256, 0, s>>>(v0.p, seg.p, ustart.p, mk, b, brefs.p);
+        bg_scatter_kernel<<<nblk(mk), 256, 0, s>>>(kk, vk, seg.p, first.p, mk, kb, ustart.p, ubid.p);
+        bg_refs_kernel<<<nblk(mk), 256, 0, s>>>(vk, seg.p, ustart.p, mk, b, brefs.p);
     }
     ANN_CUDA(cudaGetLastError());
     ix->brefs = brefs.release();
