@@ -138,6 +138,9 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
 // fma, done as 32 + 32 two-wide instructions.  TX = 16 when n > 64, else 8
 // (a tile of 128 centers would be mostly padding).
 constexpr int KM_KC = 32;  // dimensions per shared-memory pass
+// rows per pass of an iteration: many waves of the assignment (64 ms a pass for
+// 128 bytes, n = 256), and sums of 255s still fit 32 bits
+constexpr int64_t KM_SLICE = 1 << 24;
 template <int DT, int TX>
 __global__ void __launch_bounds__(256) km_assign_kernel(const void *X, int64_t N, int d, int dp, int n,
                                                         const float *cneg, const float *cmax, int32_t *assign,
@@ -279,7 +282,7 @@ __global__ void km_exact_kernel(const void *X, int64_t N, int d, int dp, int n, 
 
 // Cluster sums of the bytes of every part: integers, so any order gives the
 // same sums.  A CTA adds its share of the rows in shared memory (32 bits hold
-// 2^24 rows of 255; neighbouring lanes add to neighbouring dimensions, without
+// a slice's 2^24 rows of 255; neighbouring lanes add to neighbouring dimensions, without
 // bank conflicts) and flushes what is not zero.  One global atomic per element
 // took 190 us per part of 200,000 x 32 bytes.
 __global__ void km_accumulate_u8_kernel(const uint8_t *X, int64_t N, int d, int dp, int n, const int32_t *assign,
@@ -1040,8 +1043,11 @@ extern "C" int ann_train_centers(const void *train, int dtype, int64_t ntrain, i
     DBuf<float> cneg, cmax;
     ANN_CUDA_ALLOC(C, total);
     ANN_CUDA_ALLOC(rows, n);
-    ANN_CUDA_ALLOC(assign, (size_t)P * ntrain);
-    ANN_CUDA_ALLOC(amb, (size_t)P * ntrain);
+    // The rows are taken KM_SLICE at a time: the lists of assignments and of
+    // rows left to fp64 stay small and hold 32-bit rows, whatever ntrain is.
+    const int64_t slice = std::min(ntrain, KM_SLICE);
+    ANN_CUDA_ALLOC(assign, (size_t)P * slice);
+    ANN_CUDA_ALLOC(amb, (size_t)P * slice);
     ANN_CUDA_ALLOC(namb, P);
     ANN_CUDA_ALLOC(isums, total);
     ANN_CUDA_ALLOC(fsums, total);
@@ -1051,50 +1057,58 @@ extern "C" int ann_train_centers(const void *train, int dtype, int64_t ntrain, i
     ANN_CUDA(cudaMemcpyAsync(rows.p, init_rows, 8 * n, cudaMemcpyHostToDevice, s));
     if (dtype == ANN_U8) km_init_kernel<ANN_U8><<<nblk(total), 256, 0, s>>>(train, d, dp, P, n, rows.p, C.p);
     else km_init_kernel<ANN_F32><<<nblk(total), 256, 0, s>>>(train, d, dp, P, n, rows.p, C.p);
-    // all parts of an iteration in one launch (blockIdx.y); byte sums in shared
-    // memory where a CTA's copy of a part's sums fits and cannot overflow
+    // all parts of a slice in one launch (blockIdx.y); byte sums in shared memory
+    // where a CTA's copy of a part's sums fits (a slice's cannot overflow)
     const int BM = n > 64 ? 128 : 256;
-    const dim3 grid_a((unsigned)((ntrain + BM - 1) / BM), (unsigned)P);
     const size_t sum_bytes = 4 * ((size_t)n * dp + n);
-    const unsigned gx = (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)2 * nsm / P, (ntrain + 63) / 64));
-    const bool shared_sums = dtype == ANN_U8 && sum_bytes <= (size_t)optin && (ntrain + gx - 1) / gx < (1 << 24);
+    const bool shared_sums = dtype == ANN_U8 && sum_bytes <= (size_t)optin;
     if (shared_sums)
         ANN_CUDA(cudaFuncSetAttribute(km_accumulate_u8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)sum_bytes));
+    const dim3 grid_e((unsigned)(4 * nsm), (unsigned)P);
     for (int it = 0; it < iters; it++) {
         ANN_CUDA(cudaMemsetAsync(isums.p, 0, 8 * (size_t)total, s));
         ANN_CUDA(cudaMemsetAsync(fsums.p, 0, 8 * (size_t)total, s));
         ANN_CUDA(cudaMemsetAsync(counts.p, 0, 8 * (size_t)P * n, s));
-        ANN_CUDA(cudaMemsetAsync(namb.p, 0, 4 * (size_t)P, s));
         km_prep_kernel<<<P, 256, 0, s>>>(C.p, n, dp, cneg.p, cmax.p);
-        const dim3 grid_e((unsigned)(4 * nsm), (unsigned)P), grid_w(nblk(32 * ntrain), (unsigned)P);
-        if (dtype == ANN_U8) {
-            if (n > 64)
-                km_assign_kernel<ANN_U8, 16><<<grid_a, 256, 0, s>>>(train, ntrain, d, dp, n, cneg.p, cmax.p, assign.p,
-                                                                    amb.p, namb.p);
-            else
-                km_assign_kernel<ANN_U8, 8><<<grid_a, 256, 0, s>>>(train, ntrain, d, dp, n, cneg.p, cmax.p, assign.p,
-                                                                   amb.p, namb.p);
-            km_exact_kernel<ANN_U8><<<grid_e, 256, 0, s>>>(train, ntrain, d, dp, n, C.p, amb.p, namb.p, assign.p);
-            if (shared_sums)
-                km_accumulate_u8_kernel<<<dim3(gx, P), 512, sum_bytes, s>>>((const uint8_t *)train, ntrain, d, dp, n,
-                                                                            assign.p, isums.p, counts.p);
-            else
-                km_accumulate_kernel<ANN_U8><<<grid_w, 256, 0, s>>>(train, ntrain, d, dp, n, assign.p, isums.p,
-                                                                    fsums.p, counts.p);
-            km_update_kernel<ANN_U8><<<nblk(total), 256, 0, s>>>(total, dp, isums.p, fsums.p, counts.p, C.p);
-        } else {
-            if (n > 64)
-                km_assign_kernel<ANN_F32, 16><<<grid_a, 256, 0, s>>>(train, ntrain, d, dp, n, cneg.p, cmax.p, assign.p,
-                                                                     amb.p, namb.p);
-            else
-                km_assign_kernel<ANN_F32, 8><<<grid_a, 256, 0, s>>>(train, ntrain, d, dp, n, cneg.p, cmax.p, assign.p,
-                                                                    amb.p, namb.p);
-            km_exact_kernel<ANN_F32><<<grid_e, 256, 0, s>>>(train, ntrain, d, dp, n, C.p, amb.p, namb.p, assign.p);
-            km_accumulate_kernel<ANN_F32><<<grid_w, 256, 0, s>>>(train, ntrain, d, dp, n, assign.p, isums.p, fsums.p,
-                                                                 counts.p);
-            km_update_kernel<ANN_F32><<<nblk(total), 256, 0, s>>>(total, dp, isums.p, fsums.p, counts.p, C.p);
+        for (int64_t r0 = 0; r0 < ntrain; r0 += slice) {
+            const int64_t rows_s = std::min(slice, ntrain - r0);
+            const void *xs = (const uint8_t *)train + r0 * d * (dtype == ANN_U8 ? 1 : 4);
+            const dim3 grid_a((unsigned)((rows_s + BM - 1) / BM), (unsigned)P);
+            const dim3 grid_w(nblk(32 * rows_s), (unsigned)P);
+            const unsigned gx =
+                (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)2 * nsm / P, (rows_s + 63) / 64));
+            ANN_CUDA(cudaMemsetAsync(namb.p, 0, 4 * (size_t)P, s));
+            if (dtype == ANN_U8) {
+                if (n > 64)
+                    km_assign_kernel<ANN_U8, 16><<<grid_a, 256, 0, s>>>(xs, rows_s, d, dp, n, cneg.p, cmax.p, assign.p,
+                                                                        amb.p, namb.p);
+                else
+                    km_assign_kernel<ANN_U8, 8><<<grid_a, 256, 0, s>>>(xs, rows_s, d, dp, n, cneg.p, cmax.p, assign.p,
+                                                                       amb.p, namb.p);
+                km_exact_kernel<ANN_U8><<<grid_e, 256, 0, s>>>(xs, rows_s, d, dp, n, C.p, amb.p, namb.p, assign.p);
+                if (shared_sums)
+                    km_accumulate_u8_kernel<<<dim3(gx, P), 512, sum_bytes, s>>>((const uint8_t *)xs, rows_s, d, dp, n,
+                                                                                assign.p, isums.p, counts.p);
+                else
+                    km_accumulate_kernel<ANN_U8><<<grid_w, 256, 0, s>>>(xs, rows_s, d, dp, n, assign.p, isums.p,
+                                                                        fsums.p, counts.p);
+            } else {
+                if (n > 64)
+                    km_assign_kernel<ANN_F32, 16><<<grid_a, 256, 0, s>>>(xs, rows_s, d, dp, n, cneg.p, cmax.p, assign.p,
+                                                                         amb.p, namb.p);
+                else
+                    km_assign_kernel<ANN_F32, 8><<<grid_a, 256, 0, s>>>(xs, rows_s, d, dp, n, cneg.p, cmax.p, assign.p,
+                                                                        amb.p, namb.p);
+                km_exact_kernel<ANN_F32><<<grid_e, 256, 0, s>>>(xs, rows_s, d, dp, n, C.p, amb.p, namb.p, assign.p);
+                km_accumulate_kernel<ANN_F32><<<grid_w, 256, 0, s>>>(xs, rows_s, d, dp, n, assign.p, isums.p, fsums.p,
+                                                                     counts.p);
+            }
         }
+        if (dtype == ANN_U8)
+            km_update_kernel<ANN_U8><<<nblk(total), 256, 0, s>>>(total, dp, isums.p, fsums.p, counts.p, C.p);
+        else
+            km_update_kernel<ANN_F32><<<nblk(total), 256, 0, s>>>(total, dp, isums.p, fsums.p, counts.p, C.p);
         ANN_CUDA(cudaGetLastError());
     }
     km_store_kernel<<<nblk(total), 256, 0, s>>>(total, dtype, C.p, out_centers);

@@ -55,6 +55,28 @@ def test_kmeans_tile_edges_and_rows_left_to_fp64(ann, kind, N, d, P, n):
         np.testing.assert_allclose(got64.cpu().numpy(), want, rtol=0, atol=N * 2.0 ** -52 * np.abs(X).max())
 
 
+@pytest.mark.parametrize("N,dtype", [((1 << 24) + 300, "u8"), ((1 << 24) + 1, "f32"), ((1 << 31) + 4096, "u8")])
+def test_kmeans_rows_beyond_one_pass_and_beyond_32_bits(ann, N, dtype):
+    # two equal centers leave every row near them to the fp64 scan; rows of both clusters in the last pass
+    d, tail = 16, 200
+    if torch.cuda.mem_get_info()[0] < 2 * N * d * (1 if dtype == "u8" else 4):
+        pytest.skip("not enough device memory")
+    X = torch.empty((N, d), dtype=torch.uint8 if dtype == "u8" else torch.float32, device="cuda")
+    X.random_(0, 4)
+    X[:2] = 1
+    X[2] = 250
+    X[-tail:] = 240
+    _, got = ann.ann_train_centers(X, 1, 3, 1, np.arange(3), want_f64=True)
+    low = torch.zeros(d, dtype=torch.float64, device="cuda")
+    for r in range(0, N, 1 << 24):  # whole numbers below 2^53
+        low += X[r:r + (1 << 24)].sum(0, dtype=torch.float64)
+    del X
+    torch.cuda.empty_cache()
+    near = low.cpu().numpy() - (250 + 240 * tail)
+    want = np.stack([near / (N - tail - 1), np.ones(d), np.full(d, (250 + 240 * tail) / (tail + 1))])
+    np.testing.assert_array_equal(got[0].cpu().numpy(), want)
+
+
 @pytest.mark.parametrize("kind,N,d,P,n,t,b", [("u8", 70, 64, 4, 256, 100, 5),    # a buffer smaller than the candidates
                                               ("u8", 33, 48, 2, 256, 700, 2),    # t beyond the buffer's first size
                                               ("u8", 40, 96, 3, 33, 1, 5),
