@@ -122,8 +122,10 @@ int ann_build_knn_graph(const void *data, int dtype, int64_t N, int32_t d, int32
  * any size; those beyond shared memory are streamed through it) or the
  * largest leaf, ceil(N / 2^levels) rows of d + 20 bytes, within one CTA's
  * shared memory; otherwise ANN_ERR_ARG.  Allocates its
- * scratch (16 N bytes of sort keys, 8 N R bytes per graph copy) with
- * cudaMallocAsync on `stream`.  Asynchronous. */
+ * scratch (16 N bytes of sort keys, 8 N R bytes per graph copy and, for d 64
+ * and 128 with leaves of more than max(96, 24 R) points, another
+ * N (16 R + 2 d + 44) bytes where they can be had: without them the leaves
+ * take a slower kernel) with cudaMallocAsync on `stream`.  Asynchronous. */
 int ann_build_knn_graph_approx(const void *data, int dtype, int64_t N, int32_t d, int32_t R,
                                const int8_t *dirs, int32_t rounds, int32_t levels, int32_t iters,
                                int32_t *out_ids, void *out_keys, void *stream);

@@ -27,6 +27,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <optional>
 #include <cub/device/device_radix_sort.cuh>
 #include <utility>
 
@@ -438,8 +439,7 @@ extern "C" int ann_build_knn_graph_approx(const void *data, int dtype, int64_t N
     } while (0)
     AP_CUDA(cudaMallocAsync((void **)&ra, sizeof(uint64_t) * (size_t)N * R, s));
     if (iters > 0) AP_CUDA(cudaMallocAsync((void **)&rb, sizeof(uint64_t) * (size_t)N * R, s));
-    const bool tensor = (d == 64 || d == 128) && largest > leaf_tc_from(R);
-    if (levels > 0 || tensor) {
+    if (levels > 0) {
         AP_CUDA(cudaMallocAsync((void **)&k0, sizeof(uint64_t) * (size_t)N, s));
         AP_CUDA(cudaMallocAsync((void **)&k1, sizeof(uint64_t) * (size_t)N, s));
         cub::DoubleBuffer<uint64_t> probe(k0, k1);
@@ -450,10 +450,21 @@ extern "C" int ann_build_knn_graph_approx(const void *data, int dtype, int64_t N
     if (tiled) AP_CUDA(cudaFuncSetAttribute(rp_leaf_tiled_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             (int)smem));
     else AP_CUDA(cudaFuncSetAttribute(rp_leaf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    LeafTc tc(s);
-    if (tensor) {
-        const int rc = tc.prepare(N, d, R, levels, s);
-        if (rc != ANN_OK) {
+    // The tensor-core leaves take 16 R + 2 d + 44 bytes a row more than the
+    // kernels below them; where those cannot be had (270M to 540M rows of 128
+    // bytes, R = 16, on an empty device) the kernels that need none do the leaves.
+    std::optional<LeafTc> tc;
+    if ((d == 64 || d == 128) && largest > leaf_tc_from(R)) {
+        tc.emplace(s);
+        int rc = tc->prepare(N, d, R, levels, s);
+        if (rc == ANN_OK && levels == 0) {  // the order of the one leaf
+            const cudaError_t e = cudaMallocAsync((void **)&k0, sizeof(uint64_t) * (size_t)N, s);
+            if (e != cudaSuccess) rc = cuda_fail(e, "cudaMallocAsync(leaf order)");
+        }
+        if (rc == ANN_ERR_OOM) {
+            tc.reset();
+            cudaGetLastError();  // taken care of
+        } else if (rc != ANN_OK) {
             release();
             return rc;
         }
@@ -474,7 +485,7 @@ extern "C" int ann_build_knn_graph_approx(const void *data, int dtype, int64_t N
             AP_CUDA(cub::DeviceRadixSort::SortKeys(temp, tb, keys, (int)N, id_bits, l + proj_bits + id_bits, s));
         }
         const uint64_t *sorted = levels > 0 ? keys.Current() : nullptr;
-        if (tensor) {
+        if (tc) {
             // ids ascending inside a leaf, then the leaves' keys
             uint64_t *out = levels > 0 ? keys.Alternate() : keys.Current();
             rp_leaf_key_kernel<<<gridN, 256, 0, s>>>(N, levels, sorted, idmask, id_bits, out);
@@ -485,15 +496,15 @@ extern "C" int ann_build_knn_graph_approx(const void *data, int dtype, int64_t N
                 AP_CUDA(cub::DeviceRadixSort::SortKeys(temp, tb, keys, (int)N, id_bits, levels + id_bits, s));
             }
             sorted = keys.Current();
-            const int rc = tc.round((const uint8_t *)data, sorted, idmask, ra, s);
+            const int rc = tc->round((const uint8_t *)data, sorted, idmask, ra, s);
             if (rc != ANN_OK) {
                 release();
                 return rc;
             }
-            rp_merge_kernel<<<(unsigned)((N * 32 + 255) / 256), 256, 0, s>>>(N, R, tc.ids, tc.lists, tc.err, ra);
+            rp_merge_kernel<<<(unsigned)((N * 32 + 255) / 256), 256, 0, s>>>(N, R, tc->ids, tc->lists, tc->err, ra);
         }
         // other shapes, or (decided on the device) a tensor-core step that gave up
-        const int *only_if = tensor ? tc.err : nullptr;
+        const int *only_if = tc ? tc->err : nullptr;
         if (tiled)
             rp_leaf_tiled_kernel<<<(unsigned)(nleaves * chunks), TILE_THREADS, smem, s>>>(
                 (const uint8_t *)data, N, d, R, levels, chunks, sorted, idmask, ra, only_if);

@@ -1,0 +1,71 @@
+"""Calls whose scratch does not fit the device fall back to forms that need
+less, with the same results.  The device's current memory pool, from which the
+library takes its stream-ordered scratch, is replaced by one of a limited size
+(CUDA driver API), so that an allocation fails without filling the device."""
+from __future__ import annotations
+
+import contextlib
+import ctypes
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+from paper_1312_3062_gb300 import datagen  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def ann():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_1312_3062_gb300 import _build
+    _build.build()
+    from paper_1312_3062_gb300 import ann as mod
+    return mod
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+class PoolProps(ctypes.Structure):  # CUmemPoolProps
+    _fields_ = [("allocType", ctypes.c_int), ("handleTypes", ctypes.c_int), ("location_type", ctypes.c_int),
+                ("location_id", ctypes.c_int), ("security", ctypes.c_void_p), ("maxSize", ctypes.c_size_t),
+                ("usage", ctypes.c_ushort), ("reserved", ctypes.c_ubyte * 54)]
+
+
+@contextlib.contextmanager
+def pool_of(mbytes):
+    cu = ctypes.CDLL("libcuda.so.1")
+    torch.zeros(1, device="cuda")  # the primary context is current
+    torch.cuda.synchronize()
+    props = PoolProps(allocType=1, location_type=1, location_id=torch.cuda.current_device(), maxSize=mbytes << 20)
+    device = ctypes.c_int(props.location_id)
+    small, before, p = ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_uint64()
+    assert cu.cuDeviceGetMemPool(ctypes.byref(before), device) == 0
+    assert cu.cuMemPoolCreate(ctypes.byref(small), ctypes.byref(props)) == 0
+    assert cu.cuDeviceSetMemPool(device, small) == 0
+    try:
+        # the limit holds: twice its size is refused
+        assert cu.cuMemAllocAsync(ctypes.byref(p), ctypes.c_size_t(mbytes << 21), None) == 2
+        yield
+        torch.cuda.synchronize()
+    finally:
+        assert cu.cuDeviceSetMemPool(device, before) == 0
+        torch.cuda.synchronize()
+        assert cu.cuMemPoolDestroy(small) == 0
+
+
+@pytest.mark.parametrize("N,R,levels,mbytes", [(60_000, 16, 4, 64), (6000, 8, 0, 32)])
+def test_approx_graph_leaves_without_the_tensor_cores_scratch(ann, N, R, levels, mbytes):
+    # lists and pending groups of the tensor-core leaves take some 90 and 55 MB, the rest 18 and 1 MB
+    X = dev(datagen.mixture(N, N, 128, 11, np.uint8))
+    dirs = dev(datagen.rp_directions(N, 2, levels, 128))
+    want = ann.ann_build_knn_graph_approx(X, R, dirs, 1)
+    with pool_of(mbytes):
+        got = ann.ann_build_knn_graph_approx(X, R, dirs, 1)
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
