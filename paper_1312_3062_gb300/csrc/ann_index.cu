@@ -33,6 +33,7 @@ int fail(int code, const std::string &msg) {
 
 int cuda_fail(cudaError_t e, const char *what) {
     g_err = std::string(what) + ": " + cudaGetErrorString(e);
+    cudaGetLastError();  // reported here: the launch checks of the next call must not find it
     return e == cudaErrorMemoryAllocation ? ANN_ERR_OOM : ANN_ERR_CUDA;
 }
 

@@ -463,7 +463,6 @@ extern "C" int ann_build_knn_graph_approx(const void *data, int dtype, int64_t N
         }
         if (rc == ANN_ERR_OOM) {
             tc.reset();
-            cudaGetLastError();  // taken care of
         } else if (rc != ANN_OK) {
             release();
             return rc;

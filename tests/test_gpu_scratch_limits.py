@@ -69,3 +69,16 @@ def test_approx_graph_leaves_without_the_tensor_cores_scratch(ann, N, R, levels,
         got = ann.ann_build_knn_graph_approx(X, R, dirs, 1)
     for a, b in zip(got, want):
         assert torch.equal(a, b)
+
+
+def test_a_call_that_ran_out_of_memory_does_not_fail_the_next(ann):
+    X = dev(datagen.mixture(5, 300_000, 64, 11, np.uint8))
+    dirs = dev(datagen.rp_directions(5, 1, 3, 64))
+    with pool_of(32):
+        with pytest.raises(ann.AnnError) as e:  # 38 MB of rows
+            ann.ann_build_knn_graph_approx(X, 16, dirs, 0)
+        assert e.value.code == ann.ANN_ERR_OOM
+        few = X[:1000]
+        got = ann.ann_build_knn_graph_approx(few, 16, dirs, 0)
+    for a, b in zip(got, ann.ann_build_knn_graph_approx(few, 16, dirs, 0)):
+        assert torch.equal(a, b)
