@@ -66,7 +66,10 @@ const char *ann_last_error(void);
  * and skips row i for query i: this is the exact R-NN neighbourhood graph of
  * Sec. 3.1 / Sec. 4.1.  Rows with fewer than k candidates are padded with
  * id -1 / key UINT32_MAX (u8) or +inf (f32).  out_ids: device int32[nq*k];
- * out_keys: device, optional (NULL), nq*k keys.  k <= 32. */
+ * out_keys: device, optional (NULL), nq*k keys.  k <= 32.  The tensor-core
+ * forms (uint8 with d 64 or 128; float32 from N = 8192 and nq = 256 on) end
+ * with a wait on the host; on a stream under capture the plain SIMT scan runs
+ * instead, with the same result. */
 int ann_exact_knn(const void *refs, int64_t N, const void *queries, int64_t nq, int dtype,
                   int32_t d, int32_t k, int32_t exclude_self, int32_t *out_ids, void *out_keys,
                   void *stream);

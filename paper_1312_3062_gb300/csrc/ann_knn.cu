@@ -234,19 +234,16 @@ extern "C" int ann_exact_knn(const void *refs, int64_t N, const void *queries, i
     ANN_ARG(!exclude_self || (queries == refs && nq == N), "exclude_self needs queries == refs");
     if (nq == 0) return ANN_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    // the tensor-core form reads its error word back, which a capturing stream
-    // does not allow: there the largest k of the widest rows keeps the SIMT form
-    bool tensor = dtype == ANN_U8 && (d == 64 || d == 128);
-    if (tensor && d == 128 && k > 30) {
-        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-        ANN_CUDA(cudaStreamIsCapturing(s, &st));
-        tensor = st == cudaStreamCaptureStatusNone;
-    }
-    if (tensor)
+    // Tensor-core forms: uint8 rows of 64 and 128 and float32 at scale
+    // (candidates from dot products, exact keys).  Both read a word back from
+    // the device, which a capturing stream does not allow: it takes the SIMT form.
+    const bool u8 = dtype == ANN_U8 && (d == 64 || d == 128), f32 = dtype == ANN_F32 && N >= 8192 && nq >= 256;
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (u8 || f32) ANN_CUDA(cudaStreamIsCapturing(s, &capturing));
+    if (u8 && capturing == cudaStreamCaptureStatusNone)
         return knn_u8_tensor((const uint8_t *)refs, N, (const uint8_t *)queries, nq, d, k, exclude_self, out_ids,
                              (uint32_t *)out_keys, s);
-    // float32 at scale: candidates from tensor-core dot products, exact keys
-    if (dtype == ANN_F32 && N >= 8192 && nq >= 256)
+    if (f32 && capturing == cudaStreamCaptureStatusNone)
         return knn_f32_tensor((const float *)refs, N, (const float *)queries, nq, d, k, exclude_self, out_ids,
                               (uint32_t *)out_keys, s);
     uint32_t *rn = nullptr, *qn = nullptr;

@@ -259,3 +259,20 @@ def test_widest_lists_and_plain_searches_can_be_captured(ann):
         for a, b in zip(got, want):
             np.testing.assert_array_equal(a.cpu().numpy(), b)
             a.zero_()
+
+
+@pytest.mark.parametrize("dtype,N,nq,d,k", [(np.uint8, 3000, 200, 64, 10), (np.uint8, 3000, 200, 64, 31),
+                                            (np.uint8, 3000, 200, 128, 10), (np.uint8, 3000, 200, 128, 32),
+                                            (np.float32, 8192, 256, 36, 10), (np.float32, 8192, 255, 36, 10)])
+def test_exact_knn_can_be_captured_whatever_its_sizes(ann, dtype, N, nq, d, k):
+    X, Q = dev(datagen.mixture(3, N, d, 9, dtype)), dev(datagen.mixture(4, nq, d, 9, dtype))
+    want = ann.ann_exact_knn(X, Q, k)
+    buf = torch.zeros_like(Q)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, capture_error_mode="thread_local"):
+        got = ann.ann_exact_knn(X, buf, k, stream=torch.cuda.current_stream())
+    buf.copy_(Q)
+    g.replay()
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
