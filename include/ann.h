@@ -69,7 +69,9 @@ const char *ann_last_error(void);
  * out_keys: device, optional (NULL), nq*k keys.  k <= 32.  The tensor-core
  * forms (uint8 with d 64 or 128; float32 from N = 8192 and nq = 256 on) end
  * with a wait on the host; on a stream under capture the plain SIMT scan runs
- * instead, with the same result. */
+ * instead, with the same result, and so it does for uint8 rows where the
+ * tensor-core form's scratch (2 d + 36 bytes per row and about 50 MB) cannot
+ * be had. */
 int ann_exact_knn(const void *refs, int64_t N, const void *queries, int64_t nq, int dtype,
                   int32_t d, int32_t k, int32_t exclude_self, int32_t *out_ids, void *out_keys,
                   void *stream);

@@ -240,9 +240,13 @@ extern "C" int ann_exact_knn(const void *refs, int64_t N, const void *queries, i
     const bool u8 = dtype == ANN_U8 && (d == 64 || d == 128), f32 = dtype == ANN_F32 && N >= 8192 && nq >= 256;
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     if (u8 || f32) ANN_CUDA(cudaStreamIsCapturing(s, &capturing));
-    if (u8 && capturing == cudaStreamCaptureStatusNone)
-        return knn_u8_tensor((const uint8_t *)refs, N, (const uint8_t *)queries, nq, d, k, exclude_self, out_ids,
-                             (uint32_t *)out_keys, s);
+    if (u8 && capturing == cudaStreamCaptureStatusNone) {
+        // without room for its bf16 rows (2 d + 36 bytes each), pending groups
+        // (50 MB) and lists, the scan below, which takes 4 bytes a row
+        const int r = knn_u8_tensor((const uint8_t *)refs, N, (const uint8_t *)queries, nq, d, k, exclude_self,
+                                    out_ids, (uint32_t *)out_keys, s);
+        if (r != ANN_ERR_OOM) return r;
+    }
     if (f32 && capturing == cudaStreamCaptureStatusNone)
         return knn_f32_tensor((const float *)refs, N, (const float *)queries, nq, d, k, exclude_self, out_ids,
                               (uint32_t *)out_keys, s);

@@ -82,3 +82,13 @@ def test_a_call_that_ran_out_of_memory_does_not_fail_the_next(ann):
         got = ann.ann_build_knn_graph_approx(few, 16, dirs, 0)
     for a, b in zip(got, ann.ann_build_knn_graph_approx(few, 16, dirs, 0)):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("d,k", [(64, 32), (128, 10)])
+def test_exact_knn_without_the_tensor_cores_scratch(ann, d, k):
+    X, Q = dev(datagen.mixture(6, 20_000, d, 11, np.uint8)), dev(datagen.mixture(7, 300, d, 11, np.uint8))
+    want = ann.ann_exact_knn(X, Q, k)
+    with pool_of(32):  # the pending groups alone are 50 MB
+        got = ann.ann_exact_knn(X, Q, k)
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
