@@ -187,7 +187,11 @@ static bool launch_batch(ann_server *S, Slot &sl, std::vector<std::shared_ptr<Re
     sl.finished.store(false);
     if (ok) ok = cudaLaunchHostFunc(s, on_done, &sl) == cudaSuccess;
     if (!ok) {
-        S->thread_error = cudaGetErrorString(cudaGetLastError());
+        const cudaError_t e = cudaGetLastError();
+        S->thread_error = e != cudaSuccess ? cudaGetErrorString(e) : ann_last_error();
+        // what was issued may still use the batch's share of the pool, which
+        // goes to other requests now
+        cudaStreamSynchronize(s);
         return false;
     }
     sl.busy = true;
