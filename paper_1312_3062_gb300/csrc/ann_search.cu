@@ -169,9 +169,14 @@ static int plan_launch(const SearchArgs &base, int capT, const int32_t *list, co
     // T = 1024 / 2048 / 4096: 0.88 / 2.58 / 17.3 -> 0.68 / 2.05 / 14.3 ms.
     cfg.main.L = main_layout(ix.dtype, ix.d, capT, A.kmax, ix.b, ix.R, tn.stage, false, (uint32_t)tn.spill_heap);
     const int64_t fit = (int64_t)(g_smem_optin / (cfg.main.L.total + 1024)) * g_num_sms;
-    const bool win = capT >= kWindowedFromT && list_len > fit;
-    A.capT = capT;
     // bridge batch: budgets below the windowed kernels pop few bridges
+    auto res_layout = [&](bool w, bool split) {
+        return make_layout(ix.dtype, ix.d, ix.P, ix.n, ix.PA, capT, A.kmax, w ? 128 : 64, ix.b, ix.R, true, grouped, w,
+                           (uint32_t)tn.spill_heap, split);
+    };
+    const bool win =
+        capT >= kWindowedFromT && (list_len > fit || res_layout(false, false).total > g_smem_optin);
+    A.capT = capT;
     A.bcap = win ? 128 : 64;
     A.bstore = (int)(kFirstEnough + kFirstCap);
     A.list = list;
@@ -183,12 +188,17 @@ static int plan_launch(const SearchArgs &base, int capT, const int32_t *list, co
     cfg.chunk = std::min(list_len, kChunk);
     cfg.pro.L = prologue_layout(ix.dtype, ix.d, ix.P, ix.n, ix.PA, (int)kFirstCap, grouped, win);
     cfg.main.L = main_layout(ix.dtype, ix.d, capT, A.kmax, ix.b, ix.R, tn.stage, win, (uint32_t)tn.spill_heap);
-    cfg.res.L = make_layout(ix.dtype, ix.d, ix.P, ix.n, ix.PA, capT, A.kmax, A.bcap, ix.b, ix.R, true, grouped, win,
-                            (uint32_t)tn.spill_heap, true);
-    int r = fit_shape(cfg.pro, 4, cfg.chunk, 8, [&](size_t smem, int threads, int *blocks) {
-        return prologue_occupancy(ix, smem, threads, blocks);
-    });
-    if (r == ANN_OK)
+    cfg.res.L = res_layout(win, true);
+    if (cfg.res.L.total > g_smem_optin) cfg.res.L = res_layout(win, false);
+    // rows so wide (float32 from about 20,000 dimensions) that a query fills an
+    // SM: what holds it leanest runs it alone
+    const bool lean = cfg.pro.L.total > g_smem_optin || cfg.main.L.total > g_smem_optin;
+    int r = ANN_OK;
+    if (!lean)
+        r = fit_shape(cfg.pro, 4, cfg.chunk, 8, [&](size_t smem, int threads, int *blocks) {
+            return prologue_occupancy(ix, smem, threads, blocks);
+        });
+    if (r == ANN_OK && !lean)
         r = fit_shape(cfg.main, tn.warps, cfg.chunk, 1, [&](size_t smem, int threads, int *blocks) {
             return main_occupancy(ix.dtype, win, cfg.wide, smem, threads, blocks);
         });
@@ -201,7 +211,7 @@ static int plan_launch(const SearchArgs &base, int capT, const int32_t *list, co
     // there are more queries than that, and a suspended one would come after
     // all that were not.  SIFT-shaped rows, P = 2 x n = 64, 600 queries, T = 64 /
     // 256 / 2048: three kernels 232 / 298 / 1406 us, one 207 / 252 / 1186 us.
-    cfg.whole = cfg.res.warps >= list_len;
+    cfg.whole = lean || cfg.res.warps >= list_len;
     A.whole = cfg.whole;
     auto al = [](uint64_t x) { return (x + 255) & ~(uint64_t)255; };
     // a sorted window serves many batches of bridges

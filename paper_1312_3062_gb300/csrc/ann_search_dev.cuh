@@ -2218,7 +2218,7 @@ __global__ void __launch_bounds__(192, 2) resume_kernel(const __grid_constant__ 
     const int warp = threadIdx.x >> 5;
     uint8_t *smem = smem_all + (size_t)warp * A.L.total;
     uint8_t *wscratch = A.gscratch + ((size_t)blockIdx.x * (blockDim.x >> 5) + warp) * A.wstride;
-    if (A.whole) {  // no more queries than warps
+    if (A.whole) {  // no more queries than warps (or rows too wide for the other kernels)
         const int64_t end = query_end(A), step = (int64_t)gridDim.x * (blockDim.x >> 5);
         for (int64_t w = A.base + (int64_t)blockIdx.x * (blockDim.x >> 5) + warp; w < end; w += step)
             search_one<DT, SP, GRP, true>(A, smem, w, wscratch);

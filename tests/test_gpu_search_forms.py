@@ -64,3 +64,26 @@ def test_many_queries_equal_few_and_the_oracle(ann, dtype, N, d, comps, P, n, R,
     np.testing.assert_array_equal(many[0][sel], wi)
     np.testing.assert_array_equal(many[3][sel, 1], ws["ref_pops"])
     np.testing.assert_array_equal(many[3][sel, 2], ws["nonempty_bridge_pops"])
+
+
+# rows so wide that one query fills an SM: beside a budget's queue and visited set in shared memory (T = 8192), and
+# beside no more than the prologue's first batch (T = 32; also more queries than SMs)
+@pytest.mark.parametrize("d,T,nq", [(24_000, 8192, 12), (24_000, 8192, 300), (55_728, 32, 12), (55_728, 32, 300)])
+def test_rows_as_wide_as_shared_memory(ann, d, T, nq):
+    rng = np.random.default_rng(d)
+    N, P, n, k = 300, 2, 256, 10
+    X = datagen.mixture(1, N, d, 4, np.float32)
+    Q = datagen.mixture(2, nq, d, 4, np.float32)
+    C = np.ascontiguousarray(X[rng.permutation(N)[:n]].reshape(n, P, d // P).transpose(1, 0, 2))
+    G, _ = ann.ann_build_knn_graph(dev(X), 8)
+    ix = ann.Index.create(dev(X), G, dev(C), t=20, b=5)
+    ids, refs = ix.bridges()
+    bg = dict(bridges=ids, offsets=np.concatenate([[0], np.cumsum((refs >= 0).sum(1))]).astype(np.int64),
+              refs=refs[refs >= 0])
+    sel = rng.permutation(nq)[:12]
+    want = oracle.search(X, G.cpu().numpy(), C, bg, Q[sel], k, T, kmax=k, nthreads=8)[0]
+    for mode in (0, 1):
+        got, _, status = ann.ann_search_batch(ix, dev(Q), k, T, mode=mode)
+        torch.cuda.synchronize()
+        assert not status.any()
+        np.testing.assert_array_equal(got.cpu().numpy()[sel], want)
