@@ -267,8 +267,13 @@ enum {
  * out_stats (optional) int64[nq*ANN_NSTATS].
  * mode ANN_MODE_PLAIN: the kernels of this batch on `stream`, sized for the
  * largest budget (per-query T costs one device max and a host sync), with a
- * stream-ordered workspace of about 5 KB per query (passes of 32768 queries)
- * and up to 256 MB for the states of queries that pop many bridges.
+ * stream-ordered workspace (cudaMallocAsync): about 5 KB per query, in passes
+ * of 32768 queries; up to 256 MB for the states of queries that pop many
+ * bridges; and per warp that the device holds at once (about 1,800, or one
+ * per query if fewer) 24 min(8192, max(1024, 2 T)) bytes, from T = 1024 on
+ * another 14.4 T.  Batches that the device holds at once need the last part
+ * only.  Where a workspace cannot be had, smaller passes run, down to 128
+ * queries (7 MB below T = 1024, at most 45 MB); below that ANN_ERR_OOM.
  * mode ANN_MODE_PERSISTENT: queries are bucketed by budget (128 * 2^i) and
  * each bucket is run by kernels sized for it, the buckets side by side; the
  * sequence is captured once per (index, pointers, sizes, stream) into a CUDA

@@ -150,14 +150,18 @@ struct LaunchCfg {
 
 // A pass holds the records and first bridge batches of at most kChunk queries
 // (4.7 KB each), and states of suspended ones up to kSaveBytes; queries
-// that find no room there start again when they are resumed.
+// that find no room there start again when they are resumed.  Where the device
+// has no room for that, passes and states are a quarter as large (`shrink`
+// times over), down to 128 queries: 7 MB for budgets below 1024, 40 MB for the
+// largest (the scratch of as many warps).
 static const int64_t kChunk = 32768;
 static const size_t kSaveBytes = (size_t)256 << 20;
+static const int kMaxShrink = 4;
 
 static int plan_launch(const SearchArgs &base, int capT, const int32_t *list, const int32_t *list_count,
-                       int64_t list_len, LaunchCfg &cfg, const Tune *tune = nullptr) {
+                       int64_t list_len, LaunchCfg &cfg, const Tune *tune = nullptr, int shrink = 0) {
     // the buckets of a batch (their counts are on the device) share its queries
-    const size_t save_bytes = list_count ? kSaveBytes / 4 : kSaveBytes;
+    const size_t save_bytes = (list_count ? kSaveBytes / 4 : kSaveBytes) >> (2 * shrink);
     SearchArgs A = base;
     const DevIndex &ix = A.ix;
     const bool grouped = ix.ngroups > 0;
@@ -185,7 +189,7 @@ static int plan_launch(const SearchArgs &base, int capT, const int32_t *list, co
     cfg.win = win;
     cfg.wide = list_len > (int64_t)g_num_sms * kMainWarps * kMainCtas;
     cfg.total = list_len;
-    cfg.chunk = std::min(list_len, kChunk);
+    cfg.chunk = std::min(list_len, kChunk >> (2 * shrink));
     cfg.pro.L = prologue_layout(ix.dtype, ix.d, ix.P, ix.n, ix.PA, (int)kFirstCap, grouped, win);
     cfg.main.L = main_layout(ix.dtype, ix.d, capT, A.kmax, ix.b, ix.R, tn.stage, win, (uint32_t)tn.spill_heap);
     cfg.res.L = res_layout(win, true);
@@ -234,13 +238,15 @@ static int plan_launch(const SearchArgs &base, int capT, const int32_t *list, co
     A.save_stride = al(A.save_spill + (win ? 8ull * (uint64_t)capT : 0ull));
     A.nslots = (uint32_t)std::min<int64_t>(cfg.chunk, (int64_t)(save_bytes / A.save_stride));
     size_t o = 256;  // counters
-    cfg.o_rec = o;   o = al(o + sizeof(QRec) * (size_t)cfg.chunk);
-    cfg.o_bk = o;    o = al(o + 8 * (size_t)A.bstore * cfg.chunk);
-    cfg.o_bi = o;    o = al(o + 4 * (size_t)A.bstore * cfg.chunk);
-    cfg.o_susp = o;  o = al(o + 4 * (size_t)cfg.chunk);
-    cfg.o_save = o;  o = al(o + (size_t)A.nslots * A.save_stride);
+    // records, first batches and states are the three kernels' only
+    const size_t held = cfg.whole ? 0 : (size_t)cfg.chunk;
+    cfg.o_rec = o;   o = al(o + sizeof(QRec) * held);
+    cfg.o_bk = o;    o = al(o + 8 * (size_t)A.bstore * held);
+    cfg.o_bi = o;    o = al(o + 4 * (size_t)A.bstore * held);
+    cfg.o_susp = o;  o = al(o + 4 * held);
+    cfg.o_save = o;  o = al(o + (cfg.whole ? 0 : (size_t)A.nslots * A.save_stride));
     cfg.o_scratch = o;
-    o = al(o + std::max(cfg.main.warps * cfg.main_stride, cfg.res.warps * cfg.res_stride));
+    o = al(o + std::max(cfg.whole ? 0 : cfg.main.warps * cfg.main_stride, cfg.res.warps * cfg.res_stride));
     cfg.bytes = o;
     cfg.A = A;
     return ANN_OK;
@@ -302,14 +308,21 @@ static int do_launch(LaunchCfg &cfg, uint8_t *ws, cudaStream_t stream, int first
 // plan + stream-ordered workspace + launch
 static int launch_search(const SearchArgs &base, int capT, cudaStream_t stream, const int32_t *list,
                          int64_t list_len) {
-    LaunchCfg cfg;
-    int r = plan_launch(base, capT, list, nullptr, list_len, cfg);
-    if (r != ANN_OK) return r;
-    uint8_t *ws = nullptr;
-    ANN_CUDA(cudaMallocAsync((void **)&ws, cfg.bytes, stream));
-    r = do_launch(cfg, ws, stream);
-    cudaFreeAsync(ws, stream);
-    return r;
+    for (int shrink = 0;; shrink++) {
+        LaunchCfg cfg;
+        int r = plan_launch(base, capT, list, nullptr, list_len, cfg, nullptr, shrink);
+        if (r != ANN_OK) return r;
+        uint8_t *ws = nullptr;
+        const cudaError_t e = cudaMallocAsync((void **)&ws, cfg.bytes, stream);
+        if (e != cudaSuccess) {
+            r = cuda_fail(e, "cudaMallocAsync(search workspace)");
+            if (r == ANN_ERR_OOM && shrink < kMaxShrink) continue;
+            return r;
+        }
+        r = do_launch(cfg, ws, stream);
+        cudaFreeAsync(ws, stream);
+        return r;
+    }
 }
 
 __global__ void max_kernel(const int32_t *v, int64_t n, int32_t *out) {

@@ -92,3 +92,25 @@ def test_exact_knn_without_the_tensor_cores_scratch(ann, d, k):
         got = ann.ann_exact_knn(X, Q, k)
     for a, b in zip(got, want):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("nq,T,mbytes", [(10_000, 400, 64), (1500, 900, 32), (3000, 3000, 96)])
+def test_plain_search_in_smaller_passes(ann, nq, T, mbytes):
+    # records and first batches of 10,000 queries take 47 MB, the scratch of a full device some 90 MB (T = 400), 73 MB
+    # for 1500 queries in one kernel, and 330 MB (T = 3000)
+    N = 4000
+    X = dev(datagen.mixture(8, N, 128, 40, np.uint8))
+    Q = dev(datagen.mixture(9, nq, 128, 40, np.uint8))
+    G, _ = ann.ann_build_knn_graph(X, 10)
+    ix = ann.Index.create(X, G, ann.ann_train_centers(X, 4, 24, 2, np.arange(24)), t=100, b=5)
+
+    def search():
+        st = torch.zeros((nq, ann.ANN_NSTATS), dtype=torch.int64, device="cuda")
+        out = ann.ann_search_batch(ix, Q, 10, T, mode=0, out_stats=st)
+        return [*out, st[:, [ann.STAT_NAMES.index(s) for s in ("discovered", "ref_pops", "bridge_pops", "max_q")]]]
+
+    want = search()
+    with pool_of(mbytes):
+        got = search()
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
