@@ -278,7 +278,10 @@ enum {
  * each bucket is run by kernels sized for it, the buckets side by side; the
  * sequence is captured once per (index, pointers, sizes, stream) into a CUDA
  * graph and replayed (at most 32 plans and 16 GB of workspaces per index,
- * least recently used evicted after its stream finished).  The
+ * least recently used evicted after its last launch finished).  The plans of
+ * one stream share a workspace, which holds a plain search's for each bucket
+ * in use, with a quarter of its states (10,000 queries with budgets up to
+ * 8192: about 2 GB); where it cannot be had, passes are smaller.  The
  * first call that meets a (budget bucket, kmax) measures candidate launch
  * shapes on the batch itself and keeps the fastest for the index; that call
  * synchronizes `stream` and runs the batch a few times.

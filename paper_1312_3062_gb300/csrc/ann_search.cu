@@ -6,7 +6,9 @@
 
 #include <algorithm>
 #include <map>
+#include <memory>
 #include <mutex>
+#include <set>
 #include <tuple>
 #include <vector>
 
@@ -344,12 +346,26 @@ __global__ void bucket_kernel(int64_t nq, const int32_t *T, int32_t T_all, int32
     lists[(int64_t)bkt * nq + pos] = (int32_t)i;
 }
 
+// Device memory that the kernels of recorded plans work in.  The plans of one
+// stream share it: they run one after another, which `done`, recorded behind
+// every launch, also ensures where a stream's handle does not (a handle that
+// was destroyed and given out again, the per-thread default stream).
+struct Workspace {
+    uint8_t *p = nullptr;
+    size_t bytes = 0;
+    cudaEvent_t done = nullptr;
+    const void *last = nullptr;  // the graph launched last
+    ~Workspace() {
+        if (done) cudaEventDestroy(done);
+        if (p) cudaFree(p);
+    }
+};
+
 struct Plan {
     cudaGraphExec_t exec = nullptr;
-    int32_t *scratch = nullptr;   // counts[kBuckets], then lists[kBuckets*nq]
-    uint8_t *wscratch = nullptr;  // the buckets' workspaces, one after another
-    size_t bytes = 0;             // of the workspaces
-    uint64_t last_use = 0;        // for evicting the least recently used plan
+    int32_t *scratch = nullptr;     // counts[kBuckets], then lists[kBuckets*nq]
+    std::shared_ptr<Workspace> ws;  // the buckets' workspaces, one after another
+    uint64_t last_use = 0;          // for evicting the least recently used plan
 };
 
 // plans kept per index, and bytes of their workspaces; beyond either the least
@@ -386,10 +402,39 @@ void free_plans(ann_index *ix) {
     for (auto &kv : pc->plans) {
         if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
         if (kv.second.scratch) cudaFree(kv.second.scratch);
-        if (kv.second.wscratch) cudaFree(kv.second.wscratch);
     }
     delete pc;
     ix->plans = nullptr;
+}
+
+// bytes of the distinct workspaces of an index's plans
+static size_t held_bytes(const PlanCache *pc) {
+    std::set<const Workspace *> seen;
+    size_t b = 0;
+    for (auto &kv : pc->plans)
+        if (seen.insert(kv.second.ws.get()).second) b += kv.second.ws->bytes;
+    return b;
+}
+
+// a workspace of at least `need` bytes that a plan of this stream has already
+static std::shared_ptr<Workspace> workspace_of(const PlanCache *pc, cudaStream_t s, size_t need) {
+    for (auto &kv : pc->plans)
+        if (kv.first.stream == s && kv.second.ws->bytes >= need) return kv.second.ws;
+    return nullptr;
+}
+
+// The least recently used plan goes, once what was launched in its workspace
+// has finished (its stream may be gone).
+static int evict_plan(PlanCache *pc) {
+    auto old = pc->plans.begin();
+    for (auto it = pc->plans.begin(); it != pc->plans.end(); ++it)
+        if (it->second.last_use < old->second.last_use) old = it;
+    ANN_CUDA(cudaEventSynchronize(old->second.ws->done));
+    old->second.ws->last = nullptr;  // nothing left to wait for, and the graph's address may come back
+    cudaGraphExecDestroy(old->second.exec);
+    cudaFree(old->second.scratch);
+    pc->plans.erase(old);
+    return ANN_OK;
 }
 
 // budgets of the buckets one persistent batch may use
@@ -435,13 +480,14 @@ struct ForkSet {
 
 // one bucket's launch: the whole batch in order, or (per-query T) its list
 static int plan_bucket(const SearchArgs &A, int64_t nq, const int32_t *T, int32_t *scratch, int bkt, int capT,
-                       LaunchCfg &cfg, const Tune *tn) {
-    if (!T) return plan_launch(A, capT, nullptr, nullptr, nq, cfg, tn);
-    return plan_launch(A, capT, scratch + kBuckets + (int64_t)bkt * nq, scratch + bkt, nq, cfg, tn);
+                       LaunchCfg &cfg, const Tune *tn, int shrink) {
+    if (!T) return plan_launch(A, capT, nullptr, nullptr, nq, cfg, tn, shrink);
+    return plan_launch(A, capT, scratch + kBuckets + (int64_t)bkt * nq, scratch + bkt, nq, cfg, tn, shrink);
 }
 
 static int record_persistent(const PlanCache *pc, const SearchArgs &A, int64_t nq, const int32_t *T, int32_t T_all,
-                             int32_t *scratch, uint8_t *wscratch, size_t wbytes, cudaStream_t s, ForkSet &fs) {
+                             int32_t *scratch, uint8_t *wscratch, size_t wbytes, int shrink, cudaStream_t s,
+                             ForkSet &fs) {
     int32_t *counts = scratch, *lists = scratch + kBuckets;
     if (T) {
         ANN_CUDA(cudaMemsetAsync(counts, 0, sizeof(int32_t) * kBuckets, s));
@@ -455,7 +501,7 @@ static int record_persistent(const PlanCache *pc, const SearchArgs &A, int64_t n
         const int capT = sized_for(bkt, T, T_all);
         const Tune *tn = tuned_for(pc, bucket_cap(bkt), A.kmax);
         LaunchCfg cfg;
-        rc = plan_bucket(A, nq, T, scratch, bkt, capT, cfg, tn);
+        rc = plan_bucket(A, nq, T, scratch, bkt, capT, cfg, tn, shrink);
         if (rc != ANN_OK) break;
         if (cfg.bytes > wbytes) {
             rc = fail(ANN_ERR_CAPACITY, "search workspace smaller than its kernels need");
@@ -666,110 +712,83 @@ extern "C" int ann_search_batch(const ann_index *index, const void *queries, int
         if (capT < 32) capT = 32;
         return launch_search(A, capT, s, nullptr, nq);
     }
-    // persistent: bucket by budget, one persistent kernel per bucket, replayed as a CUDA graph
+    // persistent: bucket by budget, the buckets' kernels side by side, replayed as a CUDA graph
     ann_index *ixm = const_cast<ann_index *>(index);
     if (!ixm->plans) ixm->plans = new PlanCache();
     PlanCache *pc = (PlanCache *)ixm->plans;
     PlanKey key{queries, nq, k, T, k_all, T_all, kmax, out_ids, out_keys, out_status, out_stats, s};
     std::lock_guard<std::mutex> g(pc->mu);
     auto it = pc->plans.find(key);
-    // evict the least recently used plan once its stream has finished with it
-    auto evict = [pc]() -> int {
-        auto old = pc->plans.begin();
-        for (auto jt = pc->plans.begin(); jt != pc->plans.end(); ++jt)
-            if (jt->second.last_use < old->second.last_use) old = jt;
-        ANN_CUDA(cudaStreamSynchronize(old->first.stream));
-        cudaGraphExecDestroy(old->second.exec);
-        cudaFree(old->second.scratch);
-        if (old->second.wscratch) cudaFree(old->second.wscratch);
-        pc->plans.erase(old);
-        return ANN_OK;
-    };
     if (it == pc->plans.end() && pc->plans.size() >= kMaxPlans) {
-        const int er = evict();
+        const int er = evict_plan(pc);
         if (er != ANN_OK) return er;
     }
     if (it == pc->plans.end()) {
         Plan p;
         ANN_CUDA(cudaMalloc(&p.scratch, sizeof(int32_t) * (kBuckets + (size_t)kBuckets * nq)));
-        {
-            int r = autotune(pc, A, nq, T, T_all, p.scratch, s);
-            if (r != ANN_OK) {
-                cudaFree(p.scratch);
-                return r;
-            }
+        auto drop = [&p](int code) {
+            cudaFree(p.scratch);
+            return code;
+        };
+        r = autotune(pc, A, nq, T, T_all, p.scratch, s);
+        if (r != ANN_OK) return drop(r);
+        int b0, b1, shrink = 0;
+        bucket_range(T, T_all, b0, b1);
+        for (;; shrink++) {
             size_t need = 0;
-            int b0, b1;
-            bucket_range(T, T_all, b0, b1);
             for (int bkt = b0; bkt <= b1; bkt++) {
                 LaunchCfg cfg;
                 r = plan_bucket(A, nq, T, p.scratch, bkt, sized_for(bkt, T, T_all), cfg,
-                                tuned_for(pc, bucket_cap(bkt), kmax));
-                if (r != ANN_OK) {
-                    cudaFree(p.scratch);
-                    return r;
-                }
+                                tuned_for(pc, bucket_cap(bkt), kmax), shrink);
+                if (r != ANN_OK) return drop(r);
                 need += cfg.bytes;
             }
-            size_t held = need;
-            for (auto &kv : pc->plans) held += kv.second.bytes;
-            while (held > kMaxPlanBytes && !pc->plans.empty()) {
-                size_t left = need;
-                r = evict();
-                if (r != ANN_OK) {
-                    cudaFree(p.scratch);
-                    return r;
-                }
-                for (auto &kv : pc->plans) left += kv.second.bytes;
-                held = left;
+            p.ws = workspace_of(pc, s, need);
+            if (p.ws) break;
+            while (held_bytes(pc) + need > kMaxPlanBytes && !pc->plans.empty())
+                if ((r = evict_plan(pc)) != ANN_OK) return drop(r);
+            p.ws = std::make_shared<Workspace>();
+            cudaError_t e = cudaEventCreateWithFlags(&p.ws->done, cudaEventDisableTiming);
+            if (e != cudaSuccess) return drop(cuda_fail(e, "cudaEventCreateWithFlags"));
+            e = cudaMalloc((void **)&p.ws->p, need);
+            if (e == cudaSuccess) {
+                p.ws->bytes = need;
+                break;
             }
-            p.bytes = need;
-            if (need) {
-                cudaError_t ae = cudaMalloc(&p.wscratch, need);
-                if (ae != cudaSuccess) {
-                    cudaFree(p.scratch);
-                    return cuda_fail(ae, "cudaMalloc(search scratch)");
-                }
-            }
+            r = cuda_fail(e, "cudaMalloc(search workspace)");
+            if (r != ANN_ERR_OOM || shrink == kMaxShrink) return drop(r);
         }
-        auto drop = [&p]() {
-            cudaFree(p.scratch);
-            if (p.wscratch) cudaFree(p.wscratch);
-        };
         cudaStream_t cap;
         cudaError_t ce = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
-        if (ce != cudaSuccess) {
-            drop();
-            return cuda_fail(ce, "cudaStreamCreateWithFlags");
-        }
+        if (ce != cudaSuccess) return drop(cuda_fail(ce, "cudaStreamCreateWithFlags"));
         cudaGraph_t graph;
         ce = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
         if (ce != cudaSuccess) {
             cudaStreamDestroy(cap);
-            drop();
-            return cuda_fail(ce, "cudaStreamBeginCapture");
+            return drop(cuda_fail(ce, "cudaStreamBeginCapture"));
         }
         int rr;
         {
             ForkSet fs;
-            rr = record_persistent(pc, A, nq, T, T_all, p.scratch, p.wscratch, p.bytes, cap, fs);
+            rr = record_persistent(pc, A, nq, T, T_all, p.scratch, p.ws->p, p.ws->bytes, shrink, cap, fs);
             ce = cudaStreamEndCapture(cap, &graph);
         }
         cudaStreamDestroy(cap);
         if (rr != ANN_OK || ce != cudaSuccess) {
             if (ce == cudaSuccess) cudaGraphDestroy(graph);
-            drop();
-            return rr != ANN_OK ? rr : cuda_fail(ce, "cudaStreamEndCapture");
+            return drop(rr != ANN_OK ? rr : cuda_fail(ce, "cudaStreamEndCapture"));
         }
         ce = cudaGraphInstantiate(&p.exec, graph, 0);
         cudaGraphDestroy(graph);
-        if (ce != cudaSuccess) {
-            drop();
-            return cuda_fail(ce, "cudaGraphInstantiate");
-        }
+        if (ce != cudaSuccess) return drop(cuda_fail(ce, "cudaGraphInstantiate"));
         it = pc->plans.emplace(key, p).first;
     }
     it->second.last_use = ++pc->clock;
-    ANN_CUDA(cudaGraphLaunch(it->second.exec, s));
+    Plan &plan = it->second;
+    Workspace &ws = *plan.ws;
+    if (ws.last && ws.last != plan.exec) ANN_CUDA(cudaStreamWaitEvent(s, ws.done, 0));
+    ANN_CUDA(cudaGraphLaunch(plan.exec, s));
+    ws.last = plan.exec;
+    ANN_CUDA(cudaEventRecord(ws.done, s));
     return ANN_OK;
 }

@@ -114,3 +114,83 @@ def test_plain_search_in_smaller_passes(ann, nq, T, mbytes):
         got = search()
     for a, b in zip(got, want):
         assert torch.equal(a, b)
+
+
+@pytest.fixture(scope="module")
+def mixed(ann):
+    N, nq = 4000, 10_000
+    X = dev(datagen.mixture(8, N, 128, 40, np.uint8))
+    Q = dev(datagen.mixture(9, nq, 128, 40, np.uint8))
+    G, _ = ann.ann_build_knn_graph(X, 10)
+    C = ann.ann_train_centers(X, 4, 24, 2, np.arange(24))
+    T = dev(np.random.default_rng(1).choice([40, 200, 500, 1000, 1500, 2500], nq).astype(np.int32))
+    want = ann.ann_search_batch(ann.Index.create(X, G, C, t=100, b=5), Q, 10, T, mode=0)[0]
+    return (lambda: ann.Index.create(X, G, C, t=100, b=5)), Q, T, want
+
+
+def taken():
+    torch.cuda.synchronize()
+    free, total = torch.cuda.mem_get_info()
+    return total - free
+
+
+def test_plans_of_one_stream_share_a_workspace(ann, mixed):
+    make, Q, T, want = mixed
+    ix, outs = make(), [torch.empty_like(want) for _ in range(12)]
+    ann.ann_search_batch(ix, Q, 10, T, mode=1)  # launch shapes are measured here
+    before = taken()
+    for turn in range(2):
+        for i, o in enumerate(outs):
+            ann.ann_search_batch(ix, Q, 10, T, mode=1, out_ids=o)
+            if (turn, i) == (0, 0):
+                first = taken() - before
+    grown = taken() - before
+    for o in outs:
+        assert torch.equal(o, want)
+    # a graph, its lists and outputs for each plan, but not a workspace (about 2 GB)
+    assert grown - first < 1 << 29, (first, grown)
+    # other streams side by side, each with a workspace of its own
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    torch.cuda.synchronize()
+    for o in outs:
+        o.zero_()
+    torch.cuda.synchronize()
+    for _ in range(3):
+        for i, o in enumerate(outs):
+            ann.ann_search_batch(ix, Q, 10, T, mode=1, out_ids=o, stream=streams[i % 3])
+    torch.cuda.synchronize()
+    for o in outs:
+        assert torch.equal(o, want)
+    ix.free()
+
+
+def test_workspaces_of_many_streams_are_bounded(ann, mixed):
+    make, Q, T, want = mixed
+    ix, streams = make(), [torch.cuda.Stream() for _ in range(14)]
+    before = taken()
+    outs = [torch.empty_like(want) for _ in streams]
+    torch.cuda.synchronize()
+    for _ in range(2):
+        for s, o in zip(streams, outs):
+            ann.ann_search_batch(ix, Q, 10, T, mode=1, out_ids=o, stream=s)
+    # 14 workspaces of about 2 GB do not fit in 16 GB: the least recently used plans went
+    assert taken() - before < (16 << 30) + (1 << 30)
+    for o in outs:
+        assert torch.equal(o, want)
+    ix.free()
+
+
+def test_a_plan_in_what_memory_is_left(ann, mixed):
+    make, Q, T, want = mixed
+    torch.cuda.empty_cache()
+    ix = make()
+    ann.ann_search_batch(ix, Q[:3000], 10, T[:3000], mode=1)  # launch shapes are measured here
+    torch.cuda.synchronize()
+    rest = torch.empty(torch.cuda.mem_get_info()[0] - (5 << 28), dtype=torch.uint8, device="cuda")  # leaves 1.25 GB
+    out = torch.empty_like(want)
+    ann.ann_search_batch(ix, Q, 10, T, mode=1, out_ids=out)
+    torch.cuda.synchronize()
+    del rest
+    torch.cuda.empty_cache()
+    assert torch.equal(out, want)
+    ix.free()
