@@ -282,9 +282,11 @@ enum {
  * one stream share a workspace, which holds a plain search's for each bucket
  * in use, with a quarter of its states (10,000 queries with budgets up to
  * 8192: about 2 GB); where it cannot be had, passes are smaller.  The
- * first call that meets a (budget bucket, kmax) measures candidate launch
- * shapes on the batch itself and keeps the fastest for the index; that call
- * synchronizes `stream` and runs the batch a few times.
+ * first call in which a (budget bucket, kmax) runs in one of its forms (by
+ * the batch's size; batches that the device holds at once have no choice)
+ * measures candidate launch shapes on the batch itself and keeps the fastest
+ * for the index; that call synchronizes `stream` and runs the batch a few
+ * times.
  * Results are identical in both modes and for every launch shape.
  * Asynchronous except as stated. */
 int ann_search_batch(const ann_index *index, const void *queries, int64_t nq, const int32_t *k,

@@ -173,7 +173,8 @@ static int plan_launch(const SearchArgs &base, int capT, const int32_t *list, co
     // resident with everything in shared memory, that is the shorter chain (no
     // visited-set probe in L2 at every step): 128 queries of SIFT-shaped rows,
     // T = 1024 / 2048 / 4096: 0.88 / 2.58 / 17.3 -> 0.68 / 2.05 / 14.3 ms.
-    cfg.main.L = main_layout(ix.dtype, ix.d, capT, A.kmax, ix.b, ix.R, tn.stage, false, (uint32_t)tn.spill_heap);
+    // (the form of a launch does not depend on how its main loop is tuned)
+    cfg.main.L = main_layout(ix.dtype, ix.d, capT, A.kmax, ix.b, ix.R, true, false, (uint32_t)tn.spill_heap);
     const int64_t fit = (int64_t)(g_smem_optin / (cfg.main.L.total + 1024)) * g_num_sms;
     // bridge batch: budgets below the windowed kernels pop few bridges
     auto res_layout = [&](bool w, bool split) {
@@ -363,7 +364,7 @@ struct Workspace {
 
 struct Plan {
     cudaGraphExec_t exec = nullptr;
-    int32_t *scratch = nullptr;     // counts[kBuckets], then lists[kBuckets*nq]
+    int32_t *scratch = nullptr;     // counts[kBuckets], lists[kBuckets*nq], then a word for autotune()
     std::shared_ptr<Workspace> ws;  // the buckets' workspaces, one after another
     uint64_t last_use = 0;          // for evicting the least recently used plan
 };
@@ -393,7 +394,8 @@ struct PlanCache {
     std::mutex mu;
     uint64_t clock = 0;
     std::map<PlanKey, Plan> plans;
-    std::map<std::pair<int, int>, Tune> tuned;  // (bucket capacity, kmax) -> measured best launch shape
+    // measured best launch shape of (bucket capacity, kmax, LaunchCfg::win, LaunchCfg::wide)
+    std::map<std::tuple<int, int, bool, bool>, Tune> tuned;
 };
 
 void free_plans(ann_index *ix) {
@@ -447,16 +449,17 @@ static void bucket_range(const int32_t *T, int32_t T_all, int &b0, int &b1) {
     b0 = T ? 0 : b1;
 }
 
-static const Tune *tuned_for(const PlanCache *pc, int capT, int kmax) {
-    auto it = pc->tuned.find({capT, kmax});
-    return it == pc->tuned.end() ? nullptr : &it->second;
-}
-
 static int bucket_cap(int bkt) { return (128 << bkt) > kMaxT ? kMaxT : (128 << bkt); }
 
 // the budget a bucket's kernels are sized for: a uniform one is known
 static int sized_for(int bkt, const int32_t *T, int32_t T_all) {
     return T ? bucket_cap(bkt) : std::max(32, std::min((int)T_all, bucket_cap(bkt)));
+}
+
+// the main loop's launch shape that was measured for a bucket run in cfg's form
+static Tune *tuned_for(PlanCache *pc, int bkt, const LaunchCfg &cfg) {
+    auto it = pc->tuned.find({bucket_cap(bkt), cfg.A.kmax, cfg.win, cfg.wide});
+    return it == pc->tuned.end() ? nullptr : &it->second;
 }
 
 // One replay of the persistent form.  A uniform budget is one bucket and the
@@ -478,14 +481,19 @@ struct ForkSet {
     }
 };
 
-// one bucket's launch: the whole batch in order, or (per-query T) its list
-static int plan_bucket(const SearchArgs &A, int64_t nq, const int32_t *T, int32_t *scratch, int bkt, int capT,
-                       LaunchCfg &cfg, const Tune *tn, int shrink) {
-    if (!T) return plan_launch(A, capT, nullptr, nullptr, nq, cfg, tn, shrink);
-    return plan_launch(A, capT, scratch + kBuckets + (int64_t)bkt * nq, scratch + bkt, nq, cfg, tn, shrink);
+// one bucket's launch, in its measured shape if it has one: the whole batch in
+// order, or (per-query T) its list
+static int plan_bucket(PlanCache *pc, const SearchArgs &A, int64_t nq, const int32_t *T, int32_t T_all,
+                       int32_t *scratch, int bkt, LaunchCfg &cfg, int shrink) {
+    const int capT = sized_for(bkt, T, T_all);
+    const int32_t *list = T ? scratch + kBuckets + (int64_t)bkt * nq : nullptr, *count = T ? scratch + bkt : nullptr;
+    int r = plan_launch(A, capT, list, count, nq, cfg, nullptr, shrink);
+    if (r != ANN_OK || cfg.whole) return r;
+    const Tune *tn = tuned_for(pc, bkt, cfg);
+    return tn ? plan_launch(A, capT, list, count, nq, cfg, tn, shrink) : ANN_OK;
 }
 
-static int record_persistent(const PlanCache *pc, const SearchArgs &A, int64_t nq, const int32_t *T, int32_t T_all,
+static int record_persistent(PlanCache *pc, const SearchArgs &A, int64_t nq, const int32_t *T, int32_t T_all,
                              int32_t *scratch, uint8_t *wscratch, size_t wbytes, int shrink, cudaStream_t s,
                              ForkSet &fs) {
     int32_t *counts = scratch, *lists = scratch + kBuckets;
@@ -498,10 +506,8 @@ static int record_persistent(const PlanCache *pc, const SearchArgs &A, int64_t n
     bucket_range(T, T_all, b0, b1);
     int rc = ANN_OK;
     for (int bkt = b1; bkt >= b0 && rc == ANN_OK; bkt--) {
-        const int capT = sized_for(bkt, T, T_all);
-        const Tune *tn = tuned_for(pc, bucket_cap(bkt), A.kmax);
         LaunchCfg cfg;
-        rc = plan_bucket(A, nq, T, scratch, bkt, capT, cfg, tn, shrink);
+        rc = plan_bucket(pc, A, nq, T, T_all, scratch, bkt, cfg, shrink);
         if (rc != ANN_OK) break;
         if (cfg.bytes > wbytes) {
             rc = fail(ANN_ERR_CAPACITY, "search workspace smaller than its kernels need");
@@ -547,24 +553,32 @@ static int record_persistent(const PlanCache *pc, const SearchArgs &A, int64_t n
 // staging, and, for large budgets, other shared-memory heap capacities (a
 // smaller heap leaves room for more resident queries, a larger one moves
 // entries out less often).  All give identical results.
-static std::vector<Tune> tune_candidates(int capT) {
+static std::vector<Tune> tune_candidates(int capT, bool win) {
     std::vector<Tune> c{Tune{kMainWarps, true}, Tune{kMainWarps / 2, true}, Tune{kMainWarps, false}};
-    if (capT >= kWindowedFromT)
+    if (win)
         for (int hc : {256, 1024})
             if (hc < capT) c.push_back(Tune{kMainWarps, true, hc});
     return c;
 }
 
-// Measure the candidates of every bucket this batch uses that has no measured
-// choice yet, on (a prefix of) the batch itself, and keep the fastest.
+// Measure the candidates of every bucket this batch uses whose form has no
+// measured choice yet, on (a prefix of) the batch itself, and keep the fastest.
+// They are planned as the replay will be, for the batch's size; a device count
+// keeps a run to its share of the queries.
 static int autotune(PlanCache *pc, const SearchArgs &A, int64_t nq, const int32_t *T, int32_t T_all,
                     int32_t *scratch, cudaStream_t s) {
     int b0, b1;
     bucket_range(T, T_all, b0, b1);
-    bool todo = false;
-    for (int bkt = b0; bkt <= b1; bkt++) todo |= tuned_for(pc, bucket_cap(bkt), A.kmax) == nullptr;
-    if (!todo) return ANN_OK;
-    int32_t *counts = scratch, *lists = scratch + kBuckets;
+    LaunchCfg c0[kBuckets];  // the default shapes
+    bool todo[kBuckets] = {}, any = false;
+    for (int bkt = b0; bkt <= b1; bkt++) {
+        const int r = plan_launch(A, sized_for(bkt, T, T_all), nullptr, nullptr, nq, c0[bkt]);
+        if (r != ANN_OK) return r;
+        todo[bkt] = !c0[bkt].whole && !tuned_for(pc, bkt, c0[bkt]);  // whole: the main loop's shape is not used
+        any |= todo[bkt];
+    }
+    if (!any) return ANN_OK;
+    int32_t *counts = scratch, *lists = scratch + kBuckets, *tcount = lists + (int64_t)kBuckets * nq;
     int32_t hc[kBuckets] = {0};
     if (T) {
         ANN_CUDA(cudaMemsetAsync(counts, 0, sizeof(int32_t) * kBuckets, s));
@@ -580,24 +594,23 @@ static int autotune(PlanCache *pc, const SearchArgs &A, int64_t nq, const int32_
     ANN_CUDA(cudaEventCreate(&e1));
     int rc = ANN_OK;
     for (int bkt = b0; bkt <= b1 && rc == ANN_OK; bkt++) {
+        if (!todo[bkt] || hc[bkt] == 0) continue;
         const int capT = sized_for(bkt, T, T_all);
-        if (tuned_for(pc, bucket_cap(bkt), A.kmax) || hc[bkt] == 0) continue;
-        const std::vector<Tune> cands = tune_candidates(capT);
+        const std::vector<Tune> cands = tune_candidates(capT, c0[bkt].win);
         const int32_t *list = T ? lists + (int64_t)bkt * nq : nullptr;
         // tune on up to four rounds of the default shape's resident warps
-        LaunchCfg c0;
-        rc = plan_launch(A, capT, list, nullptr, hc[bkt], c0, &cands[0]);
-        if (rc != ANN_OK) break;
-        if (c0.whole) {  // the main loop's shape is not used
-            pc->tuned[{bucket_cap(bkt), A.kmax}] = cands[0];
-            continue;
+        const int32_t ntune = (int32_t)std::min<int64_t>(std::min<int64_t>(hc[bkt], c0[bkt].chunk),
+                                                         4 * (int64_t)c0[bkt].main.warps);
+        if (cudaMemcpyAsync(tcount, &ntune, sizeof(ntune), cudaMemcpyHostToDevice, s) != cudaSuccess) {
+            rc = cuda_fail(cudaGetLastError(), "autotune count");
+            break;
         }
-        const int64_t ntune = std::min<int64_t>(std::min<int64_t>(hc[bkt], kChunk), 4 * (int64_t)c0.main.warps);
         float best_ms = 0.f;
         int best = -1;
         for (size_t ci = 0; ci < cands.size() && rc == ANN_OK; ci++) {
             LaunchCfg cfg;
-            if (plan_launch(A, capT, list, nullptr, ntune, cfg, &cands[ci]) != ANN_OK) continue;
+            if (plan_launch(A, capT, list, tcount, nq, cfg, &cands[ci]) != ANN_OK || cfg.whole) continue;
+            cfg.total = cfg.chunk;  // the run's queries are in the first pass
             uint8_t *ws = nullptr;
             if (cudaMallocAsync((void **)&ws, cfg.bytes, s) != cudaSuccess) continue;
             float ms_min = 0.f;
@@ -624,7 +637,8 @@ static int autotune(PlanCache *pc, const SearchArgs &A, int64_t nq, const int32_
             }
         }
         cudaGetLastError();  // a candidate that failed to configure is simply not chosen
-        if (rc == ANN_OK) pc->tuned[{bucket_cap(bkt), A.kmax}] = cands[best < 0 ? 0 : best];
+        if (rc == ANN_OK && best >= 0)
+            pc->tuned[{bucket_cap(bkt), A.kmax, c0[bkt].win, c0[bkt].wide}] = cands[best];
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -725,7 +739,7 @@ extern "C" int ann_search_batch(const ann_index *index, const void *queries, int
     }
     if (it == pc->plans.end()) {
         Plan p;
-        ANN_CUDA(cudaMalloc(&p.scratch, sizeof(int32_t) * (kBuckets + (size_t)kBuckets * nq)));
+        ANN_CUDA(cudaMalloc(&p.scratch, sizeof(int32_t) * (kBuckets + (size_t)kBuckets * nq + 1)));
         auto drop = [&p](int code) {
             cudaFree(p.scratch);
             return code;
@@ -738,8 +752,7 @@ extern "C" int ann_search_batch(const ann_index *index, const void *queries, int
             size_t need = 0;
             for (int bkt = b0; bkt <= b1; bkt++) {
                 LaunchCfg cfg;
-                r = plan_bucket(A, nq, T, p.scratch, bkt, sized_for(bkt, T, T_all), cfg,
-                                tuned_for(pc, bucket_cap(bkt), kmax), shrink);
+                r = plan_bucket(pc, A, nq, T, T_all, p.scratch, bkt, cfg, shrink);
                 if (r != ANN_OK) return drop(r);
                 need += cfg.bytes;
             }

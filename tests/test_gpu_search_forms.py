@@ -3,6 +3,8 @@ resumed queries; smaller ones as one kernel from start to end.  Both give the
 same results, counters included, and the oracle's on a sample."""
 from __future__ import annotations
 
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -87,3 +89,35 @@ def test_rows_as_wide_as_shared_memory(ann, d, T, nq):
         torch.cuda.synchronize()
         assert not status.any()
         np.testing.assert_array_equal(got.cpu().numpy()[sel], want)
+
+
+def test_launch_shapes_are_measured_for_the_form_that_runs(ann):
+    # the runs that measure take their workspace from the device's memory pool, recorded plans do not: the pool's mark
+    # shows which call measured
+    cu, pool = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p()
+    torch.zeros(1, device="cuda")
+    assert cu.cuDeviceGetDefaultMemPool(ctypes.byref(pool), torch.cuda.current_device()) == 0
+    N, nq = 4000, 6000
+    X, Q = dev(datagen.mixture(1, N, 64, 10, np.uint8)), dev(datagen.mixture(2, nq, 64, 10, np.uint8))
+    G, _ = ann.ann_build_knn_graph(X, 10)
+    ix = ann.Index.create(X, G, ann.ann_train_centers(X, 4, 16, 2, np.arange(16)), t=100, b=5)
+
+    def measures(q, T):
+        mark = ctypes.c_uint64(0)
+        torch.cuda.synchronize()
+        assert cu.cuMemPoolSetAttribute(pool, 8, ctypes.byref(mark)) == 0  # CU_MEMPOOL_ATTR_USED_MEM_HIGH
+        ids, _, _ = ann.ann_search_batch(ix, q, 10, T, mode=1)
+        torch.cuda.synchronize()
+        assert cu.cuMemPoolGetAttribute(pool, 8, ctypes.byref(mark)) == 0
+        assert torch.equal(ids, ann.ann_search_batch(ix, q, 10, T, mode=0)[0])
+        return mark.value > 0
+
+    assert not measures(Q[:1], 600)   # one kernel alone: nothing to choose
+    assert measures(Q, 600)
+    assert not measures(Q, 700)       # the same bucket and form
+    assert measures(Q, 1024)          # the same bucket, but queues that spill
+    T = torch.full((nq,), 600, dtype=torch.int32, device="cuda")
+    T[:100] = 3000                    # a bucket smaller than what one kernel holds, in a batch that is not
+    assert measures(Q, T)
+    assert not measures(Q, 3000)
+    ix.free()
