@@ -283,7 +283,8 @@ enum {
  * in use, with a quarter of its states (10,000 queries with budgets up to
  * 8192: about 2 GB); where it cannot be had, passes are smaller.  The
  * first call in which a (budget bucket, kmax) runs in one of its forms (by
- * the batch's size; batches that the device holds at once have no choice)
+ * the batch's size; batches that the device holds at once have no choice,
+ * and buckets with fewer queries than that leave it to a later call)
  * measures candidate launch shapes on the batch itself and keeps the fastest
  * for the index; that call synchronizes `stream` and runs the batch a few
  * times.

@@ -561,7 +561,7 @@ static std::vector<Tune> tune_candidates(int capT, bool win) {
     return c;
 }
 
-// Measure the candidates of every bucket this batch uses whose form has no
+// Measure the candidates of every bucket this batch fills whose form has no
 // measured choice yet, on (a prefix of) the batch itself, and keep the fastest.
 // They are planned as the replay will be, for the batch's size; a device count
 // keeps a run to its share of the queries.
@@ -594,7 +594,10 @@ static int autotune(PlanCache *pc, const SearchArgs &A, int64_t nq, const int32_
     ANN_CUDA(cudaEventCreate(&e1));
     int rc = ANN_OK;
     for (int bkt = b0; bkt <= b1 && rc == ANN_OK; bkt++) {
-        if (!todo[bkt] || hc[bkt] == 0) continue;
+        // a list shorter than one round of the resident warps takes as long as its
+        // longest queries in every shape (2,000 GIST-shaped queries over seven
+        // buckets: 26 ms, 315 ms to measure them, 26 ms after): left open
+        if (!todo[bkt] || (T && hc[bkt] < c0[bkt].main.warps)) continue;
         const int capT = sized_for(bkt, T, T_all);
         const std::vector<Tune> cands = tune_candidates(capT, c0[bkt].win);
         const int32_t *list = T ? lists + (int64_t)bkt * nq : nullptr;

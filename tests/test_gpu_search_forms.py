@@ -117,7 +117,9 @@ def test_launch_shapes_are_measured_for_the_form_that_runs(ann):
     assert not measures(Q, 700)       # the same bucket and form
     assert measures(Q, 1024)          # the same bucket, but queues that spill
     T = torch.full((nq,), 600, dtype=torch.int32, device="cuda")
-    T[:100] = 3000                    # a bucket smaller than what one kernel holds, in a batch that is not
-    assert measures(Q, T)
+    assert not measures(Q, T)         # sized for its bucket, as budgets of 1024 are
+    T[:100] = 3000                    # a bucket with too few queries to tell: left to a batch that fills it
+    assert not measures(Q, T)
+    assert measures(Q, 3000)
     assert not measures(Q, 3000)
     ix.free()
