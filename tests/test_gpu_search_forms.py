@@ -123,3 +123,27 @@ def test_launch_shapes_are_measured_for_the_form_that_runs(ann):
     assert measures(Q, 3000)
     assert not measures(Q, 3000)
     ix.free()
+
+
+@pytest.mark.parametrize("mode,T", [(0, 40), (1, 40), (0, 1200), (1, "mixed")])
+def test_batches_of_more_than_one_pass(ann, mode, T):
+    # records and first batches are held for 32,768 queries at a time; with budgets of their own the lists of queries are
+    # counted on the device, and one of them ends in the second pass
+    N, nq = 3000, 33_001
+    X, Q = dev(datagen.mixture(3, N, 64, 30, np.uint8)), dev(datagen.mixture(4, nq, 64, 30, np.uint8))
+    G, _ = ann.ann_build_knn_graph(X, 8)
+    ix = ann.Index.create(X, G, ann.ann_train_centers(X, 4, 16, 2, np.arange(16)), t=50, b=5)
+    if T == "mixed":
+        T = torch.full((nq,), 90, dtype=torch.int32, device="cuda")
+        T[5:nq:400] = 300
+    for _ in range(2):
+        got = ann.ann_search_batch(ix, Q, 10, T, mode=mode)
+        torch.cuda.synchronize()
+        for lo in range(0, nq, 6000):
+            part = T[lo:lo + 6000].contiguous() if torch.is_tensor(T) else T
+            want = ann.ann_search_batch(ix, Q[lo:lo + 6000].contiguous(), 10, part, mode=0)
+            for a, b in zip(got, want):
+                assert torch.equal(a[lo:lo + 6000], b)
+        for a in got:
+            a.zero_()
+    ix.free()
