@@ -400,6 +400,14 @@ def algorithmic_bytes(stats: np.ndarray, W) -> float:
     return float(per_q.sum() + centers)
 
 
+def search_launches(torch, nq, steps):
+    """Kernels in `steps` replays of a uniform-budget batch: prologue, main and resuming kernel for every pass of 32,768
+    queries.  None for batches that the resuming kernel may hold alone (it runs at most 12 warps per SM)."""
+    if nq <= 12 * torch.cuda.get_device_properties(0).multi_processor_count:
+        return None
+    return 3 * -(-nq // 32768) * steps
+
+
 def search_kernel_digest() -> str:
     """sha256 over the search kernel's device sources (the DRAM traffic in
     profiles/ is valid only for the kernel it was measured on)."""
@@ -639,8 +647,7 @@ def measure(args, rank, ws, log, torch, ann, datagen, W, headline):
         "search_stats_mean_per_query": search_stats,
         "cpu_baseline": cpu_baseline,
         "clocks": clocks,
-        # uniform budget, one pass: prologue, main and resuming kernel per replayed graph
-        "gpu_launches": 3 * args.steps,
+        "gpu_launches": search_launches(torch, nq, args.steps),
         "index": {**{k: W["info"][k] for k in ("M", "bridged_refs", "alpha", "bytes_vectors", "bytes_graph",
                                                "bytes_bridges")}, "build_s": W["build_s"]},
     }
