@@ -1034,6 +1034,8 @@ extern "C" int ann_train_centers(const void *train, int dtype, int64_t ntrain, i
     ANN_CUDA(cudaGetDevice(&dev));
     ANN_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     ANN_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    // the longest part that is accepted (128 rows of it as float32 in shared
+    // memory): a limit of this call, none of the kernels below needs it
     if (dp > optin / 512) return fail(ANN_ERR_CUDA, "a part has too many dimensions");
     const int total = P * n * dp;
     DBuf<double> C;

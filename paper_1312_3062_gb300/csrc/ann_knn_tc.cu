@@ -704,7 +704,8 @@ size_t smem_bytes(int d) {
 // smallest makespan, waves x (tiles per range + what a new range costs in
 // tiles: the query rows' load and the insertions until its limits settle).
 // 10,000 queries are 79 blocks, half the SMs of this part; split 25 ways they
-// make 13 full waves.
+// make 13 full waves.  At most 64 ranges: each keeps two lists of k pairs per
+// query row, 33 KB a row at k = 32; so calls of up to 128 queries use 64 SMs.
 int choose_split(int64_t nblocks, int64_t ntiles, int nsm, int k) {
     const int64_t extra = 8 + k;
     int best = 1;

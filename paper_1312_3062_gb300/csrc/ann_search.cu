@@ -255,7 +255,8 @@ static int plan_launch(const SearchArgs &base, int capT, const int32_t *list, co
     return ANN_OK;
 }
 
-// the three kernels of passes over the queries; stages: how many of them to launch (3 = all)
+// the kernels of every pass over the queries: number first .. last of the three,
+// or the resuming one alone
 static int do_launch(LaunchCfg &cfg, uint8_t *ws, cudaStream_t stream, int first = 0, int last = 2) {
     SearchArgs &A = cfg.A;
     const bool u8 = A.ix.dtype == ANN_U8, grouped = A.ix.ngroups > 0;
@@ -462,11 +463,6 @@ static Tune *tuned_for(PlanCache *pc, int bkt, const LaunchCfg &cfg) {
     return it == pc->tuned.end() ? nullptr : &it->second;
 }
 
-// One replay of the persistent form.  A uniform budget is one bucket and the
-// queries are taken in order; otherwise a device pass sorts them into buckets
-// first.  The buckets run concurrently on forked streams (largest budget
-// first), each with a workspace of its own: a bucket's last queries leave most
-// SMs idle, above all those that pop many bridges.
 // streams and events of the fork/join; they must outlive the capture
 struct ForkSet {
     cudaStream_t side[kBuckets] = {};
@@ -493,6 +489,11 @@ static int plan_bucket(PlanCache *pc, const SearchArgs &A, int64_t nq, const int
     return tn ? plan_launch(A, capT, list, count, nq, cfg, tn, shrink) : ANN_OK;
 }
 
+// One replay of the persistent form.  A uniform budget is one bucket and the
+// queries are taken in order; otherwise a device pass sorts them into buckets
+// first.  The buckets run concurrently on forked streams (largest budget
+// first), each with a workspace of its own: a bucket's last queries leave most
+// SMs idle, above all those that pop many bridges.
 static int record_persistent(PlanCache *pc, const SearchArgs &A, int64_t nq, const int32_t *T, int32_t T_all,
                              int32_t *scratch, uint8_t *wscratch, size_t wbytes, int shrink, cudaStream_t s,
                              ForkSet &fs) {
@@ -713,7 +714,7 @@ extern "C" int ann_search_batch(const ann_index *index, const void *queries, int
     A.out_status = out_status;
     A.out_stats = out_stats;
     if (mode == ANN_MODE_PLAIN) {
-        // one launch sized for the largest budget in the batch
+        // sized for the largest budget in the batch
         int capT = T_all;
         if (T) {
             int32_t *dmax = nullptr, hmax = 0;

@@ -102,7 +102,7 @@ __host__ __device__ inline WarpLayout make_layout(int dtype, int d, int P, int n
     L.sc_parts = spill || split ? (uint32_t)P : (uint32_t)PA;
     L.sc = o;     o = align_up(o + L.sc_parts * n, 16);
     uint32_t lpn = 1;
-    while (lpn < (uint32_t)n) lpn <<= 1;  // the per-part sort borrows the heap region
+    while (lpn < (uint32_t)n) lpn <<= 1;  // the queue holds at least n entries
     const uint32_t qcap = spill && (uint32_t)capT > spill_heap ? spill_heap : (uint32_t)capT;
     uint32_t hc = qcap > lpn ? qcap : lpn;
     L.heap_cap = hc;
@@ -779,7 +779,7 @@ struct WalkState {
     bool first;       // nothing produced yet (lo meaningless)
     bool exhausted;   // all non-empty bridges produced
     uint32_t width;   // window width in key units (u8) or key-bit units (f32)
-    uint32_t kmin, kmaxall, msuf;
+    uint32_t kmin, kmaxall;
     uint32_t gpos, gcnt;  // sorted window in global scratch: next entry, entries
     int gbuf;             // which of the two scratch buffers holds it
 };
@@ -1510,7 +1510,7 @@ __device__ uint32_t refill_windowed(const DevIndex &ix, uint8_t *smem, const War
                 uint64_t h2 = base + span / 2;
                 while (true) {
                     c = walk<DT, 4, GRP>(ix, smem, L, ws.lo, ws.first, h2, gk0, gv0, gcap);
-                                if (c <= gcap) break;
+                    if (c <= gcap) break;
                     span = h2 - base;
                     if (span == 0) { cap_err = true; return 0; }
                     h2 = base + span / 2;
@@ -2074,7 +2074,7 @@ __device__ void search_one(const SearchArgs &A, uint8_t *smem, int64_t w, uint8_
             if (stats && lane == 0) stat[0] = max(stat[0], hsz + sp.nb + 1);
         }
         // The next pop is known now.  When it is a reference, take its kNN row
-        // (usually the speculative one) and start copying its unvisited
+        // (usually prefetched) and start copying its unvisited
         // neighbours' vectors, so both overlap the rest of this step and the
         // next pop.
         if (t + m < T && hsz > 0) {
