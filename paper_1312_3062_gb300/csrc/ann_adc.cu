@@ -90,27 +90,12 @@ __global__ void __launch_bounds__(ENC_THREADS) pq_encode_kernel(const void *__re
     codes[i * m + j] = (uint8_t)arg;
 }
 
-// two float32 operations per instruction, each rounded as the single ones are
-__device__ __forceinline__ uint64_t f2(float a, float b) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b) {  // a + (-b): the rounded difference
-    uint64_t r;
-    asm("{\n .reg .b64 t;\n xor.b64 t, %2, 0x8000000080000000;\n add.rn.f32x2 %0, %1, t;\n}" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
 // The products are single ones: a two-wide multiply and the two-wide add after
 // it came back as one fused operation, without the product's rounding.
-__device__ __forceinline__ uint64_t f2_square(uint64_t a) {
-    const float x = __uint_as_float((uint32_t)a), y = __uint_as_float((uint32_t)(a >> 32));
-    return f2(__fmul_rn(x, x), __fmul_rn(y, y));
+__device__ __forceinline__ uint64_t square2(uint64_t a) {
+    float x, y;
+    unpack2(a, x, y);
+    return pack2(__fmul_rn(x, x), __fmul_rn(y, y));
 }
 
 // Keep T of the n values in buf (n > T), the smallest ones, in any order: the
@@ -252,15 +237,15 @@ __global__ void __launch_bounds__(RR_THREADS) adc_rerank_kernel(
                     const float rb[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
                     for (int u = 0; u < 4; u++) {
-                        const uint64_t ee = f2_sub(f2(ra[u], rb[u]), f2(ww[u], ww[u]));
-                        s2 = f2_add(s2, f2_square(ee));
+                        const uint64_t ee = sub2(pack2(ra[u], rb[u]), pack2(ww[u], ww[u]));
+                        s2 = add2(s2, square2(ee));
                     }
                 }
             } else {
                 for (int t = 0; t < dp; t++) {
                     const float wt = __ldg(cw + t);
-                    const uint64_t ee = f2_sub(f2(r0[t], NL == 2 ? r0[d + t] : 0.f), f2(wt, wt));
-                    s2 = f2_add(s2, f2_square(ee));
+                    const uint64_t ee = sub2(pack2(r0[t], NL == 2 ? r0[d + t] : 0.f), pack2(wt, wt));
+                    s2 = add2(s2, square2(ee));
                 }
             }
             table[e] = __uint_as_float((uint32_t)s2);

@@ -187,6 +187,31 @@ __device__ __forceinline__ uint32_t part_key_wide(const uint8_t *qbytes, const v
 }
 
 // ---------------------------------------------------------------------------
+// two float32 operations per instruction, each rounded as the single ones are
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {  // a + (-b): the rounded difference
+    return add2(a, b ^ 0x8000000080000000ull);
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// ---------------------------------------------------------------------------
 // bridge-key arithmetic (Sec. 4.2: the bridge key is the sum over parts of the
 // part keys).  uint8: exact integer sums.  float32: the key is the float32
 // nearest to the EXACT sum of the float32 part keys (ties to even), one

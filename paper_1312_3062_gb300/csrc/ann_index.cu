@@ -113,26 +113,6 @@ __global__ void km_prep_kernel(const double *C, int n, int dp, float *cneg, floa
     if (threadIdx.x == 0) cmax[blockIdx.x] = red[0];
 }
 
-// two float32 operations per instruction, each rounded as the single ones are
-__device__ __forceinline__ uint64_t pack2(float a, float b) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float &a, float &b) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-
 // Bound by float32 issue.  A CTA takes 8 x (256 / TX) rows against tiles of
 // 8 x TX centers; a thread holds 8 x 8 distances (two centers to a register
 // pair), so every dimension costs it 4 16-byte shared loads for 64 add + 64
