@@ -114,6 +114,37 @@ def stream_ptr(stream) -> int | None:
     return stream.cuda_stream
 
 
+def _torch_stream(stream, device):
+    """The torch stream of a call's `stream` argument (None: the default stream)."""
+    import torch
+    if stream is None:
+        return torch.cuda.default_stream(device)
+    return torch.cuda.ExternalStream(stream, device=device) if isinstance(stream, int) else stream
+
+
+def _alloc(stream, device, *specs):
+    """One tensor per (shape, dtype), for a call on `stream`: taken from that stream's memory, so that a block of which
+    another stream still has work, or one that is given back while the call runs, is never shared with it.  The caller's
+    current stream may use them too."""
+    import torch
+    if not specs:
+        return []
+    cur = torch.cuda.current_stream(device)
+    if (stream_ptr(stream) or 0) == cur.cuda_stream:
+        return [torch.empty(shape, dtype=dt, device=device) for shape, dt in specs]
+    with torch.cuda.stream(_torch_stream(stream, device)):
+        out = [torch.empty(shape, dtype=dt, device=device) for shape, dt in specs]
+    for t in out:
+        t.record_stream(cur)
+    return out
+
+
+def _outputs(stream, device, *given):
+    """Outputs of a call on `stream`: (tensor or None, shape, dtype) each; those not given are allocated."""
+    new = iter(_alloc(stream, device, *((shape, dt) for t, shape, dt in given if t is None)))
+    return [next(new) if t is None else t for t, _, _ in given]
+
+
 def dtype_code(t) -> int:
     import torch
     if t.dtype == torch.uint8:
@@ -129,11 +160,8 @@ def ann_exact_knn(refs, queries, k, exclude_self=False, out_ids=None, out_keys=N
     import torch
     N, d = refs.shape
     nq = queries.shape[0]
-    if out_ids is None:
-        out_ids = torch.empty((nq, k), dtype=torch.int32, device=refs.device)
-    if out_keys is None:
-        out_keys = torch.empty((nq, k), dtype=torch.int32 if refs.dtype == torch.uint8 else torch.float32,
-                               device=refs.device)
+    out_ids, out_keys = _outputs(stream, refs.device, (out_ids, (nq, k), torch.int32),
+                                 (out_keys, (nq, k), torch.int32 if refs.dtype == torch.uint8 else torch.float32))
     check(lib.ann_exact_knn(ptr(refs), N, ptr(queries), nq, dtype_code(refs), d, k, int(exclude_self),
                             ptr(out_ids), ptr(out_keys), stream_ptr(stream)))
     return out_ids, out_keys
@@ -142,11 +170,8 @@ def ann_exact_knn(refs, queries, k, exclude_self=False, out_ids=None, out_keys=N
 def ann_build_knn_graph(data, R, out_ids=None, out_keys=None, stream=None):
     import torch
     N, d = data.shape
-    if out_ids is None:
-        out_ids = torch.empty((N, R), dtype=torch.int32, device=data.device)
-    if out_keys is None:
-        out_keys = torch.empty((N, R), dtype=torch.int32 if data.dtype == torch.uint8 else torch.float32,
-                               device=data.device)
+    out_ids, out_keys = _outputs(stream, data.device, (out_ids, (N, R), torch.int32),
+                                 (out_keys, (N, R), torch.int32 if data.dtype == torch.uint8 else torch.float32))
     check(lib.ann_build_knn_graph(ptr(data), dtype_code(data), N, d, R, ptr(out_ids), ptr(out_keys),
                                   stream_ptr(stream)))
     return out_ids, out_keys
@@ -160,10 +185,7 @@ def ann_build_knn_graph_approx(data, R, dirs, iters, out_ids=None, out_keys=None
     levels = (nseg + 1).bit_length() - 1
     if (1 << levels) - 1 != nseg or dirs.shape[2] != d:
         raise ValueError("dirs must have shape (rounds, 2^levels - 1, d)")
-    if out_ids is None:
-        out_ids = torch.empty((N, R), dtype=torch.int32, device=data.device)
-    if out_keys is None:
-        out_keys = torch.empty((N, R), dtype=torch.int32, device=data.device)
+    out_ids, out_keys = _outputs(stream, data.device, (out_ids, (N, R), torch.int32), (out_keys, (N, R), torch.int32))
     check(lib.ann_build_knn_graph_approx(ptr(data), dtype_code(data), N, d, R, ptr(dirs) if nseg else None,
                                          rounds, levels, iters, ptr(out_ids), ptr(out_keys), stream_ptr(stream)))
     return out_ids, out_keys
@@ -174,8 +196,7 @@ def ann_pq_encode(data, centers, assign, codebooks, out=None, stream=None):
     import torch
     N, d = data.shape
     m, ks, _ = codebooks.shape
-    if out is None:
-        out = torch.empty((N, m), dtype=torch.uint8, device=data.device)
+    (out,) = _outputs(stream, data.device, (out, (N, m), torch.uint8))
     check(lib.ann_pq_encode(ptr(data), dtype_code(data), N, d, ptr(centers), centers.shape[0], ptr(assign), m, ks,
                             ptr(codebooks), ptr(out), stream_ptr(stream)))
     return out
@@ -187,9 +208,8 @@ def ann_adc_rerank(queries, lists, offsets, members, centers, codes, codebooks, 
     nq, d = queries.shape
     w = lists.shape[1]
     m, ks, _ = codebooks.shape
-    ids = torch.empty((nq, T), dtype=torch.int32, device=queries.device)
-    keys = torch.empty((nq, T), dtype=torch.float32, device=queries.device)
-    seen = torch.empty((nq,), dtype=torch.int64, device=queries.device)
+    ids, keys, seen = _alloc(stream, queries.device, ((nq, T), torch.int32), ((nq, T), torch.float32),
+                             ((nq,), torch.int64))
     check(lib.ann_adc_rerank(ptr(queries), nq, d, ptr(lists), w, ptr(offsets), offsets.shape[0] - 1, ptr(members),
                              ptr(centers), ptr(codes), m, ks, ptr(codebooks), L, T, ptr(ids), ptr(keys), ptr(seen),
                              stream_ptr(stream)))
@@ -204,9 +224,14 @@ def graph_d_adc_search(coarse_index, queries, w, Tc, offsets, members, centers_f
     tensor of the coarse index's dtype (uint8 queries are widened to float32
     for the re-ranking).  Returns (ids, keys, examined, lists)."""
     import torch
-    lists, _, _ = ann_search_batch(coarse_index, queries, w, Tc, kmax=w, stream=stream)
-    qf = queries if queries.dtype == torch.float32 else queries.to(torch.float32)
-    ids, keys, seen = ann_adc_rerank(qf, lists, offsets, members, centers_f32, codes, codebooks, L, T, stream)
+    cur = torch.cuda.current_stream(queries.device)
+    # everything between the two calls runs on their stream and in its memory
+    with torch.cuda.stream(_torch_stream(stream, queries.device)):
+        lists, _, _ = ann_search_batch(coarse_index, queries, w, Tc, kmax=w, stream=stream)
+        qf = queries if queries.dtype == torch.float32 else queries.to(torch.float32)
+        ids, keys, seen = ann_adc_rerank(qf, lists, offsets, members, centers_f32, codes, codebooks, L, T, stream)
+    for t in (ids, keys, seen, lists):
+        t.record_stream(cur)
     return ids, keys, seen, lists
 
 
@@ -214,8 +239,9 @@ def ann_train_centers(train, P, n, iters, init_rows: np.ndarray, want_f64=False,
     import torch
     ntrain, d = train.shape
     init_rows = np.ascontiguousarray(init_rows, dtype=np.int64)
-    out = torch.empty((P, n, d // P), dtype=train.dtype, device=train.device)
-    out64 = torch.empty((P, n, d // P), dtype=torch.float64, device=train.device) if want_f64 else None
+    shape = (P, n, d // P)
+    out, *out64 = _alloc(stream, train.device, (shape, train.dtype), *([(shape, torch.float64)] if want_f64 else []))
+    out64 = out64[0] if want_f64 else None
     check(lib.ann_train_centers(ptr(train), dtype_code(train), ntrain, d, P, n, iters, ptr(init_rows), ptr(out),
                                 ptr(out64), stream_ptr(stream)))
     return (out, out64) if want_f64 else out
@@ -300,13 +326,10 @@ def ann_search_batch(index: Index, queries, k, T, kmax=None, mode=ANN_MODE_PLAIN
         kmax = int(k_arr.max().item()) if k_arr is not None else k_all
         kmax = max(kmax, 1)
     dev = queries.device
-    if out_ids is None:
-        out_ids = torch.empty((nq, kmax), dtype=torch.int32, device=dev)
-    if out_keys is None:
-        out_keys = torch.empty((nq, kmax), dtype=torch.int32 if queries.dtype == torch.uint8 else torch.float32,
-                               device=dev)
-    if out_status is None:
-        out_status = torch.empty((nq,), dtype=torch.int32, device=dev)
+    out_ids, out_keys, out_status = _outputs(
+        stream, dev, (out_ids, (nq, kmax), torch.int32),
+        (out_keys, (nq, kmax), torch.int32 if queries.dtype == torch.uint8 else torch.float32),
+        (out_status, (nq,), torch.int32))
     check(lib.ann_search_batch(index.handle, ptr(queries), nq, ptr(k_arr), ptr(T_arr), k_all, T_all, kmax, mode,
                                ptr(out_ids), ptr(out_keys), ptr(out_status), ptr(out_stats), stream_ptr(stream)))
     return out_ids, out_keys, out_status

@@ -182,3 +182,33 @@ def test_adc_argument_checks(ann):
     ids, keys, seen = ann.ann_adc_rerank(Q, lists, offsets, members, C, codes, cb, 10, 3)
     assert ids.cpu().tolist() == [[0, -1, -1]] * 2 and seen.cpu().tolist() == [1, 1]
     assert np.isinf(keys.cpu().numpy()[:, 1:]).all()
+
+
+def test_graph_d_adc_on_another_stream_than_the_current_one(ann):
+    # the coarse search's keys are not kept, and as many bytes as the widened queries take (k = 128 of 10,000 queries)
+    N, K, nq, m, w = 100_000, 2000, 10_000, 8, 128
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()  # noqa: E731
+    X, Q = dev(datagen.mixture(31, N, 128, 40, np.uint8)), dev(datagen.mixture(32, nq, 128, 40, np.uint8))
+    Cc = X[:K].contiguous()
+    assign = ann.ann_exact_knn(Cc, X, 1)[0][:, 0].contiguous()
+    members = torch.sort(assign.long(), stable=True).indices.to(torch.int32)
+    offsets = torch.zeros(K + 1, dtype=torch.int64, device="cuda")
+    offsets[1:] = torch.cumsum(torch.bincount(assign.long(), minlength=K), 0)
+    books = torch.randn((m, 64, 128 // m), device="cuda") * 20
+    codes = ann.ann_pq_encode(X, Cc.float(), assign, books)
+    G, _ = ann.ann_build_knn_graph(Cc, 16)
+    ix = ann.Index.create(Cc, G, ann.ann_train_centers(Cc, 2, 32, 2, np.arange(32)), t=100, b=5)
+    Cf = Cc.float()
+
+    def search(stream):
+        torch.cuda.synchronize()
+        out = ann.graph_d_adc_search(ix, Q, w, 256, offsets, members, Cf, codes, books, 4000, 100, stream=stream)
+        torch.cuda.synchronize()
+        return out
+
+    want = search(None)
+    side = torch.cuda.Stream()
+    for stream in (side, side, side.cuda_stream):
+        for a, b in zip(search(stream), want):
+            assert torch.equal(a, b)
+    ix.free()
