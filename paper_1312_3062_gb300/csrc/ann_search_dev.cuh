@@ -193,8 +193,8 @@ __host__ __device__ inline WarpLayout main_layout(int dtype, int d, int capT, in
 }
 
 // The prologue walks to the first bridge and on to kReach times the distance of
-// that bridge's nearest reference (or kFirstEnough bridges): references up to
-// about that distance are popped, and a query that needs a walk beyond has to be
+// the nearest reference of the bridges so far (or kFirstEnough bridges):
+// references up to about that distance are popped, and a query that needs a walk beyond has to be
 // resumed, one whole query's length after the batch.  Suspended of 10,000
 // queries with kReach = 0 / 1 / 1.3: T = 371 21 / 4 / 0, T = 2392 503 / 22 / 1;
 // times 0.88 / 0.81 / 0.79 and 5.75 / 5.72 / 4.98 ms (1.6: the same, 2: 0.86 ms).
@@ -1700,9 +1700,9 @@ __device__ void prologue_one(const SearchArgs &A, uint8_t *smem, int64_t w) {
     const uint64_t *bkey = (const uint64_t *)(smem + L.bkey);
     const uint32_t *bidx = (const uint32_t *)(smem + L.bidx), *misc = (const uint32_t *)(smem + L.misc);
     uint32_t bcnt = 0;
-    uint32_t reach = 0;  // walk at least to this key
+    uint32_t near = 0xffffffffu;  // the nearest reference seen
+    uint32_t reach = 0;           // walk at least to this key
     while ((bcnt == 0 || ((uint32_t)(ws.lo >> 32) < reach && bcnt < kFirstEnough)) && !ws.exhausted && !cap_err) {
-        const bool begin = bcnt == 0;
         const uint32_t c = refill<DT, GRP>(ix, smem, L, ws, cap_err);
         for (uint32_t i = lane; i < c; i += 32) {
             A.bkeys[at * A.bstore + bcnt + i] = bkey[i];
@@ -1710,20 +1710,21 @@ __device__ void prologue_one(const SearchArgs &A, uint8_t *smem, int64_t w) {
         }
         bcnt += c;
         __syncwarp();
-        if (begin && c > 0) {
-            // the nearest reference of the first bridge: the search pops
-            // references up to about its distance
-            uint32_t *cand = (uint32_t *)(smem + L.pref), *ckey = cand + 32;
-            const int32_t r = lane < ix.b ? __ldg(ix.brefs + (int64_t)bidx[0] * ix.b + lane) : -1;
-            const unsigned have = __ballot_sync(0xffffffffu, r >= 0 && r < ix.N);
-            if ((have >> lane) & 1u) cand[__popc(have & ((1u << lane) - 1))] = (uint32_t)r;
-            __syncwarp();
-            const int m = __popc(have);
-            cand_distances<DT>(ix.X, ix.d * (DT == ANN_U8 ? 1 : 4), smem + L.q, cand, m, ckey);
-            const uint32_t d = __reduce_min_sync(0xffffffffu, lane < m ? ckey[lane] : 0xffffffffu);
-            if (m) reach = DT == ANN_U8 ? (uint32_t)((float)d * kReach) : __float_as_uint(__uint_as_float(d) * kReach);
-            __syncwarp();
-        }
+        // the nearest reference of the batch's first bridges: the search pops
+        // references up to about its distance
+        uint32_t *cand = (uint32_t *)(smem + L.pref), *ckey = cand + 32;
+        const uint32_t bi = (uint32_t)(lane / ix.b);
+        const int32_t r =
+            lane < 32 / ix.b * ix.b && bi < c ? __ldg(ix.brefs + (int64_t)bidx[bi] * ix.b + lane % ix.b) : -1;
+        const unsigned have = __ballot_sync(0xffffffffu, r >= 0 && r < ix.N);
+        if ((have >> lane) & 1u) cand[__popc(have & ((1u << lane) - 1))] = (uint32_t)r;
+        __syncwarp();
+        const int m = __popc(have);
+        cand_distances<DT>(ix.X, ix.d * (DT == ANN_U8 ? 1 : 4), smem + L.q, cand, m, ckey);
+        near = min(near, __reduce_min_sync(0xffffffffu, lane < m ? ckey[lane] : 0xffffffffu));
+        if (near != 0xffffffffu)
+            reach = DT == ANN_U8 ? (uint32_t)((float)near * kReach) : __float_as_uint(__uint_as_float(near) * kReach);
+        __syncwarp();
     }
     if (lane == 0) {
         QRec r;
