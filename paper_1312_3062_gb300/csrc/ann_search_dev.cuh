@@ -193,8 +193,9 @@ __host__ __device__ inline WarpLayout main_layout(int dtype, int d, int capT, in
 }
 
 // The prologue walks to the first bridge and on to kReach times the distance of
-// the nearest reference of the bridges so far (or kFirstEnough bridges):
-// references up to about that distance are popped, and a query that needs a walk beyond has to be
+// the nearest reference of the bridges so far (or kFirstEnough bridges; where a
+// walk has neither groups nor a single prefix part, and a second one is dear, of
+// the first bridge): references up to about that distance are popped, and a query that needs a walk beyond has to be
 // resumed, one whole query's length after the batch.  Suspended of 10,000
 // queries with kReach = 0 / 1 / 1.3: T = 371 21 / 4 / 0, T = 2392 503 / 22 / 1;
 // times 0.88 / 0.81 / 0.79 and 5.75 / 5.72 / 4.98 ms (1.6: the same, 2: 0.86 ms).
@@ -202,6 +203,13 @@ constexpr float kReach = 1.3f;
 // bridges that end the prologue's walks whatever their reach, and the most one
 // walk of it returns
 constexpr uint32_t kFirstEnough = 128, kFirstCap = 256;
+// Budgets below kFewT pop few references: their prologue widens its windows
+// slowly, stays within the reach and stops after kFewReads entries (nodes,
+// groups, leaves), because one warp's long walk is later than a resumed query.
+// T = 64, 2,500 queries, before / after: 2 x 256 dictionaries 1.26 / 0.83 ms, 4 x 16
+// 0.38 / 0.32, GIST-shaped 3 x 128 3.74 / 1.64, 3 x 32 1.06 / 0.87.
+constexpr int kFewT = 256;
+constexpr uint32_t kFewReads = 4096;
 // a walk trims its buffer, of 32 entries or more, until a step's 64 leaves fit in
 static_assert(kFirstCap >= 64 + 32, "the prologue's walks could not trim their buffer");
 
@@ -1349,15 +1357,18 @@ __device__ __forceinline__ void window_resize(WalkState &ws, uint64_t hi) {
     ws.width = w > 1 ? w : 1;
 }
 
-// Refill the batch: bridges after ws.lo in order.  Returns count (0 = none left).
+// Refill the batch: bridges after ws.lo in order, up to about the key `limit`.
+// A batch of fewer than `few` widens the next window, one of fewer than half as
+// many, beyond the smallest `few`, twice as much.  Returns count (0 = none left,
+// or none up to the limit).
 template <int DT, bool GRP>
 __device__ uint32_t refill(const DevIndex &ix, uint8_t *smem, const WarpLayout &L, WalkState &ws,
-                           bool &cap_err) {
+                           bool &cap_err, uint32_t limit, uint32_t few) {
     uint64_t *bkey = (uint64_t *)(smem + L.bkey);
     uint32_t *bidx = (uint32_t *)(smem + L.bidx);
     const int lane = lane_id();
     while (!ws.exhausted) {
-        uint64_t hi = window_end(ws.lo, ws.first, ws.kmin, ws.width, ws.kmaxall);
+        uint64_t hi = window_end(ws.lo, ws.first, ws.kmin, ws.width, min(ws.kmaxall, limit));
         const uint64_t hi0 = hi;
         uint32_t c = walk<DT, 1, GRP>(ix, smem, L, ws.lo, ws.first, hi, bkey, bidx, L.bcap);
         if (hi != hi0) window_resize(ws, hi);
@@ -1389,12 +1400,13 @@ __device__ uint32_t refill(const DevIndex &ix, uint8_t *smem, const WarpLayout &
         ws.first = false;
         if (reached_end) ws.exhausted = true;
         if (c == 0) {
+            if ((uint32_t)(hi >> 32) >= limit) return 0;
             if (ws.width < 0x40000000u) ws.width <<= 1;
             continue;
         }
         // grow the window while batches stay small
-        if (c < L.bcap / 8 && ws.width < 0x40000000u) ws.width <<= 2;
-        else if (c < L.bcap / 4 && ws.width < 0x40000000u) ws.width <<= 1;
+        if (c < few / 2 && few > 16 && ws.width < 0x40000000u) ws.width <<= 2;
+        else if (c < few && ws.width < 0x40000000u) ws.width <<= 1;
         // sort the batch
         uint32_t Lp = 1;
         while (Lp < c) Lp <<= 1;
@@ -1702,8 +1714,15 @@ __device__ void prologue_one(const SearchArgs &A, uint8_t *smem, int64_t w) {
     uint32_t bcnt = 0;
     uint32_t near = 0xffffffffu;  // the nearest reference seen
     uint32_t reach = 0;           // walk at least to this key
-    while ((bcnt == 0 || ((uint32_t)(ws.lo >> 32) < reach && bcnt < kFirstEnough)) && !ws.exhausted && !cap_err) {
-        const uint32_t c = refill<DT, GRP>(ix, smem, L, ws, cap_err);
+    const bool few = T < kFewT, all_near = few || GRP || ix.PA == 1;
+    // entries read so far, groups by their mean number per prefix node
+    const uint32_t per_node = GRP ? 1u + (uint32_t)(ix.ngroups / ix.nA) : 1u;
+    while ((bcnt == 0 || ((uint32_t)(ws.lo >> 32) < reach && bcnt < kFirstEnough &&
+                          !(few && misc[9] * per_node + misc[10] >= kFewReads))) &&
+           !ws.exhausted && !cap_err) {
+        const bool look = bcnt == 0 || all_near;
+        const uint32_t c = refill<DT, GRP>(ix, smem, L, ws, cap_err, few && bcnt > 0 ? reach : 0xffffffffu,
+                                           few ? 16u : L.bcap / 4);
         for (uint32_t i = lane; i < c; i += 32) {
             A.bkeys[at * A.bstore + bcnt + i] = bkey[i];
             A.bidxs[at * A.bstore + bcnt + i] = bidx[i];
@@ -1719,7 +1738,7 @@ __device__ void prologue_one(const SearchArgs &A, uint8_t *smem, int64_t w) {
         const unsigned have = __ballot_sync(0xffffffffu, r >= 0 && r < ix.N);
         if ((have >> lane) & 1u) cand[__popc(have & ((1u << lane) - 1))] = (uint32_t)r;
         __syncwarp();
-        const int m = __popc(have);
+        const int m = look ? __popc(have) : 0;
         cand_distances<DT>(ix.X, ix.d * (DT == ANN_U8 ? 1 : 4), smem + L.q, cand, m, ckey);
         near = min(near, __reduce_min_sync(0xffffffffu, lane < m ? ckey[lane] : 0xffffffffu));
         if (near != 0xffffffffu)
