@@ -122,27 +122,20 @@ def _torch_stream(stream, device):
     return torch.cuda.ExternalStream(stream, device=device) if isinstance(stream, int) else stream
 
 
-def _alloc(stream, device, *specs):
-    """One tensor per (shape, dtype), for a call on `stream`: taken from that stream's memory, so that a block of which
-    another stream still has work, or one that is given back while the call runs, is never shared with it.  The caller's
-    current stream may use them too."""
-    import torch
-    if not specs:
-        return []
-    cur = torch.cuda.current_stream(device)
-    if (stream_ptr(stream) or 0) == cur.cuda_stream:
-        return [torch.empty(shape, dtype=dt, device=device) for shape, dt in specs]
-    with torch.cuda.stream(_torch_stream(stream, device)):
-        out = [torch.empty(shape, dtype=dt, device=device) for shape, dt in specs]
-    for t in out:
-        t.record_stream(cur)
-    return out
-
-
 def _outputs(stream, device, *given):
-    """Outputs of a call on `stream`: (tensor or None, shape, dtype) each; those not given are allocated."""
-    new = iter(_alloc(stream, device, *((shape, dt) for t, shape, dt in given if t is None)))
-    return [next(new) if t is None else t for t, _, _ in given]
+    """Outputs of a call on `stream`, as (tensor or None, shape, dtype): those not given are allocated, in memory of that
+    stream, so that a block of which another stream still has work, or one that is given back while the call runs, is
+    never shared with it.  The caller's current stream may use them too."""
+    import torch
+    if (stream_ptr(stream) or 0) == torch._C._cuda_getCurrentRawStream(device.index):
+        return [torch.empty(shape, dtype=dt, device=device) if t is None else t for t, shape, dt in given]
+    cur = torch.cuda.current_stream(device)
+    with torch.cuda.stream(_torch_stream(stream, device)):
+        out = [torch.empty(shape, dtype=dt, device=device) if t is None else t for t, shape, dt in given]
+    for t, (was, _, _) in zip(out, given):
+        if was is None:
+            t.record_stream(cur)
+    return out
 
 
 def dtype_code(t) -> int:
@@ -208,8 +201,8 @@ def ann_adc_rerank(queries, lists, offsets, members, centers, codes, codebooks, 
     nq, d = queries.shape
     w = lists.shape[1]
     m, ks, _ = codebooks.shape
-    ids, keys, seen = _alloc(stream, queries.device, ((nq, T), torch.int32), ((nq, T), torch.float32),
-                             ((nq,), torch.int64))
+    ids, keys, seen = _outputs(stream, queries.device, (None, (nq, T), torch.int32), (None, (nq, T), torch.float32),
+                               (None, (nq,), torch.int64))
     check(lib.ann_adc_rerank(ptr(queries), nq, d, ptr(lists), w, ptr(offsets), offsets.shape[0] - 1, ptr(members),
                              ptr(centers), ptr(codes), m, ks, ptr(codebooks), L, T, ptr(ids), ptr(keys), ptr(seen),
                              stream_ptr(stream)))
@@ -240,8 +233,8 @@ def ann_train_centers(train, P, n, iters, init_rows: np.ndarray, want_f64=False,
     ntrain, d = train.shape
     init_rows = np.ascontiguousarray(init_rows, dtype=np.int64)
     shape = (P, n, d // P)
-    out, *out64 = _alloc(stream, train.device, (shape, train.dtype), *([(shape, torch.float64)] if want_f64 else []))
-    out64 = out64[0] if want_f64 else None
+    (out,) = _outputs(stream, train.device, (None, shape, train.dtype))
+    out64 = _outputs(stream, train.device, (None, shape, torch.float64))[0] if want_f64 else None
     check(lib.ann_train_centers(ptr(train), dtype_code(train), ntrain, d, P, n, iters, ptr(init_rows), ptr(out),
                                 ptr(out64), stream_ptr(stream)))
     return (out, out64) if want_f64 else out
