@@ -1053,6 +1053,7 @@ extern "C" int ann_train_centers(const void *train, int dtype, int64_t ntrain, i
         ANN_CUDA(cudaMemsetAsync(isums.p, 0, 8 * (size_t)total, s));
         ANN_CUDA(cudaMemsetAsync(fsums.p, 0, 8 * (size_t)total, s));
         ANN_CUDA(cudaMemsetAsync(counts.p, 0, 8 * (size_t)P * n, s));
+        ANN_CUDA(cudaMemsetAsync(namb.p, 0, 4 * (size_t)P, s));
         km_prep_kernel<<<P, 256, 0, s>>>(C.p, n, dp, cneg.p, cmax.p);
         for (int64_t r0 = 0; r0 < ntrain; r0 += slice) {
             const int64_t rows_s = std::min(slice, ntrain - r0);
@@ -1061,7 +1062,7 @@ extern "C" int ann_train_centers(const void *train, int dtype, int64_t ntrain, i
             const dim3 grid_w(nblk(32 * rows_s), (unsigned)P);
             const unsigned gx =
                 (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)2 * nsm / P, (rows_s + 63) / 64));
-            ANN_CUDA(cudaMemsetAsync(namb.p, 0, 4 * (size_t)P, s));
+            if (r0 > 0) ANN_CUDA(cudaMemsetAsync(namb.p, 0, 4 * (size_t)P, s));
             if (dtype == ANN_U8) {
                 if (n > 64)
                     km_assign_kernel<ANN_U8, 16><<<grid_a, 256, 0, s>>>(xs, rows_s, d, dp, n, cneg.p, cmax.p, assign.p,
