@@ -374,8 +374,11 @@ int knn_f32_tensor(const float *refs, int64_t N, const float *queries, int64_t n
     // of an older part, 12.3 ms padded).
     const int ld = (3 * d + 7) / 8 * 8;
     const int64_t Np = (N + 63) / 64 * 64;
-    // tile of query rows: the tile's dot products take about 2 GB
-    int64_t tm = std::max<int64_t>(32, (((int64_t)1 << 29) / Np) / 256 * 256);
+    // Tile of query rows: the tile's dot products take about 2 GB, or up to 8 GB
+    // to make it 512 rows, below which reading all reference rows for it costs
+    // more than the products.
+    const int64_t rows8 = std::max<int64_t>(32, ((int64_t)1 << 31) / Np / 32 * 32);
+    int64_t tm = std::max(((int64_t)1 << 29) / Np / 256 * 256, std::min<int64_t>(512, rows8));
     if (tm > nq) tm = nq;
     const bool shared = queries == refs && nq <= N;  // queries are the first nq reference rows
     __nv_bfloat16 *x3 = nullptr, *q3 = nullptr;

@@ -119,6 +119,17 @@ def test_f32_knn_odd_sizes_and_alignments(ann, N, nq, d, k, shift):
     np.testing.assert_allclose(keys.cpu().numpy(), want_keys, rtol=1e-5)
 
 
+def test_f32_knn_with_millions_of_references(ann):
+    # more references than a tile of 256 query rows takes in 2 GB; two tiles and a remainder
+    N, nq, d, k = 2_200_003, 1100, 4, 10
+    X, Q = np.random.default_rng(1).random((N, d), np.float32), np.random.default_rng(2).random((nq, d), np.float32)
+    ids, keys = ann.ann_exact_knn(dev(X), dev(Q), k)
+    sel = np.r_[0, 511, 512, 1023, 1024, nq - 1]
+    want_ids, want_keys = oracle.exact_knn(X, np.ascontiguousarray(Q[sel]), k)
+    np.testing.assert_array_equal(ids.cpu().numpy()[sel], want_ids)
+    np.testing.assert_allclose(keys.cpu().numpy()[sel], want_keys, rtol=1e-5)
+
+
 @pytest.mark.parametrize("kind", ["descending", "late_cluster", "ties"])
 def test_f32_knn_when_the_first_columns_mislead(ann, kind):
     # the candidate limit starts from the first 4096 columns: here those are
