@@ -270,7 +270,7 @@ enum {
  * stream-ordered workspace (cudaMallocAsync): about 5 KB per query, in passes
  * of 32768 queries; up to 256 MB for the states of queries that pop many
  * bridges; and per warp that the device holds at once (about 1,800, or one
- * per query if fewer) 24 min(8192, max(1024, 2 T)) bytes, from T = 1024 on
+ * per query if fewer) 24 min(8192, max(192, 2 T)) bytes, from T = 1024 on
  * another 14.4 T.  Batches that the device holds at once need the last part
  * only.  Where a workspace cannot be had, smaller passes run, down to 128
  * queries (7 MB below T = 1024, at most 45 MB); below that ANN_ERR_OOM.
