@@ -1729,12 +1729,16 @@ __device__ void prologue_one(const SearchArgs &A, uint8_t *smem, int64_t w) {
         }
         bcnt += c;
         __syncwarp();
-        // the nearest reference of the batch's first bridges: the search pops
-        // references up to about its distance
+        // the nearest reference of the batch's first bridges (or of the first of
+        // all): the search pops references up to about its distance
         uint32_t *cand = (uint32_t *)(smem + L.pref), *ckey = cand + 32;
-        const uint32_t bi = (uint32_t)(lane / ix.b);
-        const int32_t r =
-            lane < 32 / ix.b * ix.b && bi < c ? __ldg(ix.brefs + (int64_t)bidx[bi] * ix.b + lane % ix.b) : -1;
+        int32_t r = -1;
+        if (all_near) {
+            const uint32_t bi = (uint32_t)(lane / ix.b);
+            if (lane < 32 / ix.b * ix.b && bi < c) r = __ldg(ix.brefs + (int64_t)bidx[bi] * ix.b + lane % ix.b);
+        } else if (lane < ix.b && c > 0) {
+            r = __ldg(ix.brefs + (int64_t)bidx[0] * ix.b + lane);
+        }
         const unsigned have = __ballot_sync(0xffffffffu, r >= 0 && r < ix.N);
         if ((have >> lane) & 1u) cand[__popc(have & ((1u << lane) - 1))] = (uint32_t)r;
         __syncwarp();
