@@ -147,3 +147,36 @@ def test_batches_of_more_than_one_pass(ann, mode, T):
         for a in got:
             a.zero_()
     ix.free()
+
+
+# the prologue's rules: budgets below 256 walk up to the reach only, dictionaries with c2 groups (4 x 8) or one prefix
+# part look at every batch's references; few cells, so that queries pop many bridges and walks end at the limit
+@pytest.mark.parametrize("dtype,d,P,n,T", [(np.uint8, 64, 4, 8, 64), (np.uint8, 64, 4, 8, 300), (np.uint8, 128, 2, 64, 255),
+                                           (np.uint8, 128, 2, 64, 256), (np.float32, 48, 3, 16, 100),
+                                           (np.float32, 64, 2, 32, 33), (np.uint8, 96, 3, 30, 1)])
+def test_first_batches_of_bridges(ann, dtype, d, P, n, T):
+    N, nq, k = 5000, 4000, 10
+    rng = np.random.default_rng(T)
+    X, Q = datagen.mixture(T, N, d, 300, dtype), datagen.mixture(T, nq, d, 300, dtype)
+    C = ann.ann_train_centers(dev(X), P, n, 2, rng.permutation(N)[:n])
+    G, _ = ann.ann_build_knn_graph(dev(X), 8)
+    ix = ann.Index.create(dev(X), G, C, t=100, b=5)
+    Qd = dev(Q)
+
+    def search(q):
+        st = torch.zeros((len(q), ann.ANN_NSTATS), dtype=torch.int64, device="cuda")
+        out = ann.ann_search_batch(ix, q, k, T, out_stats=st)
+        return [*out, st[:, [ann.STAT_NAMES.index(x) for x in ("discovered", "ref_pops", "bridge_pops", "max_q")]]]
+
+    many = search(Qd)
+    few = [torch.cat(x) for x in zip(*(search(Qd[i:i + 150].contiguous()) for i in range(0, nq, 150)))]
+    for a, b in zip(many, few):
+        assert torch.equal(a, b)
+    sel = rng.permutation(nq)[:16]
+    ids, refs = ix.bridges()
+    bg = dict(bridges=ids, offsets=np.concatenate([[0], np.cumsum((refs >= 0).sum(1))]).astype(np.int64),
+              refs=refs[refs >= 0])
+    want = oracle.search(X, G.cpu().numpy(), C.cpu().numpy(), bg, Q[sel], k, T, kmax=k, nthreads=8)[0]
+    np.testing.assert_array_equal(many[0].cpu().numpy()[sel], want)
+    assert (ix.info()["groups"] > 0) == (P == 4)
+    ix.free()
